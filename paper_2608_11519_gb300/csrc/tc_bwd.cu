@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(BCfg<D, PASS>::kThreads, 1)
     const uint32_t fin0 = accfree0 + 8u * NS;
     const uint32_t aready0 = fin0 + 8u * NS;
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_index();
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(BCfg<D, PASS>::kThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp_uniform(*tmem_slot);
 
     if (warp == C::kProdWarp) {
         // ------------------------------------------------------------ TMA producer

@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t fin = accempty0 + 16u;
     const uint32_t sfree0 = fin + 8u;                      // [kEpiGroups], count 1
     const uint32_t swritten0 = sfree0 + 8u * kEpiGroups;   // [kEpiGroups], count 128
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_index();
     const int lane = threadIdx.x & 31;
     const int slices = (int)(prm.C / D) * (MODE == 1 ? prm.n_a : 1);
 
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp_uniform(*tmem_slot);
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer

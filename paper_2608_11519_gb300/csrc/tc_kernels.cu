@@ -603,7 +603,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t sready0 = afree0 + 8u * C::kABufS;  // [NS][2]
     const uint32_t pready0 = sready0 + 16u * NS;  // [NS][2]
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_index();
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -635,7 +635,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp_uniform(*tmem_slot);
     // every global access below may depend on the kernel before this one
     pdl_wait();
 

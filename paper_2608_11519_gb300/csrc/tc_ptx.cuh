@@ -18,6 +18,15 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
     return t;
 }
 
+// Lane 0's value: tells the compiler that a value (the same in every lane already) is uniform
+// over the warp, so that what is derived from it stays in uniform registers. tcgen05 and TMA
+// instructions take their addresses and descriptors from those; from an ordinary register each
+// operand of each instruction is first moved over, on the issuing lane's critical path.
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t x) {
+    return __shfl_sync(0xffffffffu, x, 0);
+}
+__device__ __forceinline__ int warp_index() { return (int)warp_uniform(threadIdx.x >> 5); }
+
 // ---------------------------------------------------------------- programmatic launch
 // Let the next kernel on the stream (launched with programmatic stream serialization) start
 // its blocks now; they run up to their pdl_wait.
@@ -370,6 +379,18 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
     d |= static_cast<uint64_t>(1) << 46;
     d |= static_cast<uint64_t>(swz & 7u) << 61;
     return d;
+}
+
+// The same in two words: the high one holds only the stride offset, the version and the swizzle,
+// constants of a tile layout, so that a role keeps one register per descriptor.
+__device__ __forceinline__ uint32_t smem_desc_lo(uint32_t saddr, uint32_t lbo) {
+    return ((saddr >> 4) & 0x3FFFu) | (((lbo >> 4) & 0x3FFFu) << 16);
+}
+__host__ __device__ constexpr uint32_t smem_desc_hi(uint32_t sbo, uint32_t swz) {
+    return ((sbo >> 4) & 0x3FFFu) | (1u << 14) | ((swz & 7u) << 29);
+}
+__device__ __forceinline__ uint64_t desc_of(uint32_t lo, uint32_t hi) {
+    return static_cast<uint64_t>(hi) << 32 | lo;
 }
 
 // Instruction descriptor of kind::f16 with bf16 A and B and an f32 accumulator.

@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t accfull0 = empty0 + 8u * kS;
     const uint32_t accempty0 = accfull0 + 16u;
     const uint32_t fin = accempty0 + 16u;
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_index();
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = warp_uniform(*tmem_slot);
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
