@@ -268,6 +268,89 @@ __global__ void bwd_reduce_kernel(const float* __restrict__ pa, const float* __r
     if (lane == 0) cout[row] = dot;
 }
 
+// Reduce of the partials dS^T K that the token passes of tc_tok.cu leave, a CTA's slot each:
+// T = D / 4 threads per route row (four channels each), slots in CTA order.
+//   DSEEDS false: dq = s sum (with flags, only of the (b, h) with flags[bh] == 0; of the others
+//     dq += s sum of the route pass's partials pb, nchunk of them), its bf16 copy, and
+//     c1 = <dQ, Q> from that copy (as bwd_reduce_kernel's MODE 2)
+//   DSEEDS true: dseeds[h, m] = s sum over the batch and the slots (rows = H * M)
+// Four loads are in flight per thread.
+template <int D, bool DSEEDS>
+__global__ void __launch_bounds__(256)
+    tok_reduce_kernel(const float* __restrict__ part, int64_t rows, int64_t B, int64_t H, int64_t M,
+                      int64_t nt, int64_t tiles, int64_t ctas, int64_t slots, float scale,
+                      const int* __restrict__ flags, const float* __restrict__ pb, int64_t nchunk,
+                      const float* __restrict__ Q, float* __restrict__ dq,
+                      float* __restrict__ c1, __nv_bfloat16* __restrict__ op) {
+    constexpr int T = D / 4;
+    const int64_t row = ((int64_t)blockIdx.x * 256 + threadIdx.x) / T;
+    const int g = threadIdx.x % T;
+    if (row >= rows) return;  // (rows in whole groups of T threads)
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto add = [&](const float* base, int64_t n, int64_t stride) {
+        const float4* p = reinterpret_cast<const float4*>(base) + g;
+        const int64_t st = stride / 4;
+        int64_t k = 0;
+        for (; k + 4 <= n; k += 4) {
+            const float4 v0 = p[k * st], v1 = p[(k + 1) * st], v2 = p[(k + 2) * st],
+                         v3 = p[(k + 3) * st];
+            a.x += v0.x; a.y += v0.y; a.z += v0.z; a.w += v0.w;
+            a.x += v1.x; a.y += v1.y; a.z += v1.z; a.w += v1.w;
+            a.x += v2.x; a.y += v2.y; a.z += v2.z; a.w += v2.w;
+            a.x += v3.x; a.y += v3.y; a.z += v3.z; a.w += v3.w;
+        }
+        for (; k < n; ++k) {
+            const float4 v = p[k * st];
+            a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+        }
+    };
+    auto add_slots = [&](int64_t bh, int64_t m) {
+        const int64_t c0 = ((bh * nt + 1) * ctas - 1) / tiles;
+        const int64_t c1_ = (((bh + 1) * nt) * ctas - 1) / tiles;
+        add(part + (bh * slots * M + m) * D, c1_ - c0 + 1, M * D);
+    };
+    if constexpr (DSEEDS) {
+        const int64_t h = row / M, m = row % M;
+        for (int64_t b = 0; b < B; ++b) add_slots(b * H + h, m);
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(scale * a.x, scale * a.y);
+        const __nv_bfloat162 hi = __floats2bfloat162_rn(scale * a.z, scale * a.w);
+        uint2 v;
+        v.x = *reinterpret_cast<const uint32_t*>(&lo);
+        v.y = *reinterpret_cast<const uint32_t*>(&hi);
+        reinterpret_cast<uint2*>(op + row * D)[g] = v;
+    } else {
+        const int64_t bh = row / M, m = row % M;
+        float4* out = reinterpret_cast<float4*>(dq + row * D) + g;
+        float4 base = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (flags == nullptr || flags[bh] == 0) {
+            add_slots(bh, m);
+        } else {
+            base = *out;
+            add(pb + (bh * nchunk * M + m) * D, nchunk, M * D);
+        }
+        const float4 v = make_float4(base.x + scale * a.x, base.y + scale * a.y,
+                                     base.z + scale * a.z, base.w + scale * a.w);
+        *out = v;
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y);
+        const __nv_bfloat162 hi = __floats2bfloat162_rn(v.z, v.w);
+        uint2 pk;
+        pk.x = *reinterpret_cast<const uint32_t*>(&lo);
+        pk.y = *reinterpret_cast<const uint32_t*>(&hi);
+        reinterpret_cast<uint2*>(op + row * D)[g] = pk;
+        const float2 f0 = __bfloat1622float2(lo), f1 = __bfloat1622float2(hi);
+        const float4 q = reinterpret_cast<const float4*>(Q + row * D)[g];
+        float dot = f0.x * q.x;
+        dot = fmaf(f0.y, q.y, dot);
+        dot = fmaf(f1.x, q.z, dot);
+        dot = fmaf(f1.y, q.w, dot);
+        const unsigned lane = threadIdx.x & 31u;
+        const unsigned mask = ((1u << T) - 1u) << (lane & ~(unsigned)(T - 1));
+#pragma unroll
+        for (int off = T / 2; off > 0; off >>= 1) dot += __shfl_xor_sync(mask, dot, off);
+        if (g == 0) c1[row] = dot;
+    }
+}
+
 // Token pass; thread = token n, every route streamed.
 //   MODE 23 (calls 3 and 2 together): keys k = K_n, w = V_n, y = dY_n; routes a = Q, g = dZ,
 //     z = Z with L2, c2 per route and L3, c3 of the token:
@@ -473,15 +556,38 @@ __global__ void merge_flags_kernel(const float* __restrict__ part, int64_t BH,
     flags[bh] = (mx3 - R <= kMergeRange && mx2 - R <= kMergeRange) ? 0 : 1;
 }
 
-// The merged pass's route operand w dZ: W[bh][m][:] = bf16(2^(R[bh] - L2[bh][m]) dZ[bh][m][:]).
-__global__ void merge_operand_kernel(const float* __restrict__ dz, const float* __restrict__ L2,
-                                     const float* __restrict__ Rb, int64_t M, int64_t D,
-                                     int64_t total, __nv_bfloat16* __restrict__ W) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = i / D;  // bh * M + m
-        W[i] = __float2bfloat16_rn(exp2f(Rb[row / M] - L2[row]) * dz[i]);
-    }
+// The merged pass's route operand w dZ: W[bh][m][:] = bf16(2^(R[bh] - L2[bh][m]) dZ[bh][m][:]), and
+// c2 taken from it: c2w = <W, Z> / w. The pass forms w dP2 = W V^T, and dS2 = P2 (dP2 - c2)
+// cancels for a nearly one-hot P2 only when c2 sees the same rounded dZ. D / 4 threads per row.
+template <int D>
+__global__ void __launch_bounds__(256)
+    merge_operand_kernel(const float* __restrict__ dz, const float* __restrict__ Z,
+                         const float* __restrict__ L2, const float* __restrict__ Rb, int64_t M,
+                         int64_t rows, __nv_bfloat16* __restrict__ W, float* __restrict__ c2w) {
+    constexpr int T = D / 4;
+    const int64_t row = ((int64_t)blockIdx.x * 256 + threadIdx.x) / T;  // bh * M + m
+    const int g = threadIdx.x % T;
+    if (row >= rows) return;  // (rows in whole groups of T threads)
+    const float e = Rb[row / M] - L2[row];
+    const float w = exp2f(e);
+    const float4 v = reinterpret_cast<const float4*>(dz + row * D)[g];
+    const float4 z = reinterpret_cast<const float4*>(Z + row * D)[g];
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(w * v.x, w * v.y);
+    const __nv_bfloat162 hi = __floats2bfloat162_rn(w * v.z, w * v.w);
+    uint2 pk;
+    pk.x = *reinterpret_cast<const uint32_t*>(&lo);
+    pk.y = *reinterpret_cast<const uint32_t*>(&hi);
+    reinterpret_cast<uint2*>(W + row * D)[g] = pk;
+    const float2 f0 = __bfloat1622float2(lo), f1 = __bfloat1622float2(hi);
+    float dot = f0.x * z.x;
+    dot = fmaf(f0.y, z.y, dot);
+    dot = fmaf(f1.x, z.z, dot);
+    dot = fmaf(f1.y, z.w, dot);
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned mask = ((1u << T) - 1u) << (lane & ~(unsigned)(T - 1));
+#pragma unroll
+    for (int off = T / 2; off > 0; off >>= 1) dot += __shfl_xor_sync(mask, dot, off);
+    if (g == 0) c2w[row] = dot * exp2f(-e);
 }
 
 // The tensor-core path (bf16 inputs): c3, the bf16 operand copies of Q and Z, then
@@ -512,6 +618,7 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
     T* dzb = (T*)(ws + bp.off_dzb);
     T* dqb = (T*)(ws + bp.off_dqb);
     T* wop = (T*)(ws + bp.off_w);
+    float* c2w = (float*)(ws + bp.off_c2w);
     float* Rb = (float*)(ws + bp.off_rb);
     int* flags = (int*)(ws + bp.off_flags);
     float* rpart = (float*)(ws + bp.off_rpart);
@@ -548,26 +655,52 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
                                                            bp.nchunk, scale, Z32, dz, dq, c2,
                                                            nullptr, dzb);
     // T23: token rows; S = K Q^T, dP2 = V dZ^T, dP3 = dY Z^T -> dK, dV
-    o = TcBwdOperands{{K, V, dY}, {qb, dzb, zb}, L3, c3, L2, c2, nullptr, nullptr, dK, dV};
-    o.lo = qlo;
+    TcBwdOperands t23{{K, V, dY}, {qb, dzb, zb}, L3, c3, L2, c2, nullptr, nullptr, dK, dV};
+    t23.lo = qlo;
+    // R2: route rows; S = Q K^T, dP = dZ V^T; row statistics L2, c2 -> dQ2 partials
+    TcBwdOperands r2{{qb, dzb, dzb}, {K, V, V}, L2, c2, nullptr, nullptr, nullptr, pb, nullptr,
+                     nullptr};
+    r2.lo = qlo;
     if (kMerged) {
-        // T23C: S = K Q^T, T = dY Z^T + (u V) (w dZ)^T; the flagged (b, h) run T23 after it
-        merge_operand_kernel<<<cvt_blocks, 256, 0, st>>>(dz, L2, Rb, p.M, p.D, lat, wop);
-        TcBwdOperands om{{K, dY, V}, {qb, wop, zb}, L3, c3, L2, c2, nullptr, nullptr, dK, dV};
+        // the merged pass's route operand w dZ; the flagged (b, h) run the unmerged T23
+        merge_operand_kernel<D><<<(unsigned)((lat / 4 + 255) / 256), 256, 0, st>>>(
+            dz, Z32, L2, Rb, p.M, lat_rows, wop, c2w);
+        t23.flags = flags;
+        t23.want = 1;
+    }
+    if constexpr (kMerged) {
+        if (bp.tok_slots > 0) {
+            // the token passes that also form dQ and dseeds; the flagged (b, h) take T23 and R2
+            float* pt = (float*)(ws + bp.off_pt);
+            const int64_t tiles = bp.tok_nt * p.BH;
+            r2.flags = flags;
+            r2.want = 1;
+            TokOperands t{{K, V, dY}, {qb, wop, zb}, qlo, L3, c3, L2, c2w, Rb, flags, pt, dK, dV};
+            if ((e = tc_tok_pass(p, bp, false, t, scale, status, st)) != cudaSuccess) return e;
+            if ((e = tc_bwd_pass(p, bp, 3, t23, scale, status, st)) != cudaSuccess) return e;
+            if ((e = tc_bwd_pass(p, bp, 1, r2, scale, status, st)) != cudaSuccess) return e;
+            const auto blocks = [](int64_t rows) { return (unsigned)((rows * (D / 4) + 255) / 256); };
+            tok_reduce_kernel<D, false><<<blocks(lat_rows), 256, 0, st>>>(
+                pt, lat_rows, p.B, p.H, p.M, bp.tok_nt, tiles, bp.tok_ctas, bp.tok_slots, scale,
+                flags, pb, bp.nchunk, Q32, dq, c1, dqb);
+            t = TokOperands{{Kt, Vt, Vt}, {seeds, dqb, dqb}, nullptr, nullptr, nullptr, L1, c1,
+                            nullptr, nullptr, pt, dKt, dVt};
+            if ((e = tc_tok_pass(p, bp, true, t, scale, status, st)) != cudaSuccess) return e;
+            tok_reduce_kernel<D, true><<<blocks(p.H * p.M), 256, 0, st>>>(
+                pt, p.H * p.M, p.B, p.H, p.M, bp.tok_nt, tiles, bp.tok_ctas, bp.tok_slots, scale,
+                nullptr, nullptr, 0, nullptr, nullptr, nullptr, (T*)dseeds);
+            return cudaGetLastError();
+        }
+        // T23C: S = K Q^T, T = dY Z^T + (u V) (w dZ)^T
+        TcBwdOperands om{{K, dY, V}, {qb, wop, zb}, L3, c3, L2, c2w, nullptr, nullptr, dK, dV};
         om.Rb = Rb;
         om.flags = flags;
         om.want = 0;
         om.lo = qlo;
         if ((e = tc_bwd_pass(p, bp, 5, om, scale, status, st)) != cudaSuccess) return e;
-        o.flags = flags;
-        o.want = 1;
     }
-    if ((e = tc_bwd_pass(p, bp, 3, o, scale, status, st)) != cudaSuccess) return e;
-    // R2: route rows; S = Q K^T, dP = dZ V^T; row statistics L2, c2 -> dQ2 partials
-    o = TcBwdOperands{{qb, dzb, dzb}, {K, V, V}, L2, c2, nullptr, nullptr, nullptr, pb, nullptr,
-                      nullptr};
-    o.lo = qlo;
-    if ((e = tc_bwd_pass(p, bp, 1, o, scale, status, st)) != cudaSuccess) return e;
+    if ((e = tc_bwd_pass(p, bp, 3, t23, scale, status, st)) != cudaSuccess) return e;
+    if ((e = tc_bwd_pass(p, bp, 1, r2, scale, status, st)) != cudaSuccess) return e;
     bwd_reduce_kernel<D, T, 2><<<red_blocks, 256, 0, st>>>(nullptr, pb, lat_rows, p.B, p.H, p.M,
                                                            bp.nchunk, scale, Q32, nullptr, dq, c1,
                                                            nullptr, dqb);

@@ -94,8 +94,13 @@ struct BwdPlan {
     size_t off_dzb, off_dqb;    // ... and dZ, dQ
     size_t off_qlo;             // ... and Q's lo part, Q - bf16(Q) (D <= 32)
     size_t off_w;               // ... and the merged T23 pass's w dZ [BH][M][D] bf16
+    size_t off_c2w;             // ... and its c2, taken from that operand [BH][M] f32
     size_t off_rb, off_flags;   // its shift R [BH] f32 and fallback flags [BH] int32
     size_t off_rpart;           // range partials [BH][kRangeParts + 2] f32
+    // the token passes that also form dQ (tc_tok.cu): token tiles per (b, h), CTAs, partial slots
+    // per (b, h) (0: the shape runs the separate passes), and the partials [BH][slots][M][D] f32
+    int64_t tok_nt, tok_ctas, tok_slots;
+    size_t off_pt;
     size_t total;
 };
 constexpr int kRangeParts = 128;  // token slices of the merged pass's range reduction
@@ -156,6 +161,31 @@ struct TcBwdOperands {
 // pass: 0 = R3, 1 = R2, 2 = R1 (route rows), 3 = T23, 4 = T1 (token rows), 5 = T23C (T23
 // with its two dP products merged; D = 16 and 32)
 cudaError_t tc_bwd_pass(const Plan& p, const BwdPlan& bp, int pass, const TcBwdOperands& o,
+                        float scale, int* status, cudaStream_t st);
+
+// ---- token passes that also form the route-side gradient (tc_tok.cu), bf16, D = 16 and 32
+// The most routes they serve (0: none at this D): dQ's accumulators, D TMEM columns per 128 routes,
+// share the 512 columns with the score tiles (256) and the dK and dV accumulators (4 D).
+constexpr int64_t tok_max_routes(int64_t D) { return D == 16 ? 1024 : (D == 32 ? 512 : 0); }
+// a: K, V, dY (calls 3 and 2) or Kt, Vt (call 1); i: Q, w dZ, Z or seeds, dQ; lo: Q's lo operand.
+// Row statistics L3, c3 and column statistics L2, c2 with the shift Rb per (b, h), or (call 1)
+// column statistics L1, c1. out0, out1: dK, dV (dKt, dVt); part: the CTAs' partial sums of
+// dS^T K. flags, when set: only the (b, h) with flags[bh] == 0 run.
+struct TokOperands {
+    const void* a[3];
+    const void* i[3];
+    const void* lo;
+    const float* Lrow;
+    const float* crow;
+    const float* Lcol;
+    const float* ccol;
+    const float* Rb;
+    const int* flags;
+    float* part;
+    void* out0;
+    void* out1;
+};
+cudaError_t tc_tok_pass(const Plan& p, const BwdPlan& bp, bool call1, const TokOperands& o,
                         float scale, int* status, cudaStream_t st);
 
 // ---- the mixer's pointwise projections (tc_gemm.cu), bf16

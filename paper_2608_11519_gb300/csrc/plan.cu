@@ -210,12 +210,25 @@ BwdPlan make_bwd_plan(const Plan& p) {
         off = align_up(off + op, kWsAlign);
         b.off_w = off;
         off = align_up(off + op, kWsAlign);
+        b.off_c2w = off;
+        off = align_up(off + lm, kWsAlign);
         b.off_rb = off;
         off = align_up(off + (size_t)p.BH * 4, kWsAlign);
         b.off_flags = off;
         off = align_up(off + (size_t)p.BH * 4, kWsAlign);
         b.off_rpart = off;
         off = align_up(off + (size_t)p.BH * (kRangeParts + 2) * 4, kWsAlign);
+        if (p.M <= tok_max_routes(p.D) && cdiv(p.N, 128) * p.BH < INT32_MAX) {
+            // contiguous runs of 128-token tiles, one per SM; a (b, h)'s tiles reach over at
+            // most ceil(nt / run) + 1 of them
+            b.tok_nt = cdiv(p.N, 128);
+            const int64_t tiles = b.tok_nt * p.BH;
+            b.tok_ctas = tiles < kNumSMs ? tiles : kNumSMs;
+            b.tok_slots = cdiv(b.tok_nt, tiles / b.tok_ctas) + 1;
+            b.off_pt = off;
+            off = align_up(off + (size_t)p.BH * (size_t)b.tok_slots * (size_t)p.M * (size_t)p.D * 4,
+                           kWsAlign);
+        }
     }
     b.total = off;
     return b;
