@@ -268,89 +268,6 @@ __global__ void bwd_reduce_kernel(const float* __restrict__ pa, const float* __r
     if (lane == 0) cout[row] = dot;
 }
 
-// Reduce of the partials dS^T K that the token passes of tc_tok.cu leave, a CTA's slot each:
-// T = D / 4 threads per route row (four channels each), slots in CTA order.
-//   DSEEDS false: dq = s sum (with flags, only of the (b, h) with flags[bh] == 0; of the others
-//     dq += s sum of the route pass's partials pb, nchunk of them), its bf16 copy, and
-//     c1 = <dQ, Q> from that copy (as bwd_reduce_kernel's MODE 2)
-//   DSEEDS true: dseeds[h, m] = s sum over the batch and the slots (rows = H * M)
-// Four loads are in flight per thread.
-template <int D, bool DSEEDS>
-__global__ void __launch_bounds__(256)
-    tok_reduce_kernel(const float* __restrict__ part, int64_t rows, int64_t B, int64_t H, int64_t M,
-                      int64_t nt, int64_t tiles, int64_t ctas, int64_t slots, float scale,
-                      const int* __restrict__ flags, const float* __restrict__ pb, int64_t nchunk,
-                      const float* __restrict__ Q, float* __restrict__ dq,
-                      float* __restrict__ c1, __nv_bfloat16* __restrict__ op) {
-    constexpr int T = D / 4;
-    const int64_t row = ((int64_t)blockIdx.x * 256 + threadIdx.x) / T;
-    const int g = threadIdx.x % T;
-    if (row >= rows) return;  // (rows in whole groups of T threads)
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto add = [&](const float* base, int64_t n, int64_t stride) {
-        const float4* p = reinterpret_cast<const float4*>(base) + g;
-        const int64_t st = stride / 4;
-        int64_t k = 0;
-        for (; k + 4 <= n; k += 4) {
-            const float4 v0 = p[k * st], v1 = p[(k + 1) * st], v2 = p[(k + 2) * st],
-                         v3 = p[(k + 3) * st];
-            a.x += v0.x; a.y += v0.y; a.z += v0.z; a.w += v0.w;
-            a.x += v1.x; a.y += v1.y; a.z += v1.z; a.w += v1.w;
-            a.x += v2.x; a.y += v2.y; a.z += v2.z; a.w += v2.w;
-            a.x += v3.x; a.y += v3.y; a.z += v3.z; a.w += v3.w;
-        }
-        for (; k < n; ++k) {
-            const float4 v = p[k * st];
-            a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
-        }
-    };
-    auto add_slots = [&](int64_t bh, int64_t m) {
-        const int64_t c0 = ((bh * nt + 1) * ctas - 1) / tiles;
-        const int64_t c1_ = (((bh + 1) * nt) * ctas - 1) / tiles;
-        add(part + (bh * slots * M + m) * D, c1_ - c0 + 1, M * D);
-    };
-    if constexpr (DSEEDS) {
-        const int64_t h = row / M, m = row % M;
-        for (int64_t b = 0; b < B; ++b) add_slots(b * H + h, m);
-        const __nv_bfloat162 lo = __floats2bfloat162_rn(scale * a.x, scale * a.y);
-        const __nv_bfloat162 hi = __floats2bfloat162_rn(scale * a.z, scale * a.w);
-        uint2 v;
-        v.x = *reinterpret_cast<const uint32_t*>(&lo);
-        v.y = *reinterpret_cast<const uint32_t*>(&hi);
-        reinterpret_cast<uint2*>(op + row * D)[g] = v;
-    } else {
-        const int64_t bh = row / M, m = row % M;
-        float4* out = reinterpret_cast<float4*>(dq + row * D) + g;
-        float4 base = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (flags == nullptr || flags[bh] == 0) {
-            add_slots(bh, m);
-        } else {
-            base = *out;
-            add(pb + (bh * nchunk * M + m) * D, nchunk, M * D);
-        }
-        const float4 v = make_float4(base.x + scale * a.x, base.y + scale * a.y,
-                                     base.z + scale * a.z, base.w + scale * a.w);
-        *out = v;
-        const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y);
-        const __nv_bfloat162 hi = __floats2bfloat162_rn(v.z, v.w);
-        uint2 pk;
-        pk.x = *reinterpret_cast<const uint32_t*>(&lo);
-        pk.y = *reinterpret_cast<const uint32_t*>(&hi);
-        reinterpret_cast<uint2*>(op + row * D)[g] = pk;
-        const float2 f0 = __bfloat1622float2(lo), f1 = __bfloat1622float2(hi);
-        const float4 q = reinterpret_cast<const float4*>(Q + row * D)[g];
-        float dot = f0.x * q.x;
-        dot = fmaf(f0.y, q.y, dot);
-        dot = fmaf(f1.x, q.z, dot);
-        dot = fmaf(f1.y, q.w, dot);
-        const unsigned lane = threadIdx.x & 31u;
-        const unsigned mask = ((1u << T) - 1u) << (lane & ~(unsigned)(T - 1));
-#pragma unroll
-        for (int off = T / 2; off > 0; off >>= 1) dot += __shfl_xor_sync(mask, dot, off);
-        if (g == 0) c1[row] = dot;
-    }
-}
-
 // Token pass; thread = token n, every route streamed.
 //   MODE 23 (calls 3 and 2 together): keys k = K_n, w = V_n, y = dY_n; routes a = Q, g = dZ,
 //     z = Z with L2, c2 per route and L3, c3 of the token:
@@ -558,7 +475,41 @@ __global__ void merge_flags_kernel(const float* __restrict__ part, int64_t BH,
 
 // The merged pass's route operand w dZ: W[bh][m][:] = bf16(2^(R[bh] - L2[bh][m]) dZ[bh][m][:]), and
 // c2 taken from it: c2w = <W, Z> / w. The pass forms w dP2 = W V^T, and dS2 = P2 (dP2 - c2)
-// cancels for a nearly one-hot P2 only when c2 sees the same rounded dZ. D / 4 threads per row.
+// cancels for a nearly one-hot P2 only when c2 sees the same rounded dZ. v, z: this thread's four
+// channels (group g of D / 4) of the row of dZ and Z.
+__device__ __forceinline__ uint2 pack4(float4 v) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y);
+    const __nv_bfloat162 hi = __floats2bfloat162_rn(v.z, v.w);
+    return make_uint2(*reinterpret_cast<const uint32_t*>(&lo),
+                      *reinterpret_cast<const uint32_t*>(&hi));
+}
+__device__ __forceinline__ float dot4(float4 a, float4 b) {
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, a.x * b.x)));
+}
+__device__ __forceinline__ float4 unpack4(uint2 p) {
+    const float2 f0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&p.x));
+    const float2 f1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&p.y));
+    return make_float4(f0.x, f0.y, f1.x, f1.y);
+}
+// the sum of x over a row's T threads (adjacent lanes)
+template <int T>
+__device__ __forceinline__ float row_sum(float x) {
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned mask = ((1u << T) - 1u) << (lane & ~(unsigned)(T - 1));
+#pragma unroll
+    for (int off = T / 2; off > 0; off >>= 1) x += __shfl_xor_sync(mask, x, off);
+    return x;
+}
+template <int D>
+__device__ __forceinline__ void merge_operand(float4 v, float4 z, float e, int64_t row, int g,
+                                              __nv_bfloat16* W, float* c2w) {
+    const float w = exp2f(e);
+    const uint2 pk = pack4(make_float4(w * v.x, w * v.y, w * v.z, w * v.w));
+    reinterpret_cast<uint2*>(W + row * D)[g] = pk;
+    const float dot = row_sum<D / 4>(dot4(unpack4(pk), z));
+    if (g == 0) c2w[row] = dot * exp2f(-e);
+}
+
 template <int D>
 __global__ void __launch_bounds__(256)
     merge_operand_kernel(const float* __restrict__ dz, const float* __restrict__ Z,
@@ -568,26 +519,116 @@ __global__ void __launch_bounds__(256)
     const int64_t row = ((int64_t)blockIdx.x * 256 + threadIdx.x) / T;  // bh * M + m
     const int g = threadIdx.x % T;
     if (row >= rows) return;  // (rows in whole groups of T threads)
-    const float e = Rb[row / M] - L2[row];
-    const float w = exp2f(e);
-    const float4 v = reinterpret_cast<const float4*>(dz + row * D)[g];
-    const float4 z = reinterpret_cast<const float4*>(Z + row * D)[g];
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(w * v.x, w * v.y);
-    const __nv_bfloat162 hi = __floats2bfloat162_rn(w * v.z, w * v.w);
-    uint2 pk;
-    pk.x = *reinterpret_cast<const uint32_t*>(&lo);
-    pk.y = *reinterpret_cast<const uint32_t*>(&hi);
-    reinterpret_cast<uint2*>(W + row * D)[g] = pk;
-    const float2 f0 = __bfloat1622float2(lo), f1 = __bfloat1622float2(hi);
-    float dot = f0.x * z.x;
-    dot = fmaf(f0.y, z.y, dot);
-    dot = fmaf(f1.x, z.z, dot);
-    dot = fmaf(f1.y, z.w, dot);
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned mask = ((1u << T) - 1u) << (lane & ~(unsigned)(T - 1));
+    merge_operand<D>(reinterpret_cast<const float4*>(dz + row * D)[g],
+                     reinterpret_cast<const float4*>(Z + row * D)[g], Rb[row / M] - L2[row], row, g,
+                     W, c2w);
+}
+
+// dZ from the partial sums of tc_dz_pass, slot by slot in order (a chunk's token-parity parts as
+// the encode's plan cuts them: 4, 2 or 1 by the route tiles of the row's group of 512): its bf16
+// copy, c2 = <dZ, Z>, and the merged pass's operand. D / 4 threads per row, four loads in flight.
+template <int D>
+__global__ void __launch_bounds__(256)
+    dz_reduce_kernel(const float* __restrict__ part, int M, int nchunk, int64_t rows,
+                     const float* __restrict__ Z, const float* __restrict__ L2,
+                     const float* __restrict__ Rb, __nv_bfloat16* __restrict__ dzb,
+                     float* __restrict__ c2, __nv_bfloat16* __restrict__ W,
+                     float* __restrict__ c2w) {
+    constexpr int T = D / 4;
+    const int64_t row = ((int64_t)blockIdx.x * 256 + threadIdx.x) / T;  // bh * M + m
+    const int g = threadIdx.x % T;
+    if (row >= rows) return;  // (rows in whole groups of T threads)
+    const int64_t bh = row / M;
+    const int m = (int)(row - bh * M);
+    const int left = M - (m & ~511);
+    const int ul = left > 256 ? 0 : (left > 128 ? 1 : 2);  // log2 of the parts per chunk
+    const int n = nchunk << ul, mask = (1 << ul) - 1;
+    const float4* p = reinterpret_cast<const float4*>(part + (bh * nchunk * 4 * M + m) * D) + g;
+    const int64_t st = (int64_t)M * T;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < n; s0 += 4) {
+        float4 v[4];
 #pragma unroll
-    for (int off = T / 2; off > 0; off >>= 1) dot += __shfl_xor_sync(mask, dot, off);
-    if (g == 0) c2w[row] = dot * exp2f(-e);
+        for (int e = 0; e < 4; ++e) {
+            const int s = s0 + e;
+            v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (s < n) v[e] = p[((int64_t)(s >> ul) * 4 + (s & mask)) * st];
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            a.x += v[e].x;
+            a.y += v[e].y;
+            a.z += v[e].z;
+            a.w += v[e].w;
+        }
+    }
+    const float4 z = reinterpret_cast<const float4*>(Z + row * D)[g];
+    reinterpret_cast<uint2*>(dzb + row * D)[g] = pack4(a);
+    const float dot = row_sum<T>(dot4(a, z));
+    if (g == 0) c2[row] = dot;
+    merge_operand<D>(a, z, Rb[bh] - L2[row], row, g, W, c2w);
+}
+
+// Reduce of the partials dS^T K that the token passes of tc_tok.cu leave, a CTA's slot each:
+// T = D / 4 threads per route row (four channels each), slots in CTA order.
+//   DSEEDS false: dQ = s sum (of the flagged (b, h) s times the sum of the route passes' partials,
+//     pb of R3 and pa of R2, nchunk each), as bf16, and c1 = <dQ, Q> from that copy (as
+//     bwd_reduce_kernel's MODE 2)
+//   DSEEDS true: dseeds[h, m] = s sum over the batch and the slots (rows = H * M)
+// Four loads are in flight per thread.
+template <int D, bool DSEEDS>
+__global__ void __launch_bounds__(256)
+    tok_reduce_kernel(const float* __restrict__ part, int64_t rows, int64_t B, int64_t H, int64_t M,
+                      int64_t nt, int64_t tiles, int64_t ctas, int64_t slots, float scale,
+                      const int* __restrict__ flags, const float* __restrict__ pb,
+                      const float* __restrict__ pa, int64_t nchunk, const float* __restrict__ Q,
+                      float* __restrict__ c1, __nv_bfloat16* __restrict__ op) {
+    constexpr int T = D / 4;
+    const int64_t row = ((int64_t)blockIdx.x * 256 + threadIdx.x) / T;
+    const int g = threadIdx.x % T;
+    if (row >= rows) return;  // (rows in whole groups of T threads)
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto add = [&](const float* base, int64_t n, int64_t stride) {
+        const float4* p = reinterpret_cast<const float4*>(base) + g;
+        const int64_t st = stride / 4;
+        int64_t k = 0;
+        for (; k + 4 <= n; k += 4) {
+            const float4 v0 = p[k * st], v1 = p[(k + 1) * st], v2 = p[(k + 2) * st],
+                         v3 = p[(k + 3) * st];
+            a.x += v0.x; a.y += v0.y; a.z += v0.z; a.w += v0.w;
+            a.x += v1.x; a.y += v1.y; a.z += v1.z; a.w += v1.w;
+            a.x += v2.x; a.y += v2.y; a.z += v2.z; a.w += v2.w;
+            a.x += v3.x; a.y += v3.y; a.z += v3.z; a.w += v3.w;
+        }
+        for (; k < n; ++k) {
+            const float4 v = p[k * st];
+            a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+        }
+    };
+    auto add_slots = [&](int64_t bh, int64_t m) {
+        const int64_t c0 = ((bh * nt + 1) * ctas - 1) / tiles;
+        const int64_t c1_ = (((bh + 1) * nt) * ctas - 1) / tiles;
+        add(part + (bh * slots * M + m) * D, c1_ - c0 + 1, M * D);
+    };
+    if constexpr (DSEEDS) {
+        const int64_t h = row / M, m = row % M;
+        for (int64_t b = 0; b < B; ++b) add_slots(b * H + h, m);
+        reinterpret_cast<uint2*>(op + row * D)[g] =
+            pack4(make_float4(scale * a.x, scale * a.y, scale * a.z, scale * a.w));
+    } else {
+        const int64_t bh = row / M, m = row % M;
+        if (flags == nullptr || flags[bh] == 0) {
+            add_slots(bh, m);
+        } else {
+            add(pb + (bh * nchunk * M + m) * D, nchunk, M * D);
+            add(pa + (bh * nchunk * M + m) * D, nchunk, M * D);
+        }
+        const uint2 pk = pack4(make_float4(scale * a.x, scale * a.y, scale * a.z, scale * a.w));
+        reinterpret_cast<uint2*>(op + row * D)[g] = pk;
+        const float dot =
+            row_sum<T>(dot4(unpack4(pk), reinterpret_cast<const float4*>(Q + row * D)[g]));
+        if (g == 0) c1[row] = dot;
+    }
 }
 
 // The tensor-core path (bf16 inputs): c3, the bf16 operand copies of Q and Z, then
@@ -645,15 +686,9 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
         merge_flags_kernel<<<(unsigned)((p.BH + 127) / 128), 128, 0, st>>>(rpart, p.BH, Rb,
                                                                             flags);
     }
-    TcBwdOperands o{};
     // R3: route rows; S = Q K^T, dP = Z dY^T; column statistics L3, c3 -> dQ3, dZ partials
-    o = TcBwdOperands{{qb, zb, zb}, {K, dY, dY}, nullptr, nullptr, L3, c3, pa, pb, nullptr,
-                      nullptr};
-    o.lo = qlo;
-    if ((e = tc_bwd_pass(p, bp, 0, o, scale, status, st)) != cudaSuccess) return e;
-    bwd_reduce_kernel<D, T, 3><<<red_blocks, 256, 0, st>>>(pa, pb, lat_rows, p.B, p.H, p.M,
-                                                           bp.nchunk, scale, Z32, dz, dq, c2,
-                                                           nullptr, dzb);
+    TcBwdOperands r3{{qb, zb, zb}, {K, dY, dY}, nullptr, nullptr, L3, c3, pa, pb, nullptr, nullptr};
+    r3.lo = qlo;
     // T23: token rows; S = K Q^T, dP2 = V dZ^T, dP3 = dY Z^T -> dK, dV
     TcBwdOperands t23{{K, V, dY}, {qb, dzb, zb}, L3, c3, L2, c2, nullptr, nullptr, dK, dV};
     t23.lo = qlo;
@@ -661,36 +696,49 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
     TcBwdOperands r2{{qb, dzb, dzb}, {K, V, V}, L2, c2, nullptr, nullptr, nullptr, pb, nullptr,
                      nullptr};
     r2.lo = qlo;
-    if (kMerged) {
-        // the merged pass's route operand w dZ; the flagged (b, h) run the unmerged T23
-        merge_operand_kernel<D><<<(unsigned)((lat / 4 + 255) / 256), 256, 0, st>>>(
-            dz, Z32, L2, Rb, p.M, lat_rows, wop, c2w);
-        t23.flags = flags;
-        t23.want = 1;
-    }
     if constexpr (kMerged) {
+        t23.flags = flags;  // the flagged (b, h) run the unmerged T23
+        t23.want = 1;
         if (bp.tok_slots > 0) {
-            // the token passes that also form dQ and dseeds; the flagged (b, h) take T23 and R2
+            // dZ as an encode of K and dY, then the token passes that also form dQ and dseeds;
+            // the flagged (b, h) take R3 (for its dQ3), T23 and R2 (its dQ2 partials go to pa,
+            // which R3's dZ does not need here)
+            float* pz = (float*)(ws + bp.off_pz);
             float* pt = (float*)(ws + bp.off_pt);
             const int64_t tiles = bp.tok_nt * p.BH;
-            r2.flags = flags;
-            r2.want = 1;
+            const auto blocks = [](int64_t rows) { return (unsigned)((rows * (D / 4) + 255) / 256); };
+            r3.flags = r2.flags = flags;
+            r3.want = r2.want = 1;
+            r2.pb = pa;
+            if ((e = tc_dz_pass(p, qb, qlo, K, dY, L3, scale, pz, status, st)) != cudaSuccess)
+                return e;
+            dz_reduce_kernel<D><<<blocks(lat_rows), 256, 0, st>>>(
+                pz, (int)p.M, (int)p.nchunk, lat_rows, Z32, L2, Rb, dzb, c2, wop, c2w);
             TokOperands t{{K, V, dY}, {qb, wop, zb}, qlo, L3, c3, L2, c2w, Rb, flags, pt, dK, dV};
             if ((e = tc_tok_pass(p, bp, false, t, scale, status, st)) != cudaSuccess) return e;
+            if ((e = tc_bwd_pass(p, bp, 0, r3, scale, status, st)) != cudaSuccess) return e;
             if ((e = tc_bwd_pass(p, bp, 3, t23, scale, status, st)) != cudaSuccess) return e;
             if ((e = tc_bwd_pass(p, bp, 1, r2, scale, status, st)) != cudaSuccess) return e;
-            const auto blocks = [](int64_t rows) { return (unsigned)((rows * (D / 4) + 255) / 256); };
             tok_reduce_kernel<D, false><<<blocks(lat_rows), 256, 0, st>>>(
                 pt, lat_rows, p.B, p.H, p.M, bp.tok_nt, tiles, bp.tok_ctas, bp.tok_slots, scale,
-                flags, pb, bp.nchunk, Q32, dq, c1, dqb);
+                flags, pb, pa, bp.nchunk, Q32, c1, dqb);
             t = TokOperands{{Kt, Vt, Vt}, {seeds, dqb, dqb}, nullptr, nullptr, nullptr, L1, c1,
                             nullptr, nullptr, pt, dKt, dVt};
             if ((e = tc_tok_pass(p, bp, true, t, scale, status, st)) != cudaSuccess) return e;
             tok_reduce_kernel<D, true><<<blocks(p.H * p.M), 256, 0, st>>>(
                 pt, p.H * p.M, p.B, p.H, p.M, bp.tok_nt, tiles, bp.tok_ctas, bp.tok_slots, scale,
-                nullptr, nullptr, 0, nullptr, nullptr, nullptr, (T*)dseeds);
+                nullptr, nullptr, nullptr, 0, nullptr, nullptr, (T*)dseeds);
             return cudaGetLastError();
         }
+    }
+    TcBwdOperands o{};
+    if ((e = tc_bwd_pass(p, bp, 0, r3, scale, status, st)) != cudaSuccess) return e;
+    bwd_reduce_kernel<D, T, 3><<<red_blocks, 256, 0, st>>>(pa, pb, lat_rows, p.B, p.H, p.M,
+                                                           bp.nchunk, scale, Z32, dz, dq, c2,
+                                                           nullptr, dzb);
+    if constexpr (kMerged) {
+        merge_operand_kernel<D><<<(unsigned)((lat / 4 + 255) / 256), 256, 0, st>>>(
+            dz, Z32, L2, Rb, p.M, lat_rows, wop, c2w);
         // T23C: S = K Q^T, T = dY Z^T + (u V) (w dZ)^T
         TcBwdOperands om{{K, dY, V}, {qb, wop, zb}, L3, c3, L2, c2w, nullptr, nullptr, dK, dV};
         om.Rb = Rb;

@@ -101,6 +101,7 @@ struct BwdPlan {
     // per (b, h) (0: the shape runs the separate passes), and the partials [BH][slots][M][D] f32
     int64_t tok_nt, tok_ctas, tok_slots;
     size_t off_pt;
+    size_t off_pz;  // dZ's partials [BH][nchunk * sub_per_chunk][M][D] f32 (the encode's plan)
     size_t total;
 };
 constexpr int kRangeParts = 128;  // token slices of the merged pass's range reduction
@@ -243,6 +244,11 @@ void test_fault_for(int kernel, uint64_t* wait_ns, int64_t* ring_item);
 // Rows per tensor-core work unit (route group of the encode, token group of the decode).
 int64_t tc_group_rows(int64_t D);
 int64_t tc_encode_item_rows(int64_t D);  // tokens per item of the tensor-core encode
+// dZ = P3^T dY of the backward (D = 16 and 32), P3 = 2^(scale log2(e) <q, k> - L3) with Q as its hi
+// and lo operands: an encode whose partials [BH][nchunk * sub_per_chunk][M][D] are plain sums.
+cudaError_t tc_dz_pass(const Plan& p, const void* Qhi, const void* Qlo, const void* K,
+                       const void* dY, const float* L3, float scale, float* part, int* status,
+                       cudaStream_t st);
 // Decode call 3: Y = SDPA(K, Q, Z) from the Q and Z operand copies; also each token's
 // base-2 log-normaliser into `lse` [BH][N] when it is not null. With `lo` (D <= 32) the
 // scores take Q as its hi and lo bf16 operands.

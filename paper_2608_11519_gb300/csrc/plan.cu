@@ -228,6 +228,10 @@ BwdPlan make_bwd_plan(const Plan& p) {
             b.off_pt = off;
             off = align_up(off + (size_t)p.BH * (size_t)b.tok_slots * (size_t)p.M * (size_t)p.D * 4,
                            kWsAlign);
+            b.off_pz = off;
+            off = align_up(off + (size_t)p.BH * (size_t)(p.nchunk * p.sub_per_chunk) * (size_t)p.M *
+                                     (size_t)p.D * 4,
+                           kWsAlign);
         }
     }
     b.total = off;

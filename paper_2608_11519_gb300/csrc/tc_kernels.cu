@@ -33,6 +33,11 @@
 // be repaired there: the kernel raises the launch's overflow word when it ends, and the safe
 // kernel after it, which otherwise returns at once, recomputes the launch with the exact
 // maximum wherever the sum passes that limit.
+// A third form of the encode (COL) serves the backward of call 3: dZ = P3^T dY, i.e. the encode of
+// K and dY whose probabilities P3 = 2^(c S - L3) are those the forward's softmax over the routes
+// had, with the tokens' log-normalisers L3 as column statistics. It keeps no reference and no sum
+// (P3 <= 1, so nothing can overflow and no safe kernel follows); its partials are plain sums. Warp
+// 5 copies each item's L3 into the ring beside its tiles.
 // Every wait is bounded (2 s of %globaltimer, or the test hook's limit): on expiry the
 // kernel records FLAREPP_ERR_TIMEOUT in the status word, every role leaves its loops, the
 // producer waits for its copies in flight, and TMEM is freed.
@@ -73,9 +78,11 @@ constexpr float kFastLimit = 281474976710656.0f;  // 2^48
 // scores see Q to about 2^-17 instead of bf16's 2^-9. The encode keeps both A tiles in its
 // shared-memory A buffer (the lo tile after the hi tile); the decode's items carry Q's lo tile
 // as a third tile.
-template <int D, bool DEC, bool LO = false>
+// COL (the backward's dZ, an encode): every item also carries its tokens' L3.
+template <int D, bool DEC, bool LO = false, bool COL = false>
 struct Cfg {
     static_assert(!LO || D <= 32, "the hi/lo form of Q serves D = 16 and 32");
+    static_assert(!(COL && DEC), "column statistics belong to the encode");
     static constexpr bool kLoA = LO && !DEC;  // encode of call 2: A = Q as hi and lo tiles
     static constexpr bool kLoB = LO && DEC;   // decode: every item also carries Q's lo tile
     static constexpr int kANum = kLoA ? 2 : 1;  // A tiles per stream
@@ -108,7 +115,8 @@ struct Cfg {
     // own items, and the copy of its next item cannot start before the stream frees the stage
     // kStages items back; so the encode takes as many stages as shared memory holds, up to 16.
     // The decode's streams take every item, and 8 stages cover the copy latency.
-    static constexpr int kStagesFit = (232448 - 2048 - kABufS * kABytes) / kStage;
+    static constexpr int kStat = COL ? kItem * 4 : 0;  // bytes of an item's column statistics
+    static constexpr int kStagesFit = (232448 - 2048 - kABufS * kABytes) / (kStage + kStat);
     static constexpr int kStages = DEC ? 8 : (kStagesFit < 16 ? kStagesFit : 16);
     // barriers: full[S], empty[S], a_full[kABufS] (a unit's A tiles landed), a_free[kABufS]
     //           (one arrive per softmax warpgroup once it has seen the unit's last S: the
@@ -122,7 +130,7 @@ struct Cfg {
     //           a_free of unit k.
     static constexpr int kNumBars = 2 * kStages + 2 * kABufS + 4 * NS;
     static constexpr int kData = kABufS * kABytes + kStages * kStage;
-    static constexpr int kNeed = 1024 + kData + kNumBars * 8 + 16;
+    static constexpr int kNeed = 1024 + kData + kStages * kStat + kNumBars * 8 + 16;
     // at least 120 KB so that one CTA owns an SM and its 512 TMEM columns
     static constexpr int kSmem = kNeed > 122880 ? kNeed : 122880;
     static constexpr uint32_t kIdescS = idesc_bf16_f32(128, kItem, false, false);
@@ -149,6 +157,7 @@ struct TcParams {
     float* lse;  // decode: each token's base-2 log-normaliser, or null
     int64_t n_units;
     int* status;
+    const float* Lcol;  // COL: the tokens' base-2 log-normalisers [BH][N]
     int* overflow;  // raised by the fast kernel; the safe kernel runs only when it is set
     uint64_t wait_ns;     // bound of every wait (kDefaultWaitNs unless the test hook is set)
     int64_t withhold_it;  // test hook: ring item of CTA 0 the producer never loads (-1: none)
@@ -170,6 +179,7 @@ struct Unit {
 
 // The plan keeps unit counts, and so every quotient below, within 32 bits; 32-bit divisions by
 // runtime values cost a few instructions where 64-bit ones cost about seventy.
+// (the same for the forms with a lo operand or column statistics: they cut the work alike)
 template <int D, bool DEC, bool LO>
 __device__ __forceinline__ Unit get_unit(const TcParams& p, int64_t u64) {
     using C = Cfg<D, DEC, LO>;
@@ -319,6 +329,34 @@ __device__ __forceinline__ float exp_chunk(const uint32_t* sr, uint32_t* pr, int
     return t0 + t1;
 }
 
+// COL: P = 2^(c S - L) for one chunk of W columns, with the columns' L (shared memory) from L on;
+// nc2: (-c, -c). No sum is kept.
+template <int W>
+__device__ __forceinline__ void exp_chunk_col(const uint32_t* sr, uint32_t* pr, int base, int nv,
+                                              float c, uint64_t nc2, const float* L) {
+    const bool full = base + W <= nv;
+#pragma unroll
+    for (int k = 0; k < W / 2; k += 2) {
+        const ulonglong2 l = *reinterpret_cast<const ulonglong2*>(L + 2 * k);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            // L - c s, whose negation is the exponent
+            uint64_t x = pack_f32x2(__uint_as_float(sr[2 * (k + e)]),
+                                    __uint_as_float(sr[2 * (k + e) + 1]));
+            asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(x) : "l"(x), "l"(nc2), "l"(e ? l.y : l.x));
+            float a, b;
+            unpack_f32x2(x, a, b);
+            pr[k + e] = pack_bf16(ex2(-a), ex2(-b));
+        }
+    }
+    if (!full) {
+#pragma unroll
+        for (int k = 0; k < W / 2; ++k)
+            pr[k] &= (base + 2 * k < nv ? 0xffffu : 0u) |
+                     (base + 2 * k + 1 < nv ? 0xffff0000u : 0u);
+    }
+}
+
 // P for a whole item tile of ITEM columns at TMEM column scol (S is read 32 columns at a
 // time, and a last 16 when ITEM is an odd multiple of 16); packed bf16 pairs go to
 // pr[0 .. ITEM/2). Returns the
@@ -382,14 +420,15 @@ __device__ __forceinline__ void store_p(uint32_t scol, uint32_t* pr) {
 //     item to the exact-max path, which reads S again (the decode, whose units are short,
 //     takes the first item's reference from its first score; the encode, whose units are
 //     long, takes the first item's exact maximum).
-template <int D, bool DEC, bool SAFE, bool LO>
+//   COL: P from the item's column statistics (the stage's full barrier covers their copies).
+template <int D, bool DEC, bool SAFE, bool LO, bool COL>
 __device__ __forceinline__ bool softmax_step(SoftmaxStream& S, const Unit& U, uint32_t tmem,
                                              uint32_t lane_off, float c, uint64_t c2,
                                              uint32_t sready_s, uint32_t pready_s, uint32_t empty0,
                                              uint32_t afree0, bool wg_leader, uint32_t it0,
                                              volatile int* abort_flag, int* status,
-                                             uint64_t limit, volatile int* overflow) {
-    using C = Cfg<D, DEC, LO>;
+                                             uint64_t limit, uint32_t full0, const float* stats) {
+    using C = Cfg<D, DEC, LO, COL>;
     const int j = S.j;
     const int b = j % C::B;
     const uint32_t par_j = (S.ph0 + (uint32_t)j) & 1u;
@@ -417,6 +456,35 @@ __device__ __forceinline__ bool softmax_step(SoftmaxStream& S, const Unit& U, ui
     const uint32_t scol = tmem + lane_off + C::kColS + (S.s * C::B + b) * C::kItem;
     uint32_t pr[C::kItem / 2];
     float sum = 0.f;
+    if constexpr (COL) {
+        const uint32_t it = it0 + item;
+        if (!warp_wait(full0 + 8u * (it % C::kStages), (it / C::kStages) & 1, abort_flag, status,
+                       limit))
+            return false;
+        const float* L = stats + (it % C::kStages) * C::kItem;
+        const uint64_t nc2 = pack_f32x2(-c, -c);
+#pragma unroll
+        for (int h = 0; h < C::kItem / 32; ++h) {
+            uint32_t sr[32];
+            tmem_ld32(scol + 32 * h, sr);
+            tmem_wait_ld32(sr);
+            exp_chunk_col<32>(sr, pr + 16 * h, 32 * h, nv, c, nc2, L + 32 * h);
+            tmem_st16(scol + 16 * h, pr + 16 * h);
+        }
+        if constexpr (C::kItem % 32 == 16) {
+            constexpr int base = C::kItem - 16;
+            uint32_t sr[16];
+            tmem_ld16(scol + base, sr);
+            tmem_wait_ld16(sr);
+            exp_chunk_col<16>(sr, pr + base / 2, base, nv, c, nc2, L + base);
+            tmem_st8(scol + base / 2, pr + base / 2);
+        }
+        tmem_wait_st();
+        tc_fence_before();
+        mbar_arrive(pready_s + 8u * b);
+        ++S.j;
+        return true;
+    }
     if constexpr (!SAFE) {
         sum = exp_tile<C::kItem, true, true>(scol, pr, nv, c, c2, S.m, j == 0);
         tmem_wait_st();
@@ -497,13 +565,13 @@ struct UnitEnd {
     uint32_t it0;
 };
 
-template <int D, bool DEC, bool LO>
+template <int D, bool DEC, bool LO, bool COL>
 __device__ __forceinline__ bool finish_stream(SoftmaxStream& S, const UnitEnd& E, const Unit& U,
                                               const TcParams& prm, uint32_t tmem,
                                               uint32_t lane_off, int r, uint32_t sready_s,
                                               uint32_t empty0, uint32_t afree0, bool wg_leader,
                                               bool deferred, volatile int* abort_flag) {
-    using C = Cfg<D, DEC, LO>;
+    using C = Cfg<D, DEC, LO, COL>;
     const int a = S.s % U.n_a;
     const int par = S.s / U.n_a;
     float o[D];
@@ -558,8 +626,10 @@ __device__ __forceinline__ bool finish_stream(SoftmaxStream& S, const UnitEnd& E
         const int64_t route = U.g * C::kGroup + a * kTileRows + r;
         if (route < prm.M) {
             const int64_t idx = (U.bh * (prm.nchunk * 4) + U.chunk * 4 + par) * prm.M + route;
-            prm.pmax[idx] = E.cnt > 0 ? E.m : -INFINITY;
-            prm.psum[idx] = E.l;
+            if constexpr (!COL) {
+                prm.pmax[idx] = E.cnt > 0 ? E.m : -INFINITY;
+                prm.psum[idx] = E.l;
+            }
             float4* dst = reinterpret_cast<float4*>(prm.pacc + idx * D);
 #pragma unroll
             for (int kk = 0; kk < D / 4; ++kk)
@@ -571,12 +641,12 @@ __device__ __forceinline__ bool finish_stream(SoftmaxStream& S, const UnitEnd& E
 
 // ------------------------------------------------------------------ the kernel
 
-template <int D, bool DEC, bool SAFE, bool LO>
+template <int D, bool DEC, bool SAFE, bool LO, bool COL>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmL,
                     const TcParams prm) {
-    using C = Cfg<D, DEC, LO>;
+    using C = Cfg<D, DEC, LO, COL>;
     pdl_trigger();
     if constexpr (SAFE) {
         // the safe kernel recomputes the launch only when the fast one overflowed
@@ -592,7 +662,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint8_t* abuf = smem;                         // kABufS x NS x kANum A tiles
     // kStages x (B tile, C tile[, lo tile]), swizzled like the A tiles
     uint8_t* ring = smem + C::kABufS * C::kABytes;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(ring + C::kStages * C::kStage);
+    float* stats = reinterpret_cast<float*>(ring + C::kStages * C::kStage);  // COL: [kStages][kItem]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(ring + C::kStages * (C::kStage + C::kStat));
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::kNumBars);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -608,7 +679,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (threadIdx.x == 0) {
         for (int st = 0; st < C::kStages; ++st) {
-            mbar_init(full0 + 8u * st, 1);
+            mbar_init(full0 + 8u * st, COL ? 33 : 1);
             mbar_init(empty0 + 8u * st, NS);
         }
         for (int b = 0; b < C::kABufS; ++b) {
@@ -842,6 +913,34 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
         }
+        if constexpr (COL) {
+            if (warp == kProducerWarp + 1) {
+                // the column statistics of every item, copied asynchronously (each lane's
+                // copies arrive on the item's full barrier themselves)
+                uint32_t it = 0;
+                bool ok = true;
+                for (int64_t u = blockIdx.x; u < prm.n_units && ok; u += gridDim.x) {
+                    const Unit U = get_unit<D, DEC, LO>(prm, u);
+                    const float* src = prm.Lcol + U.bh * prm.N;
+                    for (int i = 0; i < U.n_items; ++i, ++it) {
+                        const int st = it % C::kStages;
+                        if (!warp_wait(empty0 + 8u * st, ((it / C::kStages) & 1) ^ 1, abort_flag,
+                                       prm.status, prm.wait_ns)) {
+                            ok = false;
+                            break;
+                        }
+                        const int64_t row = U.item0 + (int64_t)i * C::kItem;
+                        const uint32_t dst = smem_u32(stats + st * C::kItem);
+                        for (int k = lane; k < C::kItem; k += 32) {
+                            const bool in = row + k < prm.N;
+                            cp_async4(dst + 4 * k, src + (in ? row + k : 0), in);
+                        }
+                        cp_async_arrive(full0 + 8u * st);
+                    }
+                }
+                cp_async_wait_all();
+            }
+        }
     } else {
         // ------------------------------------------------------------ softmax warpgroups
         regs_raise<kRegsSoftmax>();
@@ -872,15 +971,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             st.ob = C::kOBuf == 2 ? (int)(ua & 1) : 0;
             st.ab = (int)(ua % C::kABufS);
             while (alive && st.j < st.cnt) {
-                alive = softmax_step<D, DEC, SAFE, LO>(st, U, tmem, lane_off, c, c2, sready_s,
-                                                   pready0 + 16u * st.s, empty0, afree0,
-                                                   wg_leader, it0, abort_flag, prm.status,
-                                                   prm.wait_ns, prm.overflow);
+                alive = softmax_step<D, DEC, SAFE, LO, COL>(
+                    st, U, tmem, lane_off, c, c2, sready_s, pready0 + 16u * st.s, empty0, afree0,
+                    wg_leader, it0, abort_flag, prm.status, prm.wait_ns, full0, stats);
                 if (owed && alive) {
-                    alive = finish_stream<D, DEC, LO>(st, prev,
-                                                      get_unit<D, DEC, LO>(prm, u - gridDim.x),
-                                                      prm, tmem, lane_off, r, sready_s, empty0,
-                                                      afree0, wg_leader, true, abort_flag);
+                    alive = finish_stream<D, DEC, LO, COL>(
+                        st, prev, get_unit<D, DEC, LO>(prm, u - gridDim.x), prm, tmem, lane_off, r,
+                        sready_s, empty0, afree0, wg_leader, true, abort_flag);
                     owed = false;
                 }
             }
@@ -890,14 +987,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                     prev = e;
                     owed = true;
                 } else {
-                    alive = finish_stream<D, DEC, LO>(st, e, U, prm, tmem, lane_off, r, sready_s,
-                                                      empty0, afree0, wg_leader, false, abort_flag);
+                    alive = finish_stream<D, DEC, LO, COL>(st, e, U, prm, tmem, lane_off, r,
+                                                           sready_s, empty0, afree0, wg_leader,
+                                                           false, abort_flag);
                 }
             }
             st.ph0 += (uint32_t)st.cnt;
             it0 += U.n_items;
         }
-        if (!SAFE && __any_sync(0xffffffffu, st.over) && lane == 0) *prm.overflow = 1;
+        if (!SAFE && !COL && __any_sync(0xffffffffu, st.over) && lane == 0) *prm.overflow = 1;
     }
 
     tc_fence_before();
@@ -970,20 +1068,37 @@ template <int D, bool DEC, bool LO>
 cudaError_t launch(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c,
                    const CUtensorMap& l, const TcParams& prm, cudaStream_t st) {
     using Cf = Cfg<D, DEC, LO>;
-    cudaError_t e = ensure_smem_limit((const void*)tc_chain_kernel<D, DEC, false, LO>, Cf::kSmem);
+    cudaError_t e =
+        ensure_smem_limit((const void*)tc_chain_kernel<D, DEC, false, LO, false>, Cf::kSmem);
     if (e == cudaSuccess)
-        e = ensure_smem_limit((const void*)tc_chain_kernel<D, DEC, true, LO>, Cf::kSmem);
+        e = ensure_smem_limit((const void*)tc_chain_kernel<D, DEC, true, LO, false>, Cf::kSmem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = kNumSMs;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t grid = prm.n_units < sms ? prm.n_units : sms;
-    e = launch_pdl(tc_chain_kernel<D, DEC, false, LO>, dim3((unsigned)grid), dim3(kThreads),
+    e = launch_pdl(tc_chain_kernel<D, DEC, false, LO, false>, dim3((unsigned)grid), dim3(kThreads),
                    Cf::kSmem, st, a, b, c, l, prm);
     if (e == cudaSuccess)
-        e = launch_pdl(tc_chain_kernel<D, DEC, true, LO>, dim3((unsigned)grid), dim3(kThreads),
+        e = launch_pdl(tc_chain_kernel<D, DEC, true, LO, false>, dim3((unsigned)grid), dim3(kThreads),
                        Cf::kSmem, st, a, b, c, l, prm);
     return e;
+}
+
+// The encode with column statistics (one kernel: it cannot overflow).
+template <int D>
+cudaError_t launch_col(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c,
+                       const CUtensorMap& l, const TcParams& prm, cudaStream_t st) {
+    using Cf = Cfg<D, false, true, true>;
+    const cudaError_t e =
+        ensure_smem_limit((const void*)tc_chain_kernel<D, false, false, true, true>, Cf::kSmem);
+    if (e != cudaSuccess) return e;
+    int dev = 0, sms = kNumSMs;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t grid = prm.n_units < sms ? prm.n_units : sms;
+    return launch_pdl(tc_chain_kernel<D, false, false, true, true>, dim3((unsigned)grid),
+                      dim3(kThreads), Cf::kSmem, st, a, b, c, l, prm);
 }
 
 // `l` (the map of Q's lo tiles) is read only by the LO kernels (D <= 32).
@@ -1106,6 +1221,36 @@ cudaError_t tc_decode(const Plan& p, const void* K, float scale, void* Y, char* 
     prm.overflow = (int*)(ws + p.off_overflow) + 2;
     apply_fault(3, prm);
     return launch_d<true>(p.D, lo, ma, mb, mc, ml, prm, st);
+}
+
+cudaError_t tc_dz_pass(const Plan& p, const void* Qhi, const void* Qlo, const void* K,
+                       const void* dY, const float* L3, float scale, float* part, int* status,
+                       cudaStream_t st) {
+    CUtensorMap ma, mb, mc, ml;
+    if (!make_map(&ma, Qhi, p.D, p.M, p.BH, kTileRows) ||
+        !make_map(&ml, Qlo, p.D, p.M, p.BH, kTileRows) ||
+        !make_map(&mb, K, p.D, p.N, p.BH, item_rows<false>(p.D, true)) ||
+        !make_map(&mc, dY, p.D, p.N, p.BH, item_rows<false>(p.D, true)))
+        return cudaErrorInvalidValue;
+    TcParams prm{};
+    prm.BH = p.BH;
+    prm.H = p.H;
+    prm.N = p.N;
+    prm.M = p.M;
+    prm.c = scale * kLog2e;  // Q is not negated here: the sign stays in c
+    prm.chunk_len = p.chunk_len;
+    prm.nchunk = p.nchunk;
+    prm.n_groups = p.n_groups;
+    prm.pacc = part;
+    prm.n_units = p.BH * p.n_groups * p.nchunk;
+    prm.status = status;
+    prm.Lcol = L3;
+    test_fault_for(4, &prm.wait_ns, &prm.withhold_it);
+    switch (p.D) {
+        case 16: return launch_col<16>(ma, mb, mc, ml, prm, st);
+        case 32: return launch_col<32>(ma, mb, mc, ml, prm, st);
+    }
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace flarepp
