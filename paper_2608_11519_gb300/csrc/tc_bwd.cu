@@ -373,8 +373,7 @@ __global__ void __launch_bounds__(BCfg<D, PASS>::kThreads, 1)
     using C = BCfg<D, PASS, LO>;
     constexpr int NS = C::NS;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                               ~static_cast<uintptr_t>(1023));
+    uint8_t* smem = align_shared<1024>(smem_raw);
     uint8_t* abuf = smem;                          // kABuf x [NS][kNTA] A tiles
     uint8_t* ring = smem + C::kABuf * C::kABytes;  // kStages x kNTI item tiles, swizzled
     float* stats = reinterpret_cast<float*>(ring + C::kStages * C::kStage);  // [S][2][kItem]

@@ -130,8 +130,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     using C = GCfg<D>;
     constexpr int kS = C::kStages;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                               ~static_cast<uintptr_t>(1023));
+    uint8_t* smem = align_shared<1024>(smem_raw);
     uint8_t* staging = smem + kS * C::kStage;  // [kEpiGroups][kStaging]
     uint64_t* bars = reinterpret_cast<uint64_t*>(staging + kEpiGroups * C::kStaging);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::kNumBars);

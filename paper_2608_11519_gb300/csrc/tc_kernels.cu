@@ -657,8 +657,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!run) return;
     }
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                               ~static_cast<uintptr_t>(1023));
+    uint8_t* smem = align_shared<1024>(smem_raw);
     uint8_t* abuf = smem;                         // kABufS x NS x kANum A tiles
     // kStages x (B tile, C tile[, lo tile]), swizzled like the A tiles
     uint8_t* ring = smem + C::kABufS * C::kABytes;

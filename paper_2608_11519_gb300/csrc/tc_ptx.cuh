@@ -12,6 +12,14 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// The first N-aligned byte of shared memory from p on. By an offset, not by rounding the address as an
+// integer: the compiler then still knows that the pointer is to shared memory and loads and stores
+// through it as such (a generic access takes several times as long).
+template <uint32_t N>
+__device__ __forceinline__ uint8_t* align_shared(uint8_t* p) {
+    return p + ((N - (smem_u32(p) & (N - 1))) & (N - 1));
+}
+
 __device__ __forceinline__ uint64_t globaltimer_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

@@ -87,8 +87,8 @@ struct TokCfg {
     static constexpr int kOffStat = kOffRing + 2 * kStages * kStage;
     static constexpr int kOffBars = kOffStat + 4 * kMaxM * 4;
     // full[2][stages], empty[2][stages], afull[2], aready[2], afree[2], sready[2], pready[2],
-    // dsfree[2], accdone[2], accfree[2], statfull[2], segfree[2], dqdone, fin
-    static constexpr int kNumBars = 4 * kStages + 20 + 2;
+    // accdone[2], accfree[2], statfull[2], segfree[2], dqdone, fin
+    static constexpr int kNumBars = 4 * kStages + 18 + 2;
     static constexpr int kNeed = 1024 + kOffBars + kNumBars * 8 + 16;
     static constexpr int kSmem = kNeed > 122880 ? kNeed : 122880;  // one CTA per SM
     static_assert(kSmem <= 232448, "shared memory budget");
@@ -277,8 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     using C = TokCfg<D, CALL1, LO>;
     constexpr int kS = C::kStages;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                               ~static_cast<uintptr_t>(1023));
+    uint8_t* smem = align_shared<1024>(smem_raw);
     uint8_t* ds_buf = smem;
     uint8_t* abuf = smem + C::kOffA;
     uint8_t* ring = smem + C::kOffRing;
@@ -294,8 +293,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t afree0 = aready0 + 16u;
     const uint32_t sready0 = afree0 + 16u;
     const uint32_t pready0 = sready0 + 16u;
-    const uint32_t dsfree0 = pready0 + 16u;
-    const uint32_t accdone0 = dsfree0 + 16u;
+    const uint32_t accdone0 = pready0 + 16u;
     const uint32_t accfree0 = accdone0 + 16u;
     const uint32_t statfull0 = accfree0 + 16u;
     const uint32_t segfree0 = statfull0 + 16u;
@@ -316,7 +314,6 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(afree0 + 8u * k, 1);
             mbar_init(sready0 + 8u * k, 1);
             mbar_init(pready0 + 8u * k, 8);
-            mbar_init(dsfree0 + 8u * k, 1);
             mbar_init(accdone0 + 8u * k, 1);
             mbar_init(accfree0 + 8u * k, kSoftThreads);
             mbar_init(statfull0 + 8u * k, 32);
@@ -532,7 +529,6 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int k = 0; k < kRows / 16; ++k)
                 mma_ss(tmem + C::kColQ + b * D, desc_of(d0 + (k * 16 * kItem * 2 >> 4), kHiDs),
                        desc_of(k0 + 2 * D * k, kHi), C::kIdescQ, (!o.fresh || k > 0) ? 1u : 0u);
-            mma_commit(dsfree0 + 8u * buf);
             if (o.last) {
                 mma_commit(afree0 + 8u * ab);
                 mma_commit(accdone0 + 8u * ab);
@@ -726,14 +722,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             };
             for (int b = 0; b < prm.n_blocks; ++b, ++bg) {
                 const int item = 2 * b + s;
-                const uint32_t buf = bg & 1u;
-                if (item >= prm.n_items) {
-                    // no item in this block: only follow the buffer's phases
-                    if (bg >= 2 && !wait(dsfree0 + 8u * buf, (bg >> 1) - 1)) ok = false;
-                    if (ok) prep_next(b);
+                if (item >= prm.n_items) {  // no item in this block
+                    prep_next(b);
                     if (!ok) break;
                     continue;
                 }
+                // The issuer commits this item's S after the dK and dQ products of two blocks
+                // before, so S being ready also says that this dS buffer is free.
+                const uint32_t buf = bg & 1u;
                 if (!wait(sready0 + 8u * s, is)) {
                     ok = false;
                     break;
@@ -742,11 +738,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 uint32_t sa[16], ta[16];
                 tmem_ld16(colS, sa);
                 tmem_ld16(colT, ta);
-                // the dQ product of two blocks before has read this dS buffer
-                if (bg >= 2 && !wait(dsfree0 + 8u * buf, (bg >> 1) - 1)) ok = false;
                 tmem_wait_ld16(sa);
                 tmem_wait_ld16(ta);
-                if (!ok) break;
                 const int m0 = item * kItem + 32 * h;
                 const int nv = (int)prm.M - m0;  // valid columns from this warpgroup's first on
                 const float* c0 = st0 + m0;
