@@ -171,7 +171,8 @@ flarepp_status route_impl(const flarepp_shape* shape, const void* seeds, const v
 // FLARE (Sec. 3, eq. prelim_flare_sdpa): Z = SDPA(Q_h, K, V), Y = SDPA(K, Q_h, Z) with learned
 // queries Q [H, M, D] shared by the batch. The routing chain without its first call: the
 // encode runs as call 1 does (A = the per-head queries), its merge writes Z, and the decode
-// reads a per-(b, h) copy of Q as its keys.
+// reads the per-head queries as its keys (a copy of Q for every batch element before it took, with
+// B = 32, as long as the encode: 276 us a call at the longseq shape, now 140).
 flarepp_status flare_impl(const flarepp_shape* shape, const void* Qh, const void* K, const void* V,
                           float scale, void* Y, void* workspace, size_t workspace_bytes,
                           void* stream, float* Z_out, bool reset_status = true) {
@@ -227,15 +228,11 @@ flarepp_status flare_impl(const flarepp_shape* shape, const void* Qh, const void
     cudaError_t e = tc ? tc_encode(p, 1, K, V, Qh, scale, ws, st)
                        : simt_encode_f32(p, 1, K, V, Qh, scale, ws, st);
     if (e != cudaSuccess || combine(p, 2, ws, false, st) != cudaSuccess) return FLAREPP_ERR_CUDA;
-    // the decode's keys: Q for every batch element (on the tensor-core path the bf16 operand,
-    // negated for a negative scale as the chain's call-1 merge does)
-    const void* qsrc = tc && neg ? (const void*)(ws + p.off_seedneg) : Qh;
-    char* qdst = ws + (tc ? p.off_qop : p.off_q32);
-    for (int64_t b = 0; b < p.B; ++b)
-        if (cudaMemcpyAsync(qdst + (size_t)b * q_bytes, qsrc, q_bytes, cudaMemcpyDeviceToDevice,
-                            st) != cudaSuccess)
-            return FLAREPP_ERR_CUDA;
-    e = tc ? tc_decode(p, K, scale, Y, ws, st) : simt_decode_f32(p, K, scale, Y, ws, st);
+    // the decode's keys: the heads' Q, shared by the batch (on the tensor-core path negated for a
+    // negative scale as the chain's call-1 merge does)
+    const void* q = tc && neg ? (const void*)(ws + p.off_seedneg) : Qh;
+    e = tc ? tc_decode(p, K, scale, Y, ws, st, nullptr, false, q)
+           : simt_decode_f32(p, K, scale, Y, ws, st, nullptr, (const float*)q);
     if (e != cudaSuccess) return FLAREPP_ERR_CUDA;
     if (Z_out && cudaMemcpyAsync(Z_out, ws + p.off_z32, z_bytes, cudaMemcpyDeviceToDevice, st) !=
                      cudaSuccess)

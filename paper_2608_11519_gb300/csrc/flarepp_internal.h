@@ -114,8 +114,9 @@ cudaError_t simt_encode_f32(const Plan& p, int call, const void* k, const void* 
                             const void* seeds, float scale, char* ws, cudaStream_t st);
 // Decode (call 3) on CUDA cores: Y = SDPA(K, Q32, Z32); also the base-2 log-normaliser of
 // each token's row into `lse` [BH][N] when it is not null.
+// Qh: when set, the keys are these [H][M][D] queries instead of Q32 (FLARE).
 cudaError_t simt_decode_f32(const Plan& p, const void* K, float scale, void* Y, char* ws,
-                            cudaStream_t st, float* lse = nullptr);
+                            cudaStream_t st, float* lse = nullptr, const float* Qh = nullptr);
 
 // ---- backward (bwd.cu): the passes of App. A.5. f32 inputs run on CUDA cores, bf16 inputs
 // on the tensor-core passes of tc_bwd.cu. `saved` is the training forward's state, `ws`
@@ -252,7 +253,9 @@ cudaError_t tc_dz_pass(const Plan& p, const void* Qhi, const void* Qlo, const vo
 // Decode call 3: Y = SDPA(K, Q, Z) from the Q and Z operand copies; also each token's
 // base-2 log-normaliser into `lse` [BH][N] when it is not null. With `lo` (D <= 32) the
 // scores take Q as its hi and lo bf16 operands.
+// Qh: when set, the keys are these [H][M][D] bf16 queries instead of the Q operand (FLARE).
 cudaError_t tc_decode(const Plan& p, const void* K, float scale, void* Y, char* ws,
-                      cudaStream_t st, float* lse = nullptr, bool lo = false);
+                      cudaStream_t st, float* lse = nullptr, bool lo = false,
+                      const void* Qh = nullptr);
 
 }  // namespace flarepp

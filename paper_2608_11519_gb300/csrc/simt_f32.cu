@@ -9,8 +9,8 @@ cudaError_t simt_encode_f32(const Plan& p, int call, const void* k, const void* 
 }
 
 cudaError_t simt_decode_f32(const Plan& p, const void* K, float scale, void* Y, char* ws,
-                          cudaStream_t st, float* lse) {
-    return simt::decode_t<float>(p, K, scale, Y, ws, st, lse);
+                          cudaStream_t st, float* lse, const float* Qh) {
+    return simt::decode_t<float>(p, K, scale, Y, ws, st, lse, Qh);
 }
 
 }  // namespace flarepp

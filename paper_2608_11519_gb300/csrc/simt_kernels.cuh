@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(128) simt_encode_kernel(
 template <int D, typename T>
 __global__ void __launch_bounds__(128) simt_decode_kernel(
     const T* __restrict__ k, const float* __restrict__ q32, const float* __restrict__ z32,
-    int64_t N, int64_t M, float sl2, T* __restrict__ y, float* __restrict__ lse) {
+    int64_t q_heads, int64_t N, int64_t M, float sl2, T* __restrict__ y, float* __restrict__ lse) {
     __shared__ float qs[kTile][D];
     __shared__ float zs[kTile][D];
     const int64_t ntiles = (N + 127) / 128;
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(128) simt_decode_kernel(
         o[d] = 0.f;
     }
     float mx = -INFINITY, l = 0.f;
-    const float* qb = q32 + bh * M * D;
+    const float* qb = q32 + bh % q_heads * M * D;  // q_heads: BH, or H when the batch shares Q
     const float* zb = z32 + bh * M * D;
     for (int64_t m0 = 0; m0 < M; m0 += kTile) {
         const int cnt = (int)min((int64_t)kTile, M - m0);
@@ -207,22 +207,23 @@ cudaError_t encode_t(const Plan& p, int call, const void* k, const void* v, cons
 
 template <typename T>
 cudaError_t decode_t(const Plan& p, const void* K, float scale, void* Y, char* ws,
-                     cudaStream_t st, float* lse) {
+                     cudaStream_t st, float* lse, const float* Qh) {
     const int64_t blocks = ((p.N + 127) / 128) * p.BH;
     const float sl2 = scale * kLog2e;
-    const float* q32 = (const float*)(ws + p.off_q32);
+    const float* q32 = Qh ? Qh : (const float*)(ws + p.off_q32);
+    const int64_t q_heads = Qh ? p.H : p.BH;
     const float* z32 = (const float*)(ws + p.off_z32);
     switch (p.D) {
         case 16:
-            simt_decode_kernel<16, T><<<(unsigned)blocks, 128, 0, st>>>((const T*)K, q32, z32, p.N,
+            simt_decode_kernel<16, T><<<(unsigned)blocks, 128, 0, st>>>((const T*)K, q32, z32, q_heads, p.N,
                                                                          p.M, sl2, (T*)Y, lse);
             break;
         case 32:
-            simt_decode_kernel<32, T><<<(unsigned)blocks, 128, 0, st>>>((const T*)K, q32, z32, p.N,
+            simt_decode_kernel<32, T><<<(unsigned)blocks, 128, 0, st>>>((const T*)K, q32, z32, q_heads, p.N,
                                                                          p.M, sl2, (T*)Y, lse);
             break;
         case 64:
-            simt_decode_kernel<64, T><<<(unsigned)blocks, 128, 0, st>>>((const T*)K, q32, z32, p.N,
+            simt_decode_kernel<64, T><<<(unsigned)blocks, 128, 0, st>>>((const T*)K, q32, z32, q_heads, p.N,
                                                                          p.M, sl2, (T*)Y, lse);
             break;
         default: return cudaErrorInvalidValue;

@@ -147,6 +147,7 @@ struct Cfg {
 struct TcParams {
     int64_t BH, H, N, M;
     int a_per_head;  // encode call 1: the A operand (seeds) is indexed by head
+    int b_per_head;  // FLARE's decode: the items' first tile (the learned Q) is indexed by head
     float c;         // |scale| * log2(e)
     int64_t chunk_len, nchunk, n_groups;
     float* pmax;
@@ -211,7 +212,7 @@ __device__ __forceinline__ Unit get_unit(const TcParams& p, int64_t u64) {
         U.item0 = U.chunk * p.chunk_len;
         U.item_end = min(p.N, U.item0 + p.chunk_len);
     }
-    U.zB = (int)U.bh;
+    U.zB = (int)(p.b_per_head ? (uint32_t)U.bh % (uint32_t)p.H : (uint32_t)U.bh);
     U.n_items = (int)((U.item_end - U.item0 + C::kItem - 1) / C::kItem);
     return U;
 }
@@ -882,7 +883,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const int row = (int)(U.item0 + (int64_t)i * C::kItem);
                         const uint32_t dst = smem_u32(ring + st * C::kStage);
                         tma_load_3d(dst, &tmB, 0, row, U.zB, full0 + 8u * st);
-                        tma_load_3d(dst + C::kItemTile, &tmC, 0, row, U.zB, full0 + 8u * st);
+                        tma_load_3d(dst + C::kItemTile, &tmC, 0, row, (int)U.bh, full0 + 8u * st);
                         if constexpr (C::kLoB)
                             tma_load_3d(dst + 2 * C::kItemTile, &tmL, 0, row, U.zB,
                                         full0 + 8u * st);
@@ -1195,11 +1196,12 @@ cudaError_t tc_encode(const Plan& p, int call, const void* k, const void* v, con
 }
 
 cudaError_t tc_decode(const Plan& p, const void* K, float scale, void* Y, char* ws,
-                      cudaStream_t st, float* lse, bool lo) {
+                      cudaStream_t st, float* lse, bool lo, const void* Qh) {
     CUtensorMap ma, mb, mc, ml;
     lo = lo && p.D <= 32;
     if (!make_map(&ma, K, p.D, p.N, p.BH, kTileRows) ||
-        !make_map(&mb, ws + p.off_qop, p.D, p.M, p.BH, item_rows<true>(p.D, lo)) ||
+        !make_map(&mb, Qh ? Qh : ws + p.off_qop, p.D, p.M, Qh ? p.H : p.BH,
+                  item_rows<true>(p.D, lo)) ||
         !make_map(&mc, ws + p.off_zop, p.D, p.M, p.BH, item_rows<true>(p.D, lo)))
         return cudaErrorInvalidValue;
     ml = ma;
@@ -1211,6 +1213,7 @@ cudaError_t tc_decode(const Plan& p, const void* K, float scale, void* Y, char* 
     prm.N = p.N;
     prm.M = p.M;
     prm.c = fabsf(scale) * kLog2e;
+    prm.b_per_head = Qh ? 1 : 0;
     const int64_t grp = tc_group_rows(p.D);
     prm.n_tok_groups = (p.N + grp - 1) / grp;
     prm.Y = (__nv_bfloat16*)Y;
