@@ -79,30 +79,37 @@ constexpr float kFastLimit = 281474976710656.0f;  // 2^48
 // shared-memory A buffer (the lo tile after the hi tile); the decode's items carry Q's lo tile
 // as a third tile.
 // COL (the backward's dZ, an encode): every item also carries its tokens' L3.
-template <int D, bool DEC, bool LO = false, bool COL = false>
+// DEC: 0 the encode, else a form of the decode: kNarrow with 64-route items and, at D <= 32, two O
+// accumulators per stream, kWide with items as wide as 512 TMEM columns allow beside one O.
+constexpr int kNarrow = 1, kWide = 2;
+template <int D, int DEC, bool LO = false, bool COL = false>
 struct Cfg {
     static_assert(!LO || D <= 32, "the hi/lo form of Q serves D = 16 and 32");
-    static_assert(!(COL && DEC), "column statistics belong to the encode");
+    static_assert(!COL || !DEC, "column statistics belong to the encode");
     static constexpr bool kLoA = LO && !DEC;  // encode of call 2: A = Q as hi and lo tiles
     static constexpr bool kLoB = LO && DEC;   // decode: every item also carries Q's lo tile
     static constexpr int kANum = kLoA ? 2 : 1;  // A tiles per stream
     // The A tiles (the route tiles in the encode, the token tiles in the decode) stay in shared
     // memory where the TMA puts them, swizzled like the ring tiles, and the MMAs read them there
     // (`ss` score products); nothing copies them into TMEM, so all 512 columns go to the score
-    // tiles and accumulators. The encode's units are long (hundreds of items): one A buffer,
-    // and items of 96 tokens (112 at D = 16; 64 at D = 64: S 4 x 64 + O 4 x 64 columns), so
-    // the per-item round trip is paid once per 96 tokens. The decode's units are only M/64
-    // items, so per-unit costs show: its A tiles are double-buffered so the next unit's land
-    // during this one, and where TMEM has the room (D <= 32) it keeps two O accumulators per
-    // stream, one per unit parity, so that a unit's epilogue can wait until the next unit's
-    // first item is under way; at D = 64 the columns instead widen its items to 48 routes
-    // (S 4 x 48 + O 4 x 64).
-    static constexpr int kItem = D == 64 ? (DEC ? 48 : 64) : (DEC ? 64 : (D == 16 ? 112 : 96));
+    // tiles and accumulators. The handoffs of an item between the MMA warp and the softmax cost a
+    // fixed time whatever its width, so items are wide: 96 tokens or routes at D = 32, 112 at
+    // D = 16, 64 at D = 64 (4 x S + 4 x O = 512 columns). The encode's units are long (hundreds of
+    // items): one A buffer. The decode's units are only M / 96 items, so per-unit costs show: its
+    // A tiles are double-buffered so the next unit's land during this one. Its narrow form keeps
+    // two O accumulators per stream, one per unit parity, so that a unit's epilogue can wait until
+    // the next unit's first item is under way.
+    // Which decode: the wide one when it takes fewer items per unit (launch_d). Decode of
+    // 8 x 262,144 tokens, narrow / wide: D = 32, M = 128 74 / 76 us, M = 512 209 / 199, M = 2048
+    // 734 / 678; D = 16, M = 64 47 / 49, M = 512 201 / 184. At D = 64 (narrow: one O either way)
+    // 48 -> 64 routes an item: M = 512 276 -> 254, M = 128 139 -> 127. With Q's lo tiles (the
+    // training forward) the narrow one is faster at every M: D = 32, M = 512 218 / 233.
+    static constexpr int kItem = D == 64 || DEC == kNarrow ? 64 : (D == 16 ? 112 : 96);
     static constexpr int B = 1;                         // score buffers per stream
     // shared-memory A buffers (four for the decode at small M measured no faster than two)
     static constexpr int kABufS = DEC ? 2 : 1;
     static constexpr int kAAhead = kABufS > 1 ? kABufS - 1 : 1;  // units the A copies run ahead
-    static constexpr int kOBuf = (DEC && D <= 32) ? 2 : 1;    // O accumulators per stream
+    static constexpr int kOBuf = (DEC == kNarrow && D <= 32) ? 2 : 1;    // O accumulators per stream
     static constexpr int kGroup = NS * kTileRows;     // resident rows per work unit
     static constexpr int kATile = kTileRows * D * 2;  // one 128-row operand tile
     static constexpr int kABytes = NS * kANum * kATile;
@@ -114,10 +121,11 @@ struct Cfg {
     // route tiles gives each stream one token parity) looks ahead only kStages / n_par of its
     // own items, and the copy of its next item cannot start before the stream frees the stage
     // kStages items back; so the encode takes as many stages as shared memory holds, up to 16.
-    // The decode's streams take every item, and 8 stages cover the copy latency.
+    // The decode's streams take every item, and 8 stages cover the copy latency (6 at D = 64, what
+    // shared memory leaves beside the A buffers).
     static constexpr int kStat = COL ? kItem * 4 : 0;  // bytes of an item's column statistics
     static constexpr int kStagesFit = (232448 - 2048 - kABufS * kABytes) / (kStage + kStat);
-    static constexpr int kStages = DEC ? 8 : (kStagesFit < 16 ? kStagesFit : 16);
+    static constexpr int kStages = DEC ? (D == 64 ? 6 : 8) : (kStagesFit < 16 ? kStagesFit : 16);
     // barriers: full[S], empty[S], a_full[kABufS] (a unit's A tiles landed), a_free[kABufS]
     //           (one arrive per softmax warpgroup once it has seen the unit's last S: the
     //           buffer may be refilled), sync[NS][2] = {s_ready, o_done} per stream (S of an
@@ -140,7 +148,7 @@ struct Cfg {
     static constexpr uint32_t kColO = NS * B * kItem;  // kOBuf x NS x D
     static_assert(kColO + kOBuf * NS * D <= kTmemCols, "TMEM budget");
     static_assert(kSmem <= 232448, "shared memory budget");
-    static_assert(kStages >= 2 * B * NS, "ring depth: the full wait precedes the PV");
+    static_assert(kStages >= (DEC ? 4 : 2 * B * NS), "ring depth: the full wait precedes the PV");
     static_assert(B == 1, "the s_ready / o_done protocol has one score buffer per stream");
 };
 
@@ -181,7 +189,7 @@ struct Unit {
 // The plan keeps unit counts, and so every quotient below, within 32 bits; 32-bit divisions by
 // runtime values cost a few instructions where 64-bit ones cost about seventy.
 // (the same for the forms with a lo operand or column statistics: they cut the work alike)
-template <int D, bool DEC, bool LO>
+template <int D, int DEC, bool LO>
 __device__ __forceinline__ Unit get_unit(const TcParams& p, int64_t u64) {
     using C = Cfg<D, DEC, LO>;
     const uint32_t u = (uint32_t)u64;
@@ -298,7 +306,9 @@ __device__ __forceinline__ float chunk_max(const uint32_t* sr, int base, int nv)
 // P = 2^(c S - m) for one chunk of W = 32 or 16 columns, packed bf16 pairs into
 // pr[0 .. W/2); returns the chunk's row sum. Columns at or beyond nv are not part of the
 // softmax: probability 0.
-template <int W>
+// (The wide decode's last item of a unit often ends before its last chunk, which then has no column
+// at all; elsewhere that test would only cost: 1 % in the encode.)
+template <int W, int DEC>
 __device__ __forceinline__ float exp_chunk(const uint32_t* sr, uint32_t* pr, int base, int nv,
                                            float c, uint64_t c2, float m) {
     if (base + W <= nv) {
@@ -315,6 +325,11 @@ __device__ __forceinline__ float exp_chunk(const uint32_t* sr, uint32_t* pr, int
         unpack_f32x2(acc0, a, b);
         unpack_f32x2(acc1, x, y);
         return (a + b) + (x + y);
+    }
+    if (DEC == kWide && base >= nv) {
+#pragma unroll
+        for (int k = 0; k < W / 2; ++k) pr[k] = 0u;
+        return 0.f;
     }
     float t0 = 0.f, t1 = 0.f;
 #pragma unroll
@@ -370,7 +385,7 @@ __device__ __forceinline__ void exp_chunk_col(const uint32_t* sr, uint32_t* pr, 
 // STORE (the fast kernel): each chunk's P goes back to TMEM as soon as it is packed (it covers
 // only columns already read), so S is gone by the end. Otherwise P stays in pr for the
 // caller, and S stays intact until the caller writes it.
-template <int ITEM, bool FIRST_REF, bool STORE>
+template <int ITEM, int DEC, bool FIRST_REF, bool STORE>
 __device__ __forceinline__ float exp_tile(uint32_t scol, uint32_t* pr, int nv, float c,
                                           uint64_t c2, float& m, bool first) {
     float sum = 0.f;
@@ -380,7 +395,7 @@ __device__ __forceinline__ float exp_tile(uint32_t scol, uint32_t* pr, int nv, f
         tmem_ld32(scol + 32 * h, sr);
         tmem_wait_ld32(sr);
         if (FIRST_REF && h == 0 && first) m = c * __uint_as_float(sr[0]);
-        sum += exp_chunk<32>(sr, pr + 16 * h, 32 * h, nv, c, c2, m);
+        sum += exp_chunk<32, DEC>(sr, pr + 16 * h, 32 * h, nv, c, c2, m);
         if constexpr (STORE) tmem_st16(scol + 16 * h, pr + 16 * h);
     }
     if constexpr (ITEM % 32 == 16) {
@@ -388,7 +403,7 @@ __device__ __forceinline__ float exp_tile(uint32_t scol, uint32_t* pr, int nv, f
         uint32_t sr[16];
         tmem_ld16(scol + base, sr);
         tmem_wait_ld16(sr);
-        sum += exp_chunk<16>(sr, pr + base / 2, base, nv, c, c2, m);
+        sum += exp_chunk<16, DEC>(sr, pr + base / 2, base, nv, c, c2, m);
         if constexpr (STORE) tmem_st8(scol + base / 2, pr + base / 2);
     }
     return sum;
@@ -422,7 +437,7 @@ __device__ __forceinline__ void store_p(uint32_t scol, uint32_t* pr) {
 //     takes the first item's reference from its first score; the encode, whose units are
 //     long, takes the first item's exact maximum).
 //   COL: P from the item's column statistics (the stage's full barrier covers their copies).
-template <int D, bool DEC, bool SAFE, bool LO, bool COL>
+template <int D, int DEC, bool SAFE, bool LO, bool COL>
 __device__ __forceinline__ bool softmax_step(SoftmaxStream& S, const Unit& U, uint32_t tmem,
                                              uint32_t lane_off, float c, uint64_t c2,
                                              uint32_t sready_s, uint32_t pready_s, uint32_t empty0,
@@ -487,7 +502,7 @@ __device__ __forceinline__ bool softmax_step(SoftmaxStream& S, const Unit& U, ui
         return true;
     }
     if constexpr (!SAFE) {
-        sum = exp_tile<C::kItem, true, true>(scol, pr, nv, c, c2, S.m, j == 0);
+        sum = exp_tile<C::kItem, DEC, true, true>(scol, pr, nv, c, c2, S.m, j == 0);
         tmem_wait_st();
         tc_fence_before();
         mbar_arrive(pready_s + 8u * b);
@@ -498,7 +513,7 @@ __device__ __forceinline__ bool softmax_step(SoftmaxStream& S, const Unit& U, ui
     }
     bool slow = !DEC && j == 0;
     if (!slow) {
-        sum = exp_tile<C::kItem, DEC, false>(scol, pr, nv, c, c2, S.m, j == 0);
+        sum = exp_tile<C::kItem, DEC, DEC != 0, false>(scol, pr, nv, c, c2, S.m, j == 0);
         slow = __any_sync(0xffffffffu, !(sum <= kFastLimit));
     }
     if (slow) {
@@ -540,7 +555,7 @@ __device__ __forceinline__ bool softmax_step(SoftmaxStream& S, const Unit& U, ui
                 tmem_st16(ocol + 16 * k, o);
             }
         }
-        sum = exp_tile<C::kItem, false, false>(scol, pr, nv, c, c2, S.m, false);
+        sum = exp_tile<C::kItem, DEC, false, false>(scol, pr, nv, c, c2, S.m, false);
     }
     S.l += sum;
     store_p<C::kItem>(scol, pr);
@@ -566,7 +581,7 @@ struct UnitEnd {
     uint32_t it0;
 };
 
-template <int D, bool DEC, bool LO, bool COL>
+template <int D, int DEC, bool LO, bool COL>
 __device__ __forceinline__ bool finish_stream(SoftmaxStream& S, const UnitEnd& E, const Unit& U,
                                               const TcParams& prm, uint32_t tmem,
                                               uint32_t lane_off, int r, uint32_t sready_s,
@@ -642,7 +657,7 @@ __device__ __forceinline__ bool finish_stream(SoftmaxStream& S, const UnitEnd& E
 
 // ------------------------------------------------------------------ the kernel
 
-template <int D, bool DEC, bool SAFE, bool LO, bool COL>
+template <int D, int DEC, bool SAFE, bool LO, bool COL>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_chain_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmL,
@@ -1064,7 +1079,7 @@ bool make_map(CUtensorMap* m, const void* base, int64_t D, int64_t rows, int64_t
 
 // The fast kernel, then the safe one on the same stream (it returns at once unless the
 // fast kernel raised the overflow word, which the plan keeps zeroed before each call).
-template <int D, bool DEC, bool LO>
+template <int D, int DEC, bool LO>
 cudaError_t launch(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c,
                    const CUtensorMap& l, const TcParams& prm, cudaStream_t st) {
     using Cf = Cfg<D, DEC, LO>;
@@ -1089,34 +1104,36 @@ cudaError_t launch(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap
 template <int D>
 cudaError_t launch_col(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c,
                        const CUtensorMap& l, const TcParams& prm, cudaStream_t st) {
-    using Cf = Cfg<D, false, true, true>;
+    using Cf = Cfg<D, 0, true, true>;
     const cudaError_t e =
-        ensure_smem_limit((const void*)tc_chain_kernel<D, false, false, true, true>, Cf::kSmem);
+        ensure_smem_limit((const void*)tc_chain_kernel<D, 0, false, true, true>, Cf::kSmem);
     if (e != cudaSuccess) return e;
     int dev = 0, sms = kNumSMs;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t grid = prm.n_units < sms ? prm.n_units : sms;
-    return launch_pdl(tc_chain_kernel<D, false, false, true, true>, dim3((unsigned)grid),
+    return launch_pdl(tc_chain_kernel<D, 0, false, true, true>, dim3((unsigned)grid),
                       dim3(kThreads), Cf::kSmem, st, a, b, c, l, prm);
 }
 
 // `l` (the map of Q's lo tiles) is read only by the LO kernels (D <= 32).
-template <bool DEC>
+template <int DEC>
 cudaError_t launch_d(int64_t D, bool lo, const CUtensorMap& a, const CUtensorMap& b,
                      const CUtensorMap& c, const CUtensorMap& l, const TcParams& prm,
                      cudaStream_t st) {
     if (lo) {
+        constexpr int kForm = DEC != 0 ? kNarrow : 0;
         switch (D) {
-            case 16: return launch<16, DEC, true>(a, b, c, l, prm, st);
-            case 32: return launch<32, DEC, true>(a, b, c, l, prm, st);
+            case 16: return launch<16, kForm, true>(a, b, c, l, prm, st);
+            case 32: return launch<32, kForm, true>(a, b, c, l, prm, st);
         }
         return cudaErrorInvalidValue;
     }
     switch (D) {
         case 16: return launch<16, DEC, false>(a, b, c, l, prm, st);
         case 32: return launch<32, DEC, false>(a, b, c, l, prm, st);
-        case 64: return launch<64, DEC, false>(a, b, c, l, prm, st);
+        case 64:  // (the wide decode is the narrow one there)
+            return launch<64, DEC != 0 ? kNarrow : 0, false>(a, b, c, l, prm, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -1124,13 +1141,13 @@ cudaError_t launch_d(int64_t D, bool lo, const CUtensorMap& a, const CUtensorMap
 }  // namespace
 
 // Streamed rows per item (the TMA box height of the ring tiles) of the encode or decode.
-template <bool DEC>
+template <int DEC>
 uint32_t item_rows(int64_t D, bool lo = false) {
     if (lo) return D == 16 ? Cfg<16, DEC, true>::kItem : Cfg<32, DEC, true>::kItem;
     return D == 16 ? Cfg<16, DEC>::kItem : (D == 32 ? Cfg<32, DEC>::kItem : Cfg<64, DEC>::kItem);
 }
 
-int64_t tc_encode_item_rows(int64_t D) { return item_rows<false>(D); }
+int64_t tc_encode_item_rows(int64_t D) { return item_rows<0>(D); }
 
 void test_fault_for(int kernel, uint64_t* wait_ns, int64_t* ring_item) {
     std::lock_guard<std::mutex> lock(g_fault_mu);
@@ -1169,8 +1186,8 @@ cudaError_t tc_encode(const Plan& p, int call, const void* k, const void* v, con
         a_z = p.BH;
     }
     if (!make_map(&ma, a_src, p.D, p.M, a_z, kTileRows) ||
-        !make_map(&mb, k, p.D, p.N, p.BH, item_rows<false>(p.D, lo)) ||
-        !make_map(&mc, v, p.D, p.N, p.BH, item_rows<false>(p.D, lo)))
+        !make_map(&mb, k, p.D, p.N, p.BH, item_rows<0>(p.D, lo)) ||
+        !make_map(&mc, v, p.D, p.N, p.BH, item_rows<0>(p.D, lo)))
         return cudaErrorInvalidValue;
     ml = ma;
     if (lo && !make_map(&ml, ws + p.off_qlo, p.D, p.M, a_z, kTileRows))
@@ -1192,20 +1209,24 @@ cudaError_t tc_encode(const Plan& p, int call, const void* k, const void* v, con
     prm.status = (int*)(ws + p.off_status);
     prm.overflow = (int*)(ws + p.off_overflow) + (call - 1);
     apply_fault(call, prm);
-    return launch_d<false>(p.D, lo, ma, mb, mc, ml, prm, st);
+    return launch_d<0>(p.D, lo, ma, mb, mc, ml, prm, st);
 }
 
 cudaError_t tc_decode(const Plan& p, const void* K, float scale, void* Y, char* ws,
                       cudaStream_t st, float* lse, bool lo, const void* Qh) {
     CUtensorMap ma, mb, mc, ml;
     lo = lo && p.D <= 32;
+    // the wide form when its units have fewer items, but not with Q's lo tiles
+    const int64_t narrow = item_rows<kNarrow>(p.D, lo), wide = item_rows<kWide>(p.D, lo);
+    const bool use_wide = !lo && cdiv(p.M, wide) < cdiv(p.M, narrow);
+    const uint32_t item = (uint32_t)(use_wide ? wide : narrow);
     if (!make_map(&ma, K, p.D, p.N, p.BH, kTileRows) ||
         !make_map(&mb, Qh ? Qh : ws + p.off_qop, p.D, p.M, Qh ? p.H : p.BH,
-                  item_rows<true>(p.D, lo)) ||
-        !make_map(&mc, ws + p.off_zop, p.D, p.M, p.BH, item_rows<true>(p.D, lo)))
+                  item) ||
+        !make_map(&mc, ws + p.off_zop, p.D, p.M, p.BH, item))
         return cudaErrorInvalidValue;
     ml = ma;
-    if (lo && !make_map(&ml, ws + p.off_qlo, p.D, p.M, p.BH, item_rows<true>(p.D, lo)))
+    if (lo && !make_map(&ml, ws + p.off_qlo, p.D, p.M, p.BH, item))
         return cudaErrorInvalidValue;
     TcParams prm{};
     prm.BH = p.BH;
@@ -1222,7 +1243,8 @@ cudaError_t tc_decode(const Plan& p, const void* K, float scale, void* Y, char* 
     prm.status = (int*)(ws + p.off_status);
     prm.overflow = (int*)(ws + p.off_overflow) + 2;
     apply_fault(3, prm);
-    return launch_d<true>(p.D, lo, ma, mb, mc, ml, prm, st);
+    return use_wide ? launch_d<kWide>(p.D, lo, ma, mb, mc, ml, prm, st)
+                    : launch_d<kNarrow>(p.D, lo, ma, mb, mc, ml, prm, st);
 }
 
 cudaError_t tc_dz_pass(const Plan& p, const void* Qhi, const void* Qlo, const void* K,
@@ -1231,8 +1253,8 @@ cudaError_t tc_dz_pass(const Plan& p, const void* Qhi, const void* Qlo, const vo
     CUtensorMap ma, mb, mc, ml;
     if (!make_map(&ma, Qhi, p.D, p.M, p.BH, kTileRows) ||
         !make_map(&ml, Qlo, p.D, p.M, p.BH, kTileRows) ||
-        !make_map(&mb, K, p.D, p.N, p.BH, item_rows<false>(p.D, true)) ||
-        !make_map(&mc, dY, p.D, p.N, p.BH, item_rows<false>(p.D, true)))
+        !make_map(&mb, K, p.D, p.N, p.BH, item_rows<0>(p.D, true)) ||
+        !make_map(&mc, dY, p.D, p.N, p.BH, item_rows<0>(p.D, true)))
         return cudaErrorInvalidValue;
     TcParams prm{};
     prm.BH = p.BH;
