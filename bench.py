@@ -34,7 +34,7 @@ UNIT = "token·heads/s"
 # the files that fix what a kernel launch reads and writes: the kernels and the plan that
 # sets their launch configuration (the C ABI's argument handling is not among them)
 KERNEL_SOURCES = tuple("paper_2608_11519_gb300/csrc/" + f for f in (
-    "combine.cu", "flarepp_internal.h", "plan.cu", "simt_f32.cu", "simt_kernels.cuh",
+    "combine.cu", "flarepp_internal.h", "plan.cu", "simt_f32.cu", "simt_kernels.cuh", "simt_math.cuh",
     "tc_kernels.cu", "tc_ptx.cuh"))
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0,
                   "source": "fallback"}

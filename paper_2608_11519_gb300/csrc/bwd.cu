@@ -14,14 +14,16 @@
 //
 // Two kernel shapes cover it on CUDA cores. A route pass gives one thread per route and
 // streams a chunk of tokens, accumulating the latent-side sums (dZ, dQ, dQs) into per-chunk
-// partials that a reduce kernel adds in chunk order. A token pass gives one thread per
-// token and streams every route, producing that token's dK, dV (calls 2 and 3 together) or
+// partials that a reduce kernel adds in chunk order. A token pass gives two threads to one or two
+// tokens and streams every route, producing that token's dK, dV (calls 2 and 3 together) or
 // dKt, dVt (call 1). The tensor-core path has the same structure (passes R3, T23, R2, T1,
 // R1) with bf16 copies of Q, Z, dZ and dQ as MMA operands.
 #include <cuda_bf16.h>
 #include <math.h>
 
 #include "flarepp_internal.h"
+#include "simt_math.cuh"
+#include "tc_ptx.cuh"
 
 namespace flarepp {
 namespace {
@@ -34,15 +36,6 @@ __device__ __forceinline__ float ld_f32(const float* p) { return *p; }
 __device__ __forceinline__ float ld_f32(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 __device__ __forceinline__ void st_out(float* p, float x) { *p = x; }
 __device__ __forceinline__ void st_out(__nv_bfloat16* p, float x) { *p = __float2bfloat16_rn(x); }
-
-// The bf16 forward multiplies bf16 copies of Q and Z (its MMA operands); the backward
-// differentiates that same function, so on the bf16 path it rounds Q and Z alike wherever
-// they enter a product (logits, and Z in call 3's values).
-template <typename T>
-__device__ __forceinline__ float operand(float x) {
-    if constexpr (sizeof(T) == 2) return __bfloat162float(__float2bfloat16_rn(x));
-    return x;
-}
 
 __device__ __forceinline__ float ex2(float x) {
     float y;
@@ -101,7 +94,7 @@ __global__ void to_bf16_hilo_kernel(const float* __restrict__ src, __nv_bfloat16
     }
 }
 
-// Route pass of call MODE (3, 2 or 1) over one chunk of tokens; thread = route m.
+// Route pass of call MODE (3, 2 or 1) over one chunk of tokens, float32; thread = route m.
 //   MODE 3: a = Q, keys b = K, w = dY, g = Z, column statistics L3[n], c3[n];
 //           pa += P w (dZ), pb += dS k (dQ / s)
 //   MODE 2: a = Q, keys = K, w = V, g = dZ, row statistics L2[m], c2[m]; pb += dS k
@@ -109,16 +102,19 @@ __global__ void to_bf16_hilo_kernel(const float* __restrict__ src, __nv_bfloat16
 //           pb += dS kt
 // dS here is P o (dP - c); the factor s is applied by the reduce.
 // grid.x = nchunk * n_mtiles * BH; block = m_tile threads.
-template <int D, typename T, typename AT, int MODE>
-__global__ void __launch_bounds__(128) route_pass_kernel(
-    const AT* __restrict__ a, int a_per_head, const T* __restrict__ kb, const T* __restrict__ wb,
-    const float* __restrict__ g, const float* __restrict__ Lrow, const float* __restrict__ crow,
-    const float* __restrict__ Lcol, const float* __restrict__ ccol, int64_t H, int64_t N,
-    int64_t M, int64_t chunk_len, int64_t nchunk, int64_t n_mtiles, float sl2,
-    float* __restrict__ pa, float* __restrict__ pb) {
-    __shared__ float ks[kTok][D];
-    __shared__ float ws[kTok][D];
-    __shared__ float lc[kTok], cc[kTok];
+template <int D, int MODE>
+__global__ void __launch_bounds__(128, D == 16 ? 4 : 2) route_pass_kernel(
+    const float* __restrict__ a, int a_per_head, const float* __restrict__ kb,
+    const float* __restrict__ wb, const float* __restrict__ g, const float* __restrict__ Lrow,
+    const float* __restrict__ crow, const float* __restrict__ Lcol,
+    const float* __restrict__ ccol, int64_t H, int64_t N, int64_t M, int64_t chunk_len,
+    int64_t nchunk, int64_t n_mtiles, float sl2, float* __restrict__ pa, float* __restrict__ pb) {
+    using namespace simt;
+    __shared__ __align__(16) float ks[2][kTok][D];
+    __shared__ __align__(16) float ws[2][kTok][D];
+    __shared__ float lc[2][kTok], cc[2][kTok];
+    tc::pdl_trigger();
+    tc::pdl_wait();
 
     int64_t bid = blockIdx.x;
     const int64_t c = bid % nchunk;
@@ -128,64 +124,55 @@ __global__ void __launch_bounds__(128) route_pass_kernel(
     const int64_t m = mt * blockDim.x + threadIdx.x;
     const bool active = m < M;
     const int64_t mm = active ? m : 0;
-
-    float ar[D], gr[D], accA[MODE == 3 ? D : 1], accB[D];
-    {
-        const AT* ap = a + ((a_per_head ? bh % H : bh) * M + mm) * D;
-        const float* gp = g + (bh * M + mm) * D;
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-            ar[d] = operand<T>(ld_f32(ap + d)) * sl2;
-            gr[d] = MODE == 3 ? operand<T>(gp[d]) : gp[d];
-            accB[d] = 0.f;
-            if (MODE == 3) accA[d] = 0.f;
+    const int64_t n_begin = c * chunk_len;
+    const int64_t n_end = min(N, n_begin + chunk_len);
+    auto stage = [&](int buf, int64_t n0) {
+        stage_rows<D, kTok>(ks[buf], kb + bh * N * D, n0, n_end);
+        stage_rows<D, kTok>(ws[buf], wb + bh * N * D, n0, n_end);
+        if (MODE == 3) {
+            stage_values<kTok>(lc[buf], Lcol + bh * N, n0, n_end);
+            stage_values<kTok>(cc[buf], ccol + bh * N, n0, n_end);
         }
+        copy_commit();
+    };
+    stage(0, n_begin);
+
+    f2 ar[D / 2], gr[D / 2], accA[MODE == 3 ? D / 2 : 1], accB[D / 2];
+    load_row<D>(ar, a + ((a_per_head ? bh % H : bh) * M + mm) * D, sl2, true);
+    load_row<D>(gr, g + (bh * M + mm) * D, 1.f, true);
+#pragma unroll
+    for (int d = 0; d < D / 2; ++d) {
+        accB[d] = 0;
+        if (MODE == 3) accA[d] = 0;
     }
     const float Lr = MODE == 3 ? 0.f : Lrow[bh * M + mm];
     const float cr = MODE == 3 ? 0.f : crow[bh * M + mm];
 
-    const int64_t n_begin = c * chunk_len;
-    const int64_t n_end = min(N, n_begin + chunk_len);
-    const T* kp = kb + bh * N * D;
-    const T* wp = wb + bh * N * D;
-    for (int64_t n0 = n_begin; n0 < n_end; n0 += kTok) {
+    int buf = 0;
+    for (int64_t n0 = n_begin; n0 < n_end; n0 += kTok, buf ^= 1) {
         const int cnt = (int)min((int64_t)kTok, n_end - n0);
+        const bool more = n0 + kTok < n_end;
+        if (more) stage(buf ^ 1, n0 + kTok);
+        if (more)
+            copy_wait<1>();
+        else
+            copy_wait<0>();
         __syncthreads();
-        for (int i = threadIdx.x; i < kTok * D; i += blockDim.x) {
-            const int j = i / D, d = i % D;
-            const bool in = j < cnt;
-            ks[j][d] = in ? ld_f32(kp + (n0 + j) * D + d) : 0.f;
-            ws[j][d] = in ? ld_f32(wp + (n0 + j) * D + d) : 0.f;
+#pragma unroll(D == 64 ? 1 : (MODE == 3 ? 2 : 8))
+        for (int j = 0; j < kTok; ++j) {
+            const float x = dot_row<D>(ar, ks[buf][j]);
+            const float dp = dot_row<D>(gr, ws[buf][j]);
+            const float p = j < cnt ? ex2(x - (MODE == 3 ? lc[buf][j] : Lr)) : 0.f;
+            const float ds = p * (dp - (MODE == 3 ? cc[buf][j] : cr));
+            axpy_row<D>(accB, ds, ks[buf][j]);
+            if (MODE == 3) axpy_row<D>(accA, p, ws[buf][j]);
         }
-        if (MODE == 3 && threadIdx.x < kTok) {
-            const int j = threadIdx.x;
-            lc[j] = j < cnt ? Lcol[bh * N + n0 + j] : 0.f;
-            cc[j] = j < cnt ? ccol[bh * N + n0 + j] : 0.f;
-        }
-        __syncthreads();
-        for (int j = 0; j < cnt; ++j) {
-            float x = 0.f, dp = 0.f;
-#pragma unroll
-            for (int d = 0; d < D; ++d) {
-                x = fmaf(ar[d], ks[j][d], x);
-                dp = fmaf(gr[d], ws[j][d], dp);
-            }
-            const float p = ex2(x - (MODE == 3 ? lc[j] : Lr));
-            const float ds = p * (dp - (MODE == 3 ? cc[j] : cr));
-#pragma unroll
-            for (int d = 0; d < D; ++d) {
-                accB[d] = fmaf(ds, ks[j][d], accB[d]);
-                if (MODE == 3) accA[d] = fmaf(p, ws[j][d], accA[d]);
-            }
-        }
+        __syncthreads();  // this buffer is staged into again in the next step
     }
     if (active) {
         const int64_t row = (bh * nchunk + c) * M + m;
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-            pb[row * D + d] = accB[d];
-            if (MODE == 3) pa[row * D + d] = accA[d];
-        }
+        store_row<D>(pb + row * D, accB, 1.f);
+        if (MODE == 3) store_row<D>(pa + row * D, accA, 1.f);
     }
 }
 
@@ -213,6 +200,7 @@ __global__ void bwd_reduce_kernel(const float* __restrict__ pa, const float* __r
     if (MODE == 1) {
         const int64_t h = row / M, m = row % M;
         for (int64_t b = 0; b < B; ++b)
+#pragma unroll 8
             for (int64_t c = 0; c < nchunk; ++c) {
                 const int64_t r = ((b * H + h) * nchunk + c) * M + m;
 #pragma unroll
@@ -229,6 +217,7 @@ __global__ void bwd_reduce_kernel(const float* __restrict__ pa, const float* __r
         return;
     }
     const int64_t bh = row / M, m = row % M;
+#pragma unroll 8
     for (int64_t c = 0; c < nchunk; ++c) {
         const int64_t r = (bh * nchunk + c) * M + m;
 #pragma unroll
@@ -268,7 +257,7 @@ __global__ void bwd_reduce_kernel(const float* __restrict__ pa, const float* __r
     if (lane == 0) cout[row] = dot;
 }
 
-// Token pass; thread = token n, every route streamed.
+// Token pass, float32; two threads per R tokens n, every route streamed.
 //   MODE 23 (calls 3 and 2 together): keys k = K_n, w = V_n, y = dY_n; routes a = Q, g = dZ,
 //     z = Z with L2, c2 per route and L3, c3 of the token:
 //     x = s' <k, q_m>; P2 = 2^(x - L2_m); P3 = 2^(x - L3_n);
@@ -276,84 +265,103 @@ __global__ void bwd_reduce_kernel(const float* __restrict__ pa, const float* __r
 //     dK = s sum_m dS q_m;  dV = sum_m P2 dz_m
 //   MODE 1: k = Kt_n, w = Vt_n; routes a = seeds (per head), g = dQ with L1, c1:
 //     P1 = 2^(x - L1_m); dS = P1 (<w, dq_m> - c1_m); dKt = s sum_m dS a_m; dVt = sum_m P1 dq_m
-// grid.x = ceil(N / 128) * BH; block = 128 threads.
-template <int D, typename T, typename AT, int MODE>
+// grid.x = ceil(N / 64 R) * BH; block = 128 threads, pair t with the tokens t, t + 64.
+template <int D, int MODE, int R>
 __global__ void __launch_bounds__(128) token_pass_kernel(
-    const T* __restrict__ kb, const T* __restrict__ wb, const T* __restrict__ yb,
-    const AT* __restrict__ a, int a_per_head, const float* __restrict__ g,
+    const float* __restrict__ kb, const float* __restrict__ wb, const float* __restrict__ yb,
+    const float* __restrict__ a, int a_per_head, const float* __restrict__ g,
     const float* __restrict__ z, const float* __restrict__ Lrow, const float* __restrict__ crow,
     const float* __restrict__ Lcol, const float* __restrict__ ccol, int64_t H, int64_t N,
-    int64_t M, float sl2, float scale, T* __restrict__ dk_out, T* __restrict__ dv_out) {
-    __shared__ float as_[kRoute][D];
-    __shared__ float gs[kRoute][D];
-    __shared__ float zs[MODE == 23 ? kRoute : 1][D];
-    __shared__ float ls[kRoute], cs[kRoute];
-    const int64_t ntiles = (N + 127) / 128;
+    int64_t M, float sl2, float scale, float* __restrict__ dk_out, float* __restrict__ dv_out) {
+    using namespace simt;
+    constexpr bool kThree = MODE == 23;
+    __shared__ __align__(16) float as_[2][kRoute][D];
+    __shared__ __align__(16) float gs[2][kRoute][D];
+    __shared__ __align__(16) float zs[2][kThree ? kRoute : 1][D];
+    __shared__ float ls[2][kRoute], cs[2][kRoute];
+    tc::pdl_trigger();
+    tc::pdl_wait();
+    const int64_t ntiles = (N + 64 * R - 1) / (64 * R);
     const int64_t bh = blockIdx.x / ntiles;
-    const int64_t n = (blockIdx.x % ntiles) * 128 + threadIdx.x;
-    const bool active = n < N;
-    const int64_t nn = active ? n : 0;
-    float kr[D], wr[D], yr[MODE == 23 ? D : 1], dk[D], dv[D];
+    const int h = threadIdx.x & 1;
+    const int64_t nbase = (blockIdx.x % ntiles) * 64 * R + threadIdx.x / 2;
+    const float* ab = a + (a_per_head ? bh % H : bh) * M * D;
+    auto stage = [&](int buf, int64_t m0) {
+        stage_rows<D, kRoute>(as_[buf], ab, m0, M);
+        stage_rows<D, kRoute>(gs[buf], g + bh * M * D, m0, M);
+        if constexpr (kThree) stage_rows<D, kRoute>(zs[buf], z + bh * M * D, m0, M);
+        stage_values<kRoute>(ls[buf], Lrow + bh * M, m0, M);
+        stage_values<kRoute>(cs[buf], crow + bh * M, m0, M);
+        copy_commit();
+    };
+    stage(0, 0);
+    f2 kr[R][D / 4], wr[R][D / 4], yr[R][kThree ? D / 4 : 1], dk[R][D / 4], dv[R][D / 4];
+    float L3[R], c3[R];
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-        kr[d] = ld_f32(kb + (bh * N + nn) * D + d) * sl2;
-        wr[d] = ld_f32(wb + (bh * N + nn) * D + d);
-        if (MODE == 23) yr[d] = ld_f32(yb + (bh * N + nn) * D + d);
-        dk[d] = dv[d] = 0.f;
+    for (int r = 0; r < R; ++r) {
+        const int64_t n = nbase + r * 64 < N ? nbase + r * 64 : 0;
+        load_half<D>(kr[r], kb + (bh * N + n) * D, sl2, h);
+        load_half<D>(wr[r], wb + (bh * N + n) * D, 1.f, h);
+        if constexpr (kThree) load_half<D>(yr[r], yb + (bh * N + n) * D, 1.f, h);
+#pragma unroll
+        for (int d = 0; d < D / 4; ++d) dk[r][d] = dv[r][d] = 0;
+        L3[r] = kThree ? Lcol[bh * N + n] : 0.f;
+        c3[r] = kThree ? ccol[bh * N + n] : 0.f;
     }
-    const float L3 = MODE == 23 ? Lcol[bh * N + nn] : 0.f;
-    const float c3 = MODE == 23 ? ccol[bh * N + nn] : 0.f;
-    const AT* ab = a + (a_per_head ? bh % H : bh) * M * D;
-    const float* gb = g + bh * M * D;
-    const float* zb = MODE == 23 ? z + bh * M * D : nullptr;
-    for (int64_t m0 = 0; m0 < M; m0 += kRoute) {
+    int buf = 0;
+    for (int64_t m0 = 0; m0 < M; m0 += kRoute, buf ^= 1) {
         const int cnt = (int)min((int64_t)kRoute, M - m0);
+        const bool more = m0 + kRoute < M;
+        if (more) stage(buf ^ 1, m0 + kRoute);
+        if (more)
+            copy_wait<1>();
+        else
+            copy_wait<0>();
         __syncthreads();
-        for (int i = threadIdx.x; i < kRoute * D; i += blockDim.x) {
-            const int j = i / D, d = i % D;
+#pragma unroll(D == 64 ? 1 : 8)
+        for (int j = 0; j < kRoute; ++j) {
             const bool in = j < cnt;
-            as_[j][d] = in ? operand<T>(ld_f32(ab + (m0 + j) * D + d)) : 0.f;
-            gs[j][d] = in ? gb[(m0 + j) * D + d] : 0.f;
-            if (MODE == 23) zs[j][d] = in ? operand<T>(zb[(m0 + j) * D + d]) : 0.f;
-        }
-        if (threadIdx.x < kRoute) {
-            const int j = threadIdx.x;
-            ls[j] = j < cnt ? Lrow[bh * M + m0 + j] : 0.f;
-            cs[j] = j < cnt ? crow[bh * M + m0 + j] : 0.f;
+            f2 aj[D / 4], gj[D / 4];
+            read_half<D>(aj, as_[buf][j], h);
+            read_half<D>(gj, gs[buf][j], h);
+            float x[R], p[R], ds[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                x[r] = dot_half<D>(kr[r], aj);
+                const float dp = dot_half<D>(wr[r], gj);
+                p[r] = in ? ex2(x[r] - ls[buf][j]) : 0.f;
+                ds[r] = p[r] * (dp - cs[buf][j]);
+                axpy_half<D>(dv[r], p[r], gj);
+            }
+            if constexpr (kThree) {
+                f2 zj[D / 4];
+                read_half<D>(zj, zs[buf][j], h);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const float dp3 = dot_half<D>(yr[r], zj);
+                    ds[r] = fmaf(in ? ex2(x[r] - L3[r]) : 0.f, dp3 - c3[r], ds[r]);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) axpy_half<D>(dk[r], ds[r], aj);
         }
         __syncthreads();
-        for (int j = 0; j < cnt; ++j) {
-            float x = 0.f, dp = 0.f, dp3 = 0.f;
-#pragma unroll
-            for (int d = 0; d < D; ++d) {
-                x = fmaf(kr[d], as_[j][d], x);
-                dp = fmaf(wr[d], gs[j][d], dp);
-                if (MODE == 23) dp3 = fmaf(yr[d], zs[j][d], dp3);
-            }
-            const float p = ex2(x - ls[j]);
-            float ds = p * (dp - cs[j]);
-            if (MODE == 23) ds = fmaf(ex2(x - L3), dp3 - c3, ds);
-#pragma unroll
-            for (int d = 0; d < D; ++d) {
-                dk[d] = fmaf(ds, as_[j][d], dk[d]);
-                dv[d] = fmaf(p, gs[j][d], dv[d]);
-            }
-        }
     }
-    if (active) {
 #pragma unroll
-        for (int d = 0; d < D; ++d) {
-            st_out(dk_out + (bh * N + n) * D + d, scale * dk[d]);
-            st_out(dv_out + (bh * N + n) * D + d, dv[d]);
+    for (int r = 0; r < R; ++r) {
+        const int64_t n = nbase + r * 64;
+        if (n < N) {
+            store_half<D>(dk_out + (bh * N + n) * D, dk[r], scale, h);
+            store_half<D>(dv_out + (bh * N + n) * D, dv[r], 1.f, h);
         }
     }
 }
 
-template <int D, typename T>
-cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const T* seeds, const T* Kt,
-                        const T* Vt, const T* K, const T* V, float scale, const T* Y,
-                        const T* dY, const char* saved, T* dseeds, T* dKt, T* dVt, T* dK,
-                        T* dV, char* ws, cudaStream_t st) {
+template <int D>
+cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, const float* Kt,
+                        const float* Vt, const float* K, const float* V, float scale, const float* Y,
+                        const float* dY, const char* saved, float* dseeds, float* dKt, float* dVt, float* dK,
+                        float* dV, char* ws, cudaStream_t st) {
     const SavedLayout sl = saved_layout(p);
     const float* Q32 = (const float*)(saved + sl.off_q);
     const float* Z32 = (const float*)(saved + sl.off_z);
@@ -371,37 +379,56 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const T* seeds, const 
     const int64_t tok_rows = p.BH * p.N;
     const int64_t lat_rows = p.BH * p.M;
     const unsigned route_blocks = (unsigned)(bp.nchunk * bp.n_mtiles * p.BH);
+    // two tokens per pair of threads where registers allow (8 x 16,384 tokens, M = 128, D = 32: 153 and
+    // 120 us; one token per pair 199 and 128, one per thread 210 and 130), once 128 tokens per block
+    // take both places that registers leave on every SM. One route per thread in the route passes: pairs
+    // with one or two routes are slower (132 or 140 us for call 3, 98 or 93 for calls 2 and 1; this
+    // 108 and 84).
+    constexpr int kTwo = D <= 32 ? 2 : 1;
+    const bool two_tokens = D <= 32 && ((p.N + 127) / 128) * p.BH >= 2 * kNumSMs;
     const int route_threads = (int)bp.m_tile;
-    const unsigned token_blocks = (unsigned)(((p.N + 127) / 128) * p.BH);
+    const unsigned token_blocks =
+        (unsigned)((two_tokens ? (p.N + 127) / 128 : (p.N + 63) / 64) * p.BH);
     const unsigned red_blocks = (unsigned)((lat_rows + 7) / 8);
 
-    launch_delta_tokens<D, T>(dY, Y, tok_rows, c3, st);
+    launch_delta_tokens<D, float>(dY, Y, tok_rows, c3, st);
+    const auto route = [&](auto kernel, const float* a, int per_head, const float* k,
+                           const float* w, const float* g, const float* Lr, const float* cr) {
+        return launch_pdl(kernel, dim3(route_blocks), dim3((unsigned)route_threads), 0, st, a,
+                          per_head, k, w, g, Lr, cr, (const float*)L3, (const float*)c3, p.H, p.N,
+                          p.M, bp.chunk_len, bp.nchunk, bp.n_mtiles, sl2, pa, pb);
+    };
+    const auto token = [&](auto kernel, const float* k, const float* w, const float* y,
+                           const float* a, int per_head, const float* g, const float* z,
+                           const float* Lr, const float* cr, float* o0, float* o1) {
+        return launch_pdl(kernel, dim3(token_blocks), dim3(128), 0, st, k, w, y, a, per_head, g, z,
+                          Lr, cr, (const float*)L3, (const float*)c3, p.H, p.N, p.M, sl2, scale, o0,
+                          o1);
+    };
+    const float* none = nullptr;
+    cudaError_t e;
     // call 3: dZ and the decoder's dQ
-    route_pass_kernel<D, T, float, 3><<<route_blocks, route_threads, 0, st>>>(
-        Q32, 0, K, dY, Z32, nullptr, nullptr, L3, c3, p.H, p.N, p.M, bp.chunk_len, bp.nchunk,
-        bp.n_mtiles, sl2, pa, pb);
-    bwd_reduce_kernel<D, T, 3><<<red_blocks, 256, 0, st>>>(pa, pb, lat_rows, p.B, p.H, p.M,
-                                                           bp.nchunk, scale, Z32, dz, dq, c2,
-                                                           nullptr, nullptr);
+    if ((e = route(route_pass_kernel<D, 3>, Q32, 0, K, dY, Z32, none, none)) != cudaSuccess)
+        return e;
+    bwd_reduce_kernel<D, float, 3><<<red_blocks, 256, 0, st>>>(pa, pb, lat_rows, p.B, p.H, p.M,
+                                                               bp.nchunk, scale, Z32, dz, dq, c2,
+                                                               nullptr, nullptr);
     // calls 3 and 2: dK and dV per token
-    token_pass_kernel<D, T, float, 23><<<token_blocks, 128, 0, st>>>(
-        K, V, dY, Q32, 0, dz, Z32, L2, c2, L3, c3, p.H, p.N, p.M, sl2, scale, dK, dV);
+    if ((e = token(two_tokens ? token_pass_kernel<D, 23, kTwo> : token_pass_kernel<D, 23, 1>, K, V,
+                   dY, Q32, 0, dz, Z32, L2, c2, dK, dV)) != cudaSuccess)
+        return e;
     // call 2: the encoder's dQ, added to the decoder's
-    route_pass_kernel<D, T, float, 2><<<route_blocks, route_threads, 0, st>>>(
-        Q32, 0, K, V, dz, L2, c2, nullptr, nullptr, p.H, p.N, p.M, bp.chunk_len, bp.nchunk,
-        bp.n_mtiles, sl2, nullptr, pb);
-    bwd_reduce_kernel<D, T, 2><<<red_blocks, 256, 0, st>>>(nullptr, pb, lat_rows, p.B, p.H, p.M,
-                                                           bp.nchunk, scale, Q32, nullptr, dq, c1,
-                                                           nullptr, nullptr);
+    if ((e = route(route_pass_kernel<D, 2>, Q32, 0, K, V, dz, L2, c2)) != cudaSuccess) return e;
+    bwd_reduce_kernel<D, float, 2><<<red_blocks, 256, 0, st>>>(nullptr, pb, lat_rows, p.B, p.H, p.M,
+                                                               bp.nchunk, scale, Q32, nullptr, dq,
+                                                               c1, nullptr, nullptr);
     // call 1: dKt, dVt per token, then the seeds' gradient
-    token_pass_kernel<D, T, T, 1><<<token_blocks, 128, 0, st>>>(
-        Kt, Vt, nullptr, seeds, 1, dq, nullptr, L1, c1, nullptr, nullptr, p.H, p.N, p.M, sl2,
-        scale, dKt, dVt);
-    route_pass_kernel<D, T, T, 1><<<route_blocks, route_threads, 0, st>>>(
-        seeds, 1, Kt, Vt, dq, L1, c1, nullptr, nullptr, p.H, p.N, p.M, bp.chunk_len, bp.nchunk,
-        bp.n_mtiles, sl2, nullptr, pb);
+    if ((e = token(two_tokens ? token_pass_kernel<D, 1, kTwo> : token_pass_kernel<D, 1, 1>, Kt, Vt,
+                   none, seeds, 1, dq, none, L1, c1, dKt, dVt)) != cudaSuccess)
+        return e;
+    if ((e = route(route_pass_kernel<D, 1>, seeds, 1, Kt, Vt, dq, L1, c1)) != cudaSuccess) return e;
     const int64_t seed_rows = p.H * p.M;
-    bwd_reduce_kernel<D, T, 1><<<(unsigned)((seed_rows + 7) / 8), 256, 0, st>>>(
+    bwd_reduce_kernel<D, float, 1><<<(unsigned)((seed_rows + 7) / 8), 256, 0, st>>>(
         nullptr, pb, seed_rows, p.B, p.H, p.M, bp.nchunk, scale, nullptr, nullptr, nullptr,
         nullptr, dseeds, nullptr);
     return cudaGetLastError();
@@ -767,15 +794,15 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t route_bwd_t(const Plan& p, const BwdPlan& bp, const void* seeds, const void* Kt,
-                        const void* Vt, const void* K, const void* V, float scale, const void* Y,
-                        const void* dY, const char* saved, void* dseeds, void* dKt, void* dVt,
-                        void* dK, void* dV, char* ws, cudaStream_t st) {
-#define FLAREPP_BWD(DD)                                                                          \
-    return route_bwd_d<DD, T>(p, bp, (const T*)seeds, (const T*)Kt, (const T*)Vt, (const T*)K,  \
-                              (const T*)V, scale, (const T*)Y, (const T*)dY, saved, (T*)dseeds, \
-                              (T*)dKt, (T*)dVt, (T*)dK, (T*)dV, ws, st);
+cudaError_t route_bwd_f32(const Plan& p, const BwdPlan& bp, const void* seeds, const void* Kt,
+                          const void* Vt, const void* K, const void* V, float scale, const void* Y,
+                          const void* dY, const char* saved, void* dseeds, void* dKt, void* dVt,
+                          void* dK, void* dV, char* ws, cudaStream_t st) {
+    const auto f = [](const void* x) { return (const float*)x; };
+    const auto o = [](void* x) { return (float*)x; };
+#define FLAREPP_BWD(DD)                                                                     \
+    return route_bwd_d<DD>(p, bp, f(seeds), f(Kt), f(Vt), f(K), f(V), scale, f(Y), f(dY), saved, \
+                           o(dseeds), o(dKt), o(dVt), o(dK), o(dV), ws, st);
     switch (p.D) {
         case 16: FLAREPP_BWD(16)
         case 32: FLAREPP_BWD(32)
@@ -803,8 +830,8 @@ cudaError_t route_bwd(const Plan& p, const BwdPlan& bp, const void* seeds, const
         }
 #undef FLAREPP_TCBWD
     }
-    return route_bwd_t<float>(p, bp, seeds, Kt, Vt, K, V, scale, Y, dY, saved, dseeds, dKt, dVt,
-                              dK, dV, ws, st);
+    return route_bwd_f32(p, bp, seeds, Kt, Vt, K, V, scale, Y, dY, saved, dseeds, dKt, dVt, dK, dV,
+                         ws, st);
 }
 
 }  // namespace flarepp

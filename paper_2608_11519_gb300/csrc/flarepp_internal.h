@@ -107,6 +107,8 @@ struct BwdPlan {
 constexpr int kRangeParts = 128;  // token slices of the merged pass's range reduction
 BwdPlan make_bwd_plan(const Plan& p);
 
+// Routes per thread of the CUDA-core encode: two when a full tile of 128 routes leaves two warps.
+constexpr int simt_encode_rows(int64_t M, int64_t D) { return M >= 128 && D <= 32 ? 2 : 1; }
 // ---- CUDA-core kernels (simt_kernels.cuh, instantiated in simt_f32.cu), float32 inputs
 // Encode one call over all chunks: call 1 takes the seeds ([H][M][D]), call 2 takes Q32
 // from the workspace. Writes the chunk partials.

@@ -44,15 +44,17 @@ flarepp_status make_plan(const flarepp_shape* s, Plan* p) {
     if (bh == 0 || s->N == 0 || s->M == 0) return FLAREPP_OK;  // nothing to plan
 
     if (p->path == kPathSimt) {
-        // CUDA-core encode: one thread per route, up to 128 routes per CTA; chunks sized so
-        // that the grid holds about four waves of CTAs per SM.
+        // CUDA-core encode: up to 128 routes per CTA, one or two per thread; chunks sized so that
+        // the grid is one wave of the CTAs that registers allow per SM (four of 128 threads, six
+        // of 64 with two routes each; two at D = 64).
         p->m_tile = s->M >= 128 ? 128 : cdiv(s->M, 32) * 32;
         p->n_mtiles = cdiv(s->M, p->m_tile);
         p->sub_per_chunk = 1;
-        const int64_t target = 4 * kNumSMs;
-        int64_t want = cdiv(target, bh * p->n_mtiles);
+        const int64_t target =
+            (simt_encode_rows(s->M, s->D) == 2 ? 6 : (s->D <= 32 ? 4 : 2)) * kNumSMs;
+        int64_t want = target / (bh * p->n_mtiles);
         if (want < 1) want = 1;
-        p->chunk_len = cdiv(cdiv(s->N, want), 32) * 32;
+        p->chunk_len = cdiv(cdiv(s->N, want), 16) * 16;
         p->nchunk = cdiv(s->N, p->chunk_len);
     } else {
         // Tensor-core encode: a work unit is (bh, group of <= 512 routes, chunk of tokens) and
@@ -169,10 +171,11 @@ BwdPlan make_bwd_plan(const Plan& p) {
         if (want < 1) want = 1;
         b.chunk_len = cdiv(cdiv(p.N, want), item) * item;
     } else {
-        // one thread per route, up to 128 routes per CTA; chunks for about four waves
-        int64_t want = cdiv(4 * kNumSMs, p.BH * b.n_mtiles);
+        // one thread per route, up to 128 routes per CTA; chunks for one wave of the CTAs that
+        // registers allow per SM (four, two at D >= 32)
+        int64_t want = (p.D == 16 ? 4 : 2) * kNumSMs / (p.BH * b.n_mtiles);
         if (want < 1) want = 1;
-        b.chunk_len = cdiv(cdiv(p.N, want), 32) * 32;
+        b.chunk_len = cdiv(cdiv(p.N, want), 16) * 16;
     }
     b.nchunk = cdiv(p.N, b.chunk_len);
     const size_t part = (size_t)p.BH * (size_t)b.nchunk * (size_t)p.M * (size_t)p.D * 4;
