@@ -13,15 +13,16 @@
 //
 // The contraction over C runs in slices of D channels (one head), the unit that both A
 // layouts share; each slice is one TMA box of 128 tokens x D for A and NT channels x D for B,
-// swizzled to the D-wide row. A work tile is 128 tokens (of one batch element) x NT output
-// channels; persistent CTAs walk the tiles with the channel tile varying fastest, so the CTAs
+// swizzled to the D-wide row. A work tile is 128 tokens (of one batch element), or 256 as two row
+// tiles that share B's slices (MODE 1), x NT output channels; persistent CTAs walk the tiles with the channel tile varying fastest, so the CTAs
 // that share a token tile run together and read it from L2.
 //
 // Roles (12 warps): warp 0 the TMA producer, warp 1 the MMA issuer (one elected lane; one
 // commit per slice frees its ring stage, one per tile hands the accumulator over), warps 4..11
 // two epilogue warpgroups (TMEM lane = token row; each takes every other head of the tile and
-// writes it with one TMA store per head from a shared-memory staging block). Two TMEM accumulators of NT <= 256 columns let the
-// epilogue of one tile overlap the products of the next. Every wait is bounded (2 s of
+// writes it with one TMA store per head from a shared-memory staging block). Two TMEM accumulators
+// of NT <= 256 columns take the row tiles in turn, so the epilogue of one overlaps the products of
+// the next. Every wait is bounded (2 s of
 // %globaltimer): on expiry the kernel records FLAREPP_ERR_TIMEOUT in the status word, every
 // role leaves its loops, the producer waits for its copies in flight, the MMA issuer for its
 // products, and TMEM is freed.
@@ -47,16 +48,18 @@ constexpr int kMaxNT = 256;   // output channels per tile, at most
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 constexpr uint32_t kTmemCols = 512;
 
-template <int D>
+template <int D, int MODE>
 struct GCfg {
     static constexpr int kASlice = kRows * D * 2;
     static constexpr int kBSlice = kMaxNT * D * 2;
-    static constexpr int kStage = kASlice + kBSlice;
+    static constexpr int kHalves = MODE == 1 ? 2 : 1;  // row tiles per work tile, at most
+    static constexpr int kStage = kHalves * kASlice + kBSlice;
     static constexpr int kStages = (160 * 1024) / kStage > 8 ? 8 : (160 * 1024) / kStage;
     static constexpr uint32_t kSwz = D == 16 ? kSw32 : (D == 32 ? kSw64 : kSw128);
     static constexpr uint32_t kSBO = 8 * D * 2;
-    // per epilogue warpgroup: its heads of one tile, [head][128 rows][D] bf16, for TMA stores
-    static constexpr int kStaging = (kMaxNT / 2) * kRows * 2;
+    // per epilogue warpgroup: [128 rows][D] bf16 blocks for TMA stores, as many as its heads of a tile
+    static constexpr int kSlots = kMaxNT / 2 / D;
+    static constexpr int kStaging = kSlots * kRows * D * 2;
     // full, empty, accfull[2], accempty[2], fin, then per epilogue warpgroup staging_free and
     // staging_written
     static constexpr int kNumBars = 2 * kStages + 4 + 1 + 2 * kEpiGroups;
@@ -73,22 +76,26 @@ struct GemmParams {
     int NT;             // output channels per tile (whole heads, <= 256, divides C)
     uint32_t idesc;     // MMA instruction descriptor for M = 128, N = NT
     int64_t row_tiles;  // 128-token tiles per batch element
+    int64_t pair;       // row tiles per work tile (1 or 2)
+    int64_t groups;     // work tiles down a batch element: ceil(row_tiles / pair)
     int64_t col_tiles;  // n_out / NT
-    int64_t n_tiles;
+    int64_t n_tiles;    // B * groups * col_tiles
     __nv_bfloat16* out[4];  // MODE 0: the P [B][H][N][D] tensors; MODE 1: O [B][N][C]
     int* status;
 };
 
 struct GTile {
     int64_t b, rt, ct;
+    int halves;  // row tiles rt, rt + 1, ... of this work tile
 };
 
 __device__ __forceinline__ GTile gtile(const GemmParams& p, int64_t t) {
     GTile T;
     T.ct = t % p.col_tiles;
     const int64_t r = t / p.col_tiles;
-    T.rt = r % p.row_tiles;
-    T.b = r / p.row_tiles;
+    T.rt = (r % p.groups) * p.pair;
+    T.b = r / p.groups;
+    T.halves = (int)min(p.pair, p.row_tiles - T.rt);
     return T;
 }
 
@@ -127,7 +134,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                    const __grid_constant__ CUtensorMap tmO0, const __grid_constant__ CUtensorMap tmO1,
                    const __grid_constant__ CUtensorMap tmO2, const __grid_constant__ CUtensorMap tmO3,
                    const GemmParams prm) {
-    using C = GCfg<D>;
+    using C = GCfg<D, MODE>;
     constexpr int kS = C::kStages;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align_shared<1024>(smem_raw);
@@ -183,7 +190,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // ------------------------------------------------------------ TMA producer
         uint32_t it = 0;
         bool ok = true;
-        const uint32_t bytes = (uint32_t)(C::kASlice + prm.NT * D * 2);
+        const uint32_t b_bytes = (uint32_t)(prm.NT * D * 2);
         for (int64_t t = blockIdx.x; t < prm.n_tiles && ok; t += gridDim.x) {
             const GTile T = gtile(prm, t);
             for (int h = 0; h < slices; ++h, ++it) {
@@ -195,18 +202,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 if (elect_one()) {
                     const uint32_t dst = smem_u32(smem + st * C::kStage);
-                    mbar_expect_tx(full0 + 8u * st, bytes);
-                    if (MODE == 0) {
-                        tma_load_3d(dst, &tmA, h * D, (int)(T.rt * kRows), (int)T.b,
-                                    full0 + 8u * st);
-                    } else {
-                        // slice h: head h % H of A tensor h / H
-                        const int p = h / (int)prm.H, hh = h % (int)prm.H;
-                        const CUtensorMap* ma = p == 0 ? &tmA : p == 1 ? &tmA1 : p == 2 ? &tmA2 : &tmA3;
-                        tma_load_3d(dst, ma, 0, (int)(T.rt * kRows), (int)(T.b * prm.H + hh),
-                                    full0 + 8u * st);
-                    }
-                    tma_load_3d(dst + C::kASlice, &tmB, h * D, (int)(T.ct * prm.NT), 0,
+                    mbar_expect_tx(full0 + 8u * st, (uint32_t)(T.halves * C::kASlice) + b_bytes);
+                    // MODE 1: slice h is head h % H of A tensor h / H
+                    const int p = MODE == 0 ? 0 : h / (int)prm.H;
+                    const int z = MODE == 0 ? (int)T.b : (int)(T.b * prm.H + h % (int)prm.H);
+                    const CUtensorMap* ma = p == 0 ? &tmA : p == 1 ? &tmA1 : p == 2 ? &tmA2 : &tmA3;
+                    for (int x = 0; x < (MODE == 0 ? 1 : T.halves); ++x)
+                        tma_load_3d(dst + x * C::kASlice, ma, MODE == 0 ? h * D : 0,
+                                    (int)((T.rt + x) * kRows), z, full0 + 8u * st);
+                    tma_load_3d(dst + C::kHalves * C::kASlice, &tmB, h * D, (int)(T.ct * prm.NT), 0,
                                 full0 + 8u * st);
                 }
                 __syncwarp();
@@ -223,39 +227,42 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        uint32_t it = 0, j = 0;
+        // row tile number seq of this CTA is summed in accumulator seq & 1
+        uint32_t it = 0, seq = 0;
         bool ok = true;
-        for (int64_t t = blockIdx.x; t < prm.n_tiles && ok; t += gridDim.x, ++j) {
-            const int ab = j & 1;
-            if (j >= 2 &&
-                !warp_wait(accempty0 + 8u * ab, ((j >> 1) - 1) & 1, abort_flag, prm.status)) {
-                ok = false;
-                break;
-            }
-            tc_fence_after();
-            const uint32_t acc = tmem + ab * kMaxNT;
-            for (int h = 0; h < slices; ++h, ++it) {
+        for (int64_t t = blockIdx.x; t < prm.n_tiles && ok; t += gridDim.x) {
+            const int halves = MODE == 0 ? 1 : gtile(prm, t).halves;
+            for (int h = 0; h < slices && ok; ++h, ++it) {
                 const int st = it % kS;
                 if (!warp_wait(full0 + 8u * st, (it / kS) & 1, abort_flag, prm.status)) {
                     ok = false;
                     break;
                 }
+                for (int x = 0; x < halves && h == 0 && ok; ++x)  // the accumulators are read out
+                    ok = seq + x < 2 ||
+                         warp_wait(accempty0 + 8u * ((seq + x) & 1), (((seq + x) >> 1) - 1) & 1,
+                                   abort_flag, prm.status);
+                if (!ok) break;
                 tc_fence_after();
-                const uint32_t a = smem_u32(smem + st * C::kStage);
-                const uint32_t b = a + C::kASlice;
+                const uint32_t a0 = smem_u32(smem + st * C::kStage);
+                if (elect_one()) {
+                    const uint64_t bd =
+                        smem_desc(a0 + C::kHalves * C::kASlice, 16, C::kSBO, C::kSwz);
 #pragma unroll
-                for (int k = 0; k < D / 16; ++k) {
-                    const uint64_t ad = smem_desc(a + 32 * k, 16, C::kSBO, C::kSwz);
-                    const uint64_t bd = smem_desc(b + 32 * k, 16, C::kSBO, C::kSwz);
-                    if (elect_one()) mma_ss(acc, ad, bd, prm.idesc, (h > 0 || k > 0) ? 1u : 0u);
-                    __syncwarp();
+                    for (int x = 0; x < C::kHalves; ++x) {
+                        if (x >= halves) break;
+                        const uint32_t acc = tmem + ((seq + x) & 1) * kMaxNT;
+                        const uint64_t ad = smem_desc(a0 + x * C::kASlice, 16, C::kSBO, C::kSwz);
+#pragma unroll
+                        for (int k = 0; k < D / 16; ++k)  // 32 bytes on: 2 in the descriptors' units
+                            mma_ss(acc, ad + 2 * k, bd + 2 * k, prm.idesc, (h > 0 || k > 0) ? 1u : 0u);
+                        if (h == slices - 1) mma_commit(accfull0 + 8u * ((seq + x) & 1));
+                    }
+                    mma_commit(empty0 + 8u * st);  // the slice's stage is free
                 }
-                if (elect_one()) mma_commit(empty0 + 8u * st);  // the slice's stage is free
                 __syncwarp();
             }
-            if (!ok) break;
-            if (elect_one()) mma_commit(accfull0 + 8u * ab);
-            __syncwarp();
+            seq += halves;
         }
         if (elect_one()) mma_commit(fin);
         __syncwarp();
@@ -266,12 +273,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else if (warp >= kFirstEpiWarp) {
         // ------------------------------------------------------------ epilogue
         // Warpgroup e takes the tile's heads e, e + 2, ...: each head's 128 x D block goes from
-        // TMEM through shared memory ([128 rows][D], one row per thread) to one TMA tensor
-        // store (rows beyond N are clipped by the store). Two mbarriers per warpgroup order the
-        // staging buffer (bounded waits): staging_free, which the leader arrives on once its
-        // previous stores have read the buffer, and staging_written, on which every thread
-        // arrives after its rows (and a proxy fence) and which the leader waits for before it
-        // issues the stores.
+        // TMEM through a slot of shared memory ([128 rows][D], one row per thread) to a TMA tensor
+        // store of its own (rows beyond N are clipped by the store). The slots are a ring, so
+        // blocks are written while the stores of the ones before them drain. Two mbarriers per
+        // warpgroup order a block (bounded waits): staging_free, which the leader arrives on once
+        // the store that last read the slot has done so, and staging_written, on which every thread
+        // arrives after its row (and a proxy fence) and which the leader waits for before it issues
+        // the store.
         const int q = warp % 4;
         const int e = (warp - kFirstEpiWarp) / 4;
         const int r = 32 * q + lane;
@@ -279,65 +287,74 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t lane_off = (uint32_t)(32 * q) << 16;
         const int heads = prm.NT / D;
         uint8_t* stg = staging + e * C::kStaging;
-        uint32_t j = 0;
-        bool pending = false;
-        for (int64_t t = blockIdx.x; t < prm.n_tiles; t += gridDim.x, ++j) {
+        uint32_t j = 0, u = 0;  // row tiles and blocks so far
+        bool ok = true;
+        for (int64_t t = blockIdx.x; t < prm.n_tiles && ok; t += gridDim.x) {
             const GTile T = gtile(prm, t);
-            const int ab = j & 1;
-            if (!warp_wait(accfull0 + 8u * ab, (j >> 1) & 1, abort_flag, prm.status)) break;
-            tc_fence_after();
-            if (pending) {
-                if (leader) {
-                    bulk_wait_read();
-                    mbar_arrive(sfree0 + 8u * e);
+            for (int x = 0; x < (MODE == 0 ? 1 : T.halves) && ok; ++x, ++j) {
+                const int ab = j & 1;
+                if (!warp_wait(accfull0 + 8u * ab, (j >> 1) & 1, abort_flag, prm.status)) {
+                    ok = false;
+                    break;
                 }
-                if (!warp_wait(sfree0 + 8u * e, (j - 1) & 1, abort_flag, prm.status)) break;
-            }
-            const uint32_t acc = tmem + lane_off + ab * kMaxNT;
-            int slot = 0;
-            for (int hh = e; hh < heads; hh += kEpiGroups, ++slot) {
-                uint32_t v[D];
+                tc_fence_after();
+                const uint32_t acc = tmem + lane_off + ab * kMaxNT;
+                if (e >= heads) mbar_arrive(accempty0 + 8u * ab);
+                for (int hh = e; hh < heads; hh += kEpiGroups) {
+                    uint32_t v[D];
 #pragma unroll
-                for (int k = 0; k < D / 16; ++k) tmem_ld16(acc + hh * D + 16 * k, v + 16 * k);
+                    for (int k = 0; k < D / 16; ++k) tmem_ld16(acc + hh * D + 16 * k, v + 16 * k);
 #pragma unroll
-                for (int k = 0; k < D / 16; ++k) tmem_wait_ld16(v + 16 * k);
-                // the block is stored swizzled like the operands (16-byte chunk g of row r at
-                // g ^ (bits 7.. of the row's byte offset)), which the store map undoes: one
-                // thread per row then writes without shared-memory bank conflicts
-                uint4* dst = reinterpret_cast<uint4*>(stg + ((size_t)slot * kRows + r) * D * 2);
-                const int sw = ((r * D * 2) >> 7) & (D / 8 - 1);
+                    for (int k = 0; k < D / 16; ++k) tmem_wait_ld16(v + 16 * k);
+                    if (hh + kEpiGroups >= heads) {
+                        tc_fence_before();
+                        mbar_arrive(accempty0 + 8u * ab);  // the accumulator is read out
+                    }
+                    if (leader) {
+                        bulk_wait_read<C::kSlots - 1>();
+                        mbar_arrive(sfree0 + 8u * e);
+                    }
+                    if (!warp_wait(sfree0 + 8u * e, u & 1, abort_flag, prm.status)) {
+                        ok = false;
+                        break;
+                    }
+                    // the block is stored swizzled like the operands (16-byte chunk g of row r at
+                    // g ^ (bits 7.. of the row's byte offset)), which the store map undoes: one
+                    // thread per row then writes without shared-memory bank conflicts
+                    uint8_t* block = stg + (u % C::kSlots) * (uint32_t)(kRows * D * 2);
+                    uint4* dst = reinterpret_cast<uint4*>(block + r * D * 2);
+                    const int sw = ((r * D * 2) >> 7) & (D / 8 - 1);
 #pragma unroll
-                for (int g = 0; g < D / 8; ++g) {
-                    uint4 o;
-                    o.x = pack_bf16(__uint_as_float(v[8 * g + 0]), __uint_as_float(v[8 * g + 1]));
-                    o.y = pack_bf16(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3]));
-                    o.z = pack_bf16(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5]));
-                    o.w = pack_bf16(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7]));
-                    dst[g ^ sw] = o;
-                }
-            }
-            tc_fence_before();
-            mbar_arrive(accempty0 + 8u * ab);  // the accumulator is read out
-            fence_proxy_async();
-            mbar_arrive(swritten0 + 8u * e);
-            if (q == 0 && !warp_wait(swritten0 + 8u * e, j & 1, abort_flag, prm.status)) break;
-            if (leader) {
-                slot = 0;
-                const int n0 = (int)(T.rt * kRows);
-                for (int hh = e; hh < heads; hh += kEpiGroups, ++slot) {
-                    const int64_t c = T.ct * prm.NT + (int64_t)hh * D;  // first channel
-                    const uint32_t src = smem_u32(stg + (size_t)slot * kRows * D * 2);
-                    if (MODE == 0) {
-                        const int64_t p = c / prm.C, h = (c % prm.C) / D;
-                        const CUtensorMap* m = p == 0 ? &tmO0 : p == 1 ? &tmO1 : p == 2 ? &tmO2 : &tmO3;
-                        tma_store_3d(m, src, 0, n0, (int)(T.b * prm.H + h));
-                    } else {
-                        tma_store_3d(&tmO0, src, (int)c, n0, (int)T.b);
+                    for (int g = 0; g < D / 8; ++g) {
+                        uint4 o;
+                        o.x = pack_bf16(__uint_as_float(v[8 * g + 0]), __uint_as_float(v[8 * g + 1]));
+                        o.y = pack_bf16(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3]));
+                        o.z = pack_bf16(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5]));
+                        o.w = pack_bf16(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7]));
+                        dst[g ^ sw] = o;
+                    }
+                    fence_proxy_async();
+                    mbar_arrive(swritten0 + 8u * e);
+                    if (q == 0 && !warp_wait(swritten0 + 8u * e, u & 1, abort_flag, prm.status)) {
+                        ok = false;
+                        break;
+                    }
+                    ++u;
+                    if (leader) {
+                        const int n0 = (int)((T.rt + x) * kRows);
+                        const int c = (int)(T.ct * prm.NT) + hh * D;  // first channel
+                        if (MODE == 0) {
+                            const int cc = (int)prm.C, p = c / cc, h = c % cc / D;
+                            const CUtensorMap* m =
+                                p == 0 ? &tmO0 : p == 1 ? &tmO1 : p == 2 ? &tmO2 : &tmO3;
+                            tma_store_3d(m, smem_u32(block), 0, n0, (int)(T.b * prm.H + h));
+                        } else {
+                            tma_store_3d(&tmO0, smem_u32(block), c, n0, (int)T.b);
+                        }
+                        bulk_commit();
                     }
                 }
-                bulk_commit();
             }
-            pending = true;
         }
         if (leader) bulk_wait_all();
     }
@@ -383,21 +400,41 @@ bool make_map(CUtensorMap* m, const void* base, int64_t D, int64_t inner, int64_
 
 template <int D, int MODE>
 cudaError_t launch(const CUtensorMap* a, const CUtensorMap& b, const CUtensorMap* o,
-                   const GemmParams& prm, cudaStream_t st) {
-    using Cf = GCfg<D>;
+                   const GemmParams& prm, int64_t sms, cudaStream_t st) {
+    using Cf = GCfg<D, MODE>;
     const cudaError_t attr = ensure_smem_limit((const void*)tc_gemm_kernel<D, MODE>, Cf::kSmem);
     if (attr != cudaSuccess) return attr;
-    if (prm.n_tiles == 0) return cudaSuccess;
-    int dev = 0, sms = kNumSMs;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t grid = prm.n_tiles < sms ? prm.n_tiles : sms;
     tc_gemm_kernel<D, MODE><<<(unsigned)grid, kThreads, Cf::kSmem, st>>>(
         a[0], a[1], a[2], a[3], b, o[0], o[1], o[2], o[3], prm);
     return cudaGetLastError();
 }
 
-// output channels per tile: D times the largest power of two of heads that divides H and
+template <int MODE>
+cudaError_t run(int64_t D, const CUtensorMap* a, const CUtensorMap& b, const CUtensorMap* o,
+                GemmParams& prm, cudaStream_t st) {
+    int dev = 0, sms = kNumSMs;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    prm.row_tiles = (prm.N + kRows - 1) / kRows;
+    prm.col_tiles = prm.n_out / prm.NT;
+    // MODE 1 is bound by its reads, most of them slices of B: two row tiles share each slice, once
+    // that leaves every SM a work tile (262,144 tokens, C = 256: dX 157 -> 113 us, the output 57 -> 46;
+    // the bytes of HBM alone take 99 and 40). MODE 0 is bound by its writes (537 MB there: 155 us; a
+    // fill of as many bytes takes 136) and slower with two row tiles (172).
+    prm.pair = MODE == 1 && prm.B * prm.row_tiles * prm.col_tiles >= 2 * sms ? 2 : 1;
+    prm.groups = (prm.row_tiles + prm.pair - 1) / prm.pair;
+    prm.n_tiles = prm.B * prm.groups * prm.col_tiles;
+    if (prm.n_tiles == 0) return cudaSuccess;
+    switch (D) {
+        case 16: return launch<16, MODE>(a, b, o, prm, sms, st);
+        case 32: return launch<32, MODE>(a, b, o, prm, sms, st);
+        case 64: return launch<64, MODE>(a, b, o, prm, sms, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+// output channels per tile: D times the largest power of two of heads that divides the H given and
 // keeps the tile within 256 channels
 int tile_channels(int64_t H, int64_t D) {
     int heads = 1;
@@ -434,11 +471,8 @@ cudaError_t tc_projection(int64_t B, int64_t N, int64_t H, int64_t D, int P, con
     prm.H = H;
     prm.C = C;
     prm.n_out = P * C;
-    prm.NT = tile_channels(H, D);
+    prm.NT = tile_channels(P * H, D);  // a tile may span projections
     prm.idesc = idesc_bf16_f32(kRows, prm.NT, false, false);
-    prm.row_tiles = (N + kRows - 1) / kRows;
-    prm.col_tiles = prm.n_out / prm.NT;
-    prm.n_tiles = B * prm.row_tiles * prm.col_tiles;
     for (int p = 0; p < 4; ++p) prm.out[p] = (__nv_bfloat16*)outs[p < P ? p : p - 2];
     prm.status = status;
     CUtensorMap ma[4], mb, mo[4];
@@ -450,12 +484,7 @@ cudaError_t tc_projection(int64_t B, int64_t N, int64_t H, int64_t D, int P, con
     for (int p = 0; p < 4; ++p)
         if (!make_store_map(&mo[p], prm.out[p], D, N, B * H, (uint32_t)D))
             return cudaErrorInvalidValue;
-    switch (D) {
-        case 16: return launch<16, 0>(ma, mb, mo, prm, st);
-        case 32: return launch<32, 0>(ma, mb, mo, prm, st);
-        case 64: return launch<64, 0>(ma, mb, mo, prm, st);
-        default: return cudaErrorInvalidValue;
-    }
+    return run<0>(D, ma, mb, mo, prm, st);
 }
 
 cudaError_t tc_output_projection(int64_t B, int64_t N, int64_t H, int64_t D, const void* Y,
@@ -478,9 +507,6 @@ cudaError_t tc_heads_projection(int64_t B, int64_t N, int64_t H, int64_t D, int 
     prm.n_out = C;
     prm.NT = tile_channels(H, D);
     prm.idesc = idesc_bf16_f32(kRows, prm.NT, false, false);
-    prm.row_tiles = (N + kRows - 1) / kRows;
-    prm.col_tiles = C / prm.NT;
-    prm.n_tiles = B * prm.row_tiles * prm.col_tiles;
     prm.out[0] = prm.out[1] = prm.out[2] = prm.out[3] = (__nv_bfloat16*)O;
     prm.status = status;
     CUtensorMap ma[4], mb, mo[4];
@@ -491,12 +517,7 @@ cudaError_t tc_heads_projection(int64_t B, int64_t N, int64_t H, int64_t D, int 
         !make_store_map(&mo[0], O, C, N, B, (uint32_t)D))
         return cudaErrorInvalidValue;
     mo[1] = mo[2] = mo[3] = mo[0];
-    switch (D) {
-        case 16: return launch<16, 1>(ma, mb, mo, prm, st);
-        case 32: return launch<32, 1>(ma, mb, mo, prm, st);
-        case 64: return launch<64, 1>(ma, mb, mo, prm, st);
-        default: return cudaErrorInvalidValue;
-    }
+    return run<1>(D, ma, mb, mo, prm, st);
 }
 
 }  // namespace flarepp

@@ -129,8 +129,9 @@ __device__ __forceinline__ void bulk_commit() {
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 // the shared-memory sources of this thread's committed bulk stores may be reused
+template <int N>
 __device__ __forceinline__ void bulk_wait_read() {
-    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
 // this thread's committed bulk stores are complete
 __device__ __forceinline__ void bulk_wait_all() {
