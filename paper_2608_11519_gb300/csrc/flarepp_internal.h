@@ -216,7 +216,7 @@ struct WgradSource {
 };
 struct WgradPlan {
     int NT;
-    int64_t row_tiles, col_tiles, chunk_len, chunks_per_b, n_chunks;
+    int64_t row_tiles, row_groups, col_tiles, chunk_len, chunks_per_b, n_chunks;
     size_t part_bytes;  // float32 partials [n_chunks][R][Cc]
 };
 WgradPlan wgrad_plan(int64_t B, int64_t N, int64_t R, int64_t Cc);

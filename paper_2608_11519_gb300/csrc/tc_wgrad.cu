@@ -12,13 +12,17 @@
 //   HEADS: up to four tensors [B*H][N][D] side by side (channel r: tensor r / C, head
 //          (r % C) / D, column r % D), or
 //   PLAIN: one matrix [B][N][C] (channel r: column r).
-// A work item is (128 rows of dW, NT columns of dW, a chunk of one batch element's tokens);
-// it writes its float32 partial sum to part[chunk][R][Cc], and a reduce kernel adds the
-// chunks in order (deterministic).
+// A work item is (256 rows of dW, NT columns of dW, a chunk of one batch element's tokens), the
+// rows as two halves of 128 that share B's tile, each with an accumulator of its own: the reads
+// bound the kernel, and with 128 rows every tile of B is fetched twice as often (dW_in of 262,144
+// tokens, C = 256, four projections: 164 -> 128 us; HBM's bytes alone 99). The item writes its
+// float32 partial sum to part[chunk][R][Cc], and a reduce kernel adds the chunks (in a fixed order:
+// deterministic).
 //
 // Roles (8 warps): warp 0 the TMA producer, warp 1 the MMA issuer, warps 4..7 the epilogue
-// (TMEM lane = row of dW). Two TMEM accumulators let the epilogue of one item overlap the
-// products of the next. Every wait is bounded (2 s of %globaltimer), as in the other kernels.
+// (TMEM lane = row of dW). There is about one item per SM, so that nothing is left to overlap an
+// item's epilogue with and the partial sums are few. Every wait is bounded (2 s of %globaltimer), as
+// in the other kernels.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -35,7 +39,8 @@ using namespace tc;
 
 constexpr int kThreads = 256;
 constexpr int kFirstEpiWarp = 4;
-constexpr int kRowsW = 128;   // rows of dW per item (TMEM lanes, MMA M)
+constexpr int kRowsW = 128;   // rows of dW per half of an item (TMEM lanes, MMA M)
+constexpr int kHalves = 2;    // halves per item, at most
 constexpr int kMaxNT = 256;   // columns of dW per item, at most
 constexpr int kTok = 64;      // tokens per pipeline stage (four K = 16 steps)
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
@@ -46,7 +51,7 @@ struct WCfg {
     static constexpr int kAtom = kTok * D * 2;  // one 64-token x D column, swizzled
     static constexpr int kAStage = (kRowsW / D) * kAtom;
     static constexpr int kBStage = (kMaxNT / D) * kAtom;
-    static constexpr int kStage = kAStage + kBStage;
+    static constexpr int kStage = kHalves * kAStage + kBStage;
     static constexpr int kStages = (192 * 1024) / kStage > 6 ? 6 : (192 * 1024) / kStage;
     static constexpr uint32_t kSwz = D == 16 ? kSw32 : (D == 32 ? kSw64 : kSw128);
     static constexpr uint32_t kSBO = 8 * D * 2;  // 8-token groups along K
@@ -64,21 +69,23 @@ struct WgParams {
     int NT;
     uint32_t idesc;
     int64_t chunk_len, chunks_per_b, n_chunks;
-    int64_t row_tiles, col_tiles, n_items;
+    int64_t row_tiles, row_groups, col_tiles, n_items;
     float* part;  // [n_chunks][R][Cc]
     int* status;
 };
 
 struct WItem {
     int64_t rt, ct, b, n0, n1, chunk;
+    int halves;  // row tiles rt, rt + 1, ... of this item
 };
 
 __device__ __forceinline__ WItem witem(const WgParams& p, int64_t v) {
     WItem w;
-    const int64_t tiles = p.row_tiles * p.col_tiles;
+    const int64_t tiles = p.row_groups * p.col_tiles;
     const int64_t t = v % tiles;  // tiles of one chunk run together (their tokens are shared)
     w.chunk = v / tiles;
-    w.rt = t / p.col_tiles;
+    w.rt = t / p.col_tiles * kHalves;
+    w.halves = (int)min((int64_t)kHalves, p.row_tiles - w.rt);
     w.ct = t % p.col_tiles;
     w.b = w.chunk / p.chunks_per_b;
     w.n0 = (w.chunk % p.chunks_per_b) * p.chunk_len;
@@ -178,9 +185,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         // ------------------------------------------------------------ TMA producer
         uint32_t it = 0;
         bool ok = true;
-        const uint32_t bytes = (uint32_t)(W::kAStage + (prm.NT / D) * W::kAtom);
         for (int64_t v = blockIdx.x; v < prm.n_items && ok; v += gridDim.x) {
             const WItem I = witem(prm, v);
+            const uint32_t bytes = (uint32_t)(I.halves * W::kAStage + (prm.NT / D) * W::kAtom);
             for (int64_t n = I.n0; n < I.n1; n += kTok, ++it) {
                 const int st = it % kS;
                 if (it >= (uint32_t)kS &&
@@ -191,9 +198,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (elect_one()) {
                     const uint32_t dst = smem_u32(smem + st * W::kStage);
                     mbar_expect_tx(full0 + 8u * st, bytes);
-                    load_atoms<D>(dst, prm.a_heads, &tA0, &tA1, &tA2, &tA3, I.rt * kRowsW,
-                                  kRowsW, prm.a_apb, prm.C, I.b, (int)n, full0 + 8u * st);
-                    load_atoms<D>(dst + W::kAStage, prm.b_heads, &tB0, &tB1, &tB2, &tB3,
+                    for (int x = 0; x < I.halves; ++x)
+                        load_atoms<D>(dst + x * W::kAStage, prm.a_heads, &tA0, &tA1, &tA2, &tA3,
+                                      (I.rt + x) * kRowsW, kRowsW, prm.a_apb, prm.C, I.b, (int)n,
+                                      full0 + 8u * st);
+                    load_atoms<D>(dst + kHalves * W::kAStage, prm.b_heads, &tB0, &tB1, &tB2, &tB3,
                                   I.ct * prm.NT, prm.NT, prm.b_apb, prm.C, I.b, (int)n,
                                   full0 + 8u * st);
                 }
@@ -211,19 +220,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        uint32_t it = 0, j = 0;
+        // row tile number seq of this CTA is summed in accumulator seq & 1
+        uint32_t it = 0, seq = 0;
         bool ok = true;
-        for (int64_t v = blockIdx.x; v < prm.n_items && ok; v += gridDim.x, ++j) {
+        for (int64_t v = blockIdx.x; v < prm.n_items && ok; v += gridDim.x) {
             const WItem I = witem(prm, v);
-            const int ab = j & 1;
-            if (j >= 2 &&
-                !warp_wait(accempty0 + 8u * ab, ((j >> 1) - 1) & 1, abort_flag, prm.status)) {
-                ok = false;
-                break;
-            }
-            tc_fence_after();
-            const uint32_t acc = tmem + ab * kMaxNT;
-            bool first = true;
+            for (int x = 0; x < I.halves && ok; ++x)  // the accumulators are read out
+                ok = seq + x < 2 ||
+                     warp_wait(accempty0 + 8u * ((seq + x) & 1), (((seq + x) >> 1) - 1) & 1,
+                               abort_flag, prm.status);
+            if (!ok) break;
             for (int64_t n = I.n0; n < I.n1; n += kTok, ++it) {
                 const int st = it % kS;
                 if (!warp_wait(full0 + 8u * st, (it / kS) & 1, abort_flag, prm.status)) {
@@ -231,24 +237,32 @@ __global__ void __launch_bounds__(kThreads, 1)
                     break;
                 }
                 tc_fence_after();
-                const uint32_t a = smem_u32(smem + st * W::kStage);
-                const uint32_t b = a + W::kAStage;
+                const uint32_t a0 = smem_u32(smem + st * W::kStage);
+                if (elect_one()) {
+                    // MN-major operands: K steps of 16 tokens inside each atom (16 D 2 bytes on, in
+                    // the descriptors' units of 16); atoms (D-wide channel columns) kAtom bytes
+                    // apart along M and N
+                    const uint64_t bd =
+                        smem_desc(a0 + kHalves * W::kAStage, W::kAtom, W::kSBO, W::kSwz);
 #pragma unroll
-                for (int k = 0; k < kTok / 16; ++k) {
-                    // MN-major operands: K steps of 16 tokens inside each atom; atoms (D-wide
-                    // channel columns) kAtom bytes apart along M and N
-                    const uint64_t ad = smem_desc(a + k * 16 * D * 2, W::kAtom, W::kSBO, W::kSwz);
-                    const uint64_t bd = smem_desc(b + k * 16 * D * 2, W::kAtom, W::kSBO, W::kSwz);
-                    if (elect_one()) mma_ss(acc, ad, bd, prm.idesc, (first && k == 0) ? 0u : 1u);
-                    __syncwarp();
+                    for (int x = 0; x < kHalves; ++x) {
+                        if (x >= I.halves) break;
+                        const uint32_t acc = tmem + ((seq + x) & 1) * kMaxNT;
+                        const uint64_t ad = smem_desc(a0 + x * W::kAStage, W::kAtom, W::kSBO, W::kSwz);
+#pragma unroll
+                        for (int k = 0; k < kTok / 16; ++k)
+                            mma_ss(acc, ad + 2 * D * k, bd + 2 * D * k, prm.idesc,
+                                   (n == I.n0 && k == 0) ? 0u : 1u);
+                    }
+                    mma_commit(empty0 + 8u * st);
                 }
-                first = false;
-                if (elect_one()) mma_commit(empty0 + 8u * st);
                 __syncwarp();
             }
             if (!ok) break;
-            if (elect_one()) mma_commit(accfull0 + 8u * ab);
+            if (elect_one())
+                for (int x = 0; x < I.halves; ++x) mma_commit(accfull0 + 8u * ((seq + x) & 1));
             __syncwarp();
+            seq += I.halves;
         }
         if (elect_one()) mma_commit(fin);
         __syncwarp();
@@ -262,29 +276,35 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int r = 32 * q + lane;
         const uint32_t lane_off = (uint32_t)(32 * q) << 16;
         uint32_t j = 0;
-        for (int64_t v = blockIdx.x; v < prm.n_items; v += gridDim.x, ++j) {
+        bool ok = true;
+        for (int64_t v = blockIdx.x; v < prm.n_items && ok; v += gridDim.x) {
             const WItem I = witem(prm, v);
-            const int ab = j & 1;
-            if (!warp_wait(accfull0 + 8u * ab, (j >> 1) & 1, abort_flag, prm.status)) break;
-            tc_fence_after();
-            const uint32_t acc = tmem + lane_off + ab * kMaxNT;
-            const int64_t row = I.rt * kRowsW + r;
-            float* dst = prm.part + (I.chunk * prm.R + row) * prm.Cc + I.ct * prm.NT;
-            for (int c = 0; c < prm.NT; c += 16) {
-                uint32_t v16[16];
-                tmem_ld16(acc + c, v16);
-                tmem_wait_ld16(v16);
-                if (row < prm.R) {
-                    float4* d4 = reinterpret_cast<float4*>(dst + c);
-#pragma unroll
-                    for (int g = 0; g < 4; ++g)
-                        d4[g] = make_float4(__uint_as_float(v16[4 * g]), __uint_as_float(v16[4 * g + 1]),
-                                            __uint_as_float(v16[4 * g + 2]),
-                                            __uint_as_float(v16[4 * g + 3]));
+            for (int x = 0; x < I.halves; ++x, ++j) {
+                const int ab = j & 1;
+                if (!warp_wait(accfull0 + 8u * ab, (j >> 1) & 1, abort_flag, prm.status)) {
+                    ok = false;
+                    break;
                 }
+                tc_fence_after();
+                const uint32_t acc = tmem + lane_off + ab * kMaxNT;
+                const int64_t row = (I.rt + x) * kRowsW + r;
+                float* dst = prm.part + (I.chunk * prm.R + row) * prm.Cc + I.ct * prm.NT;
+                for (int c = 0; c < prm.NT; c += 16) {
+                    uint32_t v16[16];
+                    tmem_ld16(acc + c, v16);
+                    tmem_wait_ld16(v16);
+                    if (row < prm.R) {
+                        float4* d4 = reinterpret_cast<float4*>(dst + c);
+#pragma unroll
+                        for (int g = 0; g < 4; ++g)
+                            d4[g] = make_float4(
+                                __uint_as_float(v16[4 * g]), __uint_as_float(v16[4 * g + 1]),
+                                __uint_as_float(v16[4 * g + 2]), __uint_as_float(v16[4 * g + 3]));
+                    }
+                }
+                tc_fence_before();
+                mbar_arrive(accempty0 + 8u * ab);
             }
-            tc_fence_before();
-            mbar_arrive(accempty0 + 8u * ab);
         }
     }
     tc_fence_before();
@@ -293,18 +313,49 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 1) tmem_dealloc(tmem, kTmemCols);
 }
 
-// dW = sum of the chunks' partials, in chunk order; rows r < R_out take the sum of the rows
-// r + k * R_out for k < fold (fold 2 adds the gradients of tied projections).
-__global__ void wgrad_reduce_kernel(const float* __restrict__ part, int64_t n_chunks, int64_t R,
-                                    int64_t Cc, int64_t R_out, int fold,
-                                    __nv_bfloat16* __restrict__ out) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= R_out * Cc) return;
-    const int64_t r = i / Cc, c = i % Cc;
-    float acc = 0.f;
-    for (int k = 0; k < fold; ++k)
-        for (int64_t ch = 0; ch < n_chunks; ++ch) acc += part[(ch * R + r + k * R_out) * Cc + c];
-    out[i] = __float2bfloat16_rn(acc);
+// dW = sum of the chunks' partials; rows r < R_out take the sum of the rows r + k * R_out for
+// k < fold (fold 2 adds the gradients of tied projections). A block of eight warps has 128 values of
+// dW, four per lane; warp w adds the partials w, w + 8, ... of the fold * n_chunks, then the eight
+// sums are added in warp order. (One thread per value going through all chunks was a chain of loads:
+// 44 us for dWo and 26 for dW_in at 262,144 tokens, C = 256, four projections; now 10 and 12.)
+constexpr int kReduceWarps = 8;
+__global__ void __launch_bounds__(32 * kReduceWarps)
+    wgrad_reduce_kernel(const float* __restrict__ part, int64_t n_chunks, int64_t R, int64_t Cc,
+                        int64_t R_out, int fold, __nv_bfloat16* __restrict__ out) {
+    __shared__ float4 sums[kReduceWarps][32];
+    const int w = threadIdx.x / 32, lane = threadIdx.x & 31;
+    const int64_t i = ((int64_t)blockIdx.x * 32 + lane) * 4;  // Cc is a multiple of 16
+    const bool in = i < R_out * Cc;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (in) {
+        for (int k = 0; k < fold; ++k) {
+            const float* src = part + k * R_out * Cc + i;
+#pragma unroll 4
+            for (int64_t ch = w; ch < n_chunks; ch += kReduceWarps) {
+                const float4 v = *reinterpret_cast<const float4*>(src + ch * R * Cc);
+                acc.x += v.x;
+                acc.y += v.y;
+                acc.z += v.z;
+                acc.w += v.w;
+            }
+        }
+    }
+    sums[w][lane] = acc;
+    __syncthreads();
+    if (w != 0 || !in) return;
+    for (int g = 1; g < kReduceWarps; ++g) {
+        const float4 v = sums[g][lane];
+        acc.x += v.x;
+        acc.y += v.y;
+        acc.z += v.z;
+        acc.w += v.w;
+    }
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x, acc.y);
+    const __nv_bfloat162 hi = __floats2bfloat162_rn(acc.z, acc.w);
+    uint2 o;
+    o.x = *reinterpret_cast<const uint32_t*>(&lo);
+    o.y = *reinterpret_cast<const uint32_t*>(&hi);
+    *reinterpret_cast<uint2*>(out + i) = o;
 }
 
 __global__ void transpose_bf16_kernel(const __nv_bfloat16* __restrict__ src, int64_t R,
@@ -421,10 +472,10 @@ WgradPlan wgrad_plan(int64_t B, int64_t N, int64_t R, int64_t Cc) {
     w.NT = nt;
     w.row_tiles = (R + kRowsW - 1) / kRowsW;
     w.col_tiles = Cc / nt;
-    // about four items per SM, chunks of whole 64-token stages inside one batch element
-    const int64_t tiles = w.row_tiles * w.col_tiles;
-    int64_t want = (4 * kNumSMs + tiles - 1) / tiles;
-    int64_t per_b = (want + B - 1) / B;
+    // one item per SM (chunks of whole 64-token stages inside one batch element)
+    w.row_groups = (w.row_tiles + kHalves - 1) / kHalves;
+    const int64_t tiles = w.row_groups * w.col_tiles;
+    int64_t per_b = kNumSMs / (tiles * B);
     if (per_b < 1) per_b = 1;
     w.chunk_len = ((N + per_b - 1) / per_b + kTok - 1) / kTok * kTok;
     if (w.chunk_len < kTok) w.chunk_len = kTok;
@@ -455,7 +506,8 @@ cudaError_t tc_wgrad(int64_t B, int64_t N, int64_t H, int64_t D, const WgradSour
     prm.n_chunks = w.n_chunks;
     prm.row_tiles = w.row_tiles;
     prm.col_tiles = w.col_tiles;
-    prm.n_items = w.n_chunks * w.row_tiles * w.col_tiles;
+    prm.row_groups = w.row_groups;
+    prm.n_items = w.n_chunks * w.row_groups * w.col_tiles;
     prm.part = part;
     prm.status = status;
     CUtensorMap ma[4], mb[4];
@@ -472,7 +524,7 @@ cudaError_t tc_wgrad(int64_t B, int64_t N, int64_t H, int64_t D, const WgradSour
     }
     if (e != cudaSuccess) return e;
     const int64_t n = R_out * Cc;
-    wgrad_reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
+    wgrad_reduce_kernel<<<(unsigned)((n + 127) / 128), 32 * kReduceWarps, 0, st>>>(
         part, w.n_chunks, R, Cc, R_out, fold, (__nv_bfloat16*)dW);
     return cudaGetLastError();
 }

@@ -1,8 +1,9 @@
-"""The mixer's projections where their tiles change form: row tiles taken in pairs (from 304 tiles of
-128 tokens on, in the products that read the heads' tensors), an odd number of them, a last one of a
-few rows, pairs that would cross from one batch element into the next; and column tiles that span two
-projections. Layer and gradients against the oracle, each within 2e-2 of its own scale as in the
-parity tests (bf16 operands and results, float32 sums)."""
+"""The mixer's projections and weight gradients where their tiles change form: row tiles taken in
+pairs (from 304 tiles of 128 tokens on, in the products that read the heads' tensors), an odd number
+of them, a last one of a few rows, pairs that would cross from one batch element into the next; column
+tiles that span two projections; and the weight gradients' items of 256 rows, whole and cut short.
+Layer and gradients against the oracle, each within 2e-2 of its own scale as in the parity tests (bf16
+operands and results, float32 sums)."""
 import math
 
 import numpy as np
@@ -28,6 +29,8 @@ SHAPES = [  # B, H, N, M, D, P
     (1, 1, 304 * 128 + 1, 16, 16, 4),  # 305: the last pair has one tile, of one row
     (102, 1, 300, 16, 64, 2),          # three row tiles per batch element: a pair and a single
     (3, 3, 200, 16, 32, 4),            # four heads per column tile of twelve, three per projection
+    (160, 1, 70, 16, 32, 2),           # more weight-gradient items than SMs, six tokens in a last stage
+    (2, 5, 130, 16, 64, 4),            # C = 320: weight-gradient rows in 128s, the last half of an item
 ]
 
 
