@@ -437,16 +437,17 @@ def arm_config(w, variant, world, l2="auto"):
 
 
 def chain_bwd_launches(w):
-    """Kernels of one chain backward: on the tensor-core path c3, two operand copies, R3 and
-    its reduce, then T23, R2 and its reduce, T1, R1 and the seeds' reduce; for D <= 32 also the
-    range and flag kernels and the w dZ operand, with the merged pass (the token passes that
-    also form dQ, up to 512 routes at D = 32 and 1024 at D = 16, take R1's place as well). On
-    the CUDA-core path c3 and three route passes, two token passes and three reduces."""
+    """Kernels of one chain backward: on the tensor-core path the prologue (c3, the operand
+    copies, the ranges), R3 and its reduce, then T23, R2 and its reduce, T1, R1 and the seeds'
+    reduce; for D <= 32 also the flags and the w dZ operand, with the merged pass. Up to 512
+    routes at D = 32 and 1024 at D = 16: the prologue, dZ and its reduce, the token passes that
+    also form dQ with a reduce each, and the three passes that flagged heads alone run. On the
+    CUDA-core path c3 and three route passes, two token passes and three reduces."""
     if w.dtype != "bf16":
         return 9
     if w.D > 32:
-        return 11
-    return 14 if w.M <= (512 if w.D == 32 else 1024) else 15
+        return 9
+    return 10 if w.M <= (512 if w.D == 32 else 1024) else 12
 
 
 def chain_fwd_launches(w):

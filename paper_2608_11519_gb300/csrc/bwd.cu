@@ -45,14 +45,12 @@ __device__ __forceinline__ float ex2(float x) {
 
 // c3[n] = <dY_n, Y_n>: each thread reads one 16-byte vector of a row of dY and of Y (so a
 // warp reads consecutive rows whole), and the D / V threads of a row add their partial dot
-// products with shuffles. rows * D / V threads in all.
+// products with shuffles. rows * D / V threads in all, t of them.
 template <int D, typename T>
-__global__ void __launch_bounds__(256) delta_tokens_kernel(const T* __restrict__ dY,
-                                                           const T* __restrict__ Y, int64_t rows,
-                                                           float* __restrict__ c3) {
+__device__ __forceinline__ void delta_token(const T* __restrict__ dY, const T* __restrict__ Y,
+                                            int64_t rows, float* __restrict__ c3, int64_t t) {
     constexpr int V = 16 / (int)sizeof(T);  // elements per 16-byte vector
     constexpr int TPR = D / V;              // threads per row (2 .. 16, a power of two)
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t r = t / TPR;
     float acc = 0.f;
     if (r < rows) {
@@ -67,31 +65,18 @@ __global__ void __launch_bounds__(256) delta_tokens_kernel(const T* __restrict__
     for (int off = TPR / 2; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
     if (r < rows && (t % TPR) == 0) c3[r] = acc;
 }
+template <int D, typename T>
+__global__ void __launch_bounds__(256) delta_tokens_kernel(const T* __restrict__ dY,
+                                                           const T* __restrict__ Y, int64_t rows,
+                                                           float* __restrict__ c3) {
+    delta_token<D, T>(dY, Y, rows, c3, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+}
 
 template <int D, typename T>
 void launch_delta_tokens(const T* dY, const T* Y, int64_t rows, float* c3, cudaStream_t st) {
     constexpr int TPR = D / (16 / (int)sizeof(T));
     const int64_t threads = rows * TPR;
     delta_tokens_kernel<D, T><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(dY, Y, rows, c3);
-}
-
-// bf16 copy of a float32 array (the tensor-core passes' Q and Z operands)
-__global__ void to_bf16_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ dst,
-                               int64_t n) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        dst[i] = __float2bfloat16_rn(src[i]);
-}
-
-// hi = bf16(src), lo = bf16(src - hi): the operand pair the training forward gave Q
-__global__ void to_bf16_hilo_kernel(const float* __restrict__ src, __nv_bfloat16* __restrict__ hi,
-                                    __nv_bfloat16* __restrict__ lo, int64_t n) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const __nv_bfloat16 h = __float2bfloat16_rn(src[i]);
-        hi[i] = h;
-        lo[i] = __float2bfloat16_rn(src[i] - __bfloat162float(h));
-    }
 }
 
 // Route pass of call MODE (3, 2 or 1) over one chunk of tokens, float32; thread = route m.
@@ -441,17 +426,34 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, co
 // over more than ~60 binary orders) is flagged and runs the unmerged T23 pass instead.
 constexpr float kMergeRange = 60.f;
 
-// part[bh][j] for j < kRangeParts: max of L3 over slice j of the tokens; part[bh][kRangeParts]
-// and [kRangeParts + 1]: min and max of L2 (from slice 0's block). One block per (bh, j).
-__global__ void __launch_bounds__(256) merge_range_kernel(const float* __restrict__ L2,
-                                                          const float* __restrict__ L3, int64_t M,
-                                                          int64_t N, float* __restrict__ part) {
+// four floats as four bf16 and back
+__device__ __forceinline__ uint2 pack4(float4 v) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y);
+    const __nv_bfloat162 hi = __floats2bfloat162_rn(v.z, v.w);
+    return make_uint2(*reinterpret_cast<const uint32_t*>(&lo),
+                      *reinterpret_cast<const uint32_t*>(&hi));
+}
+__device__ __forceinline__ float dot4(float4 a, float4 b) {
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, a.x * b.x)));
+}
+__device__ __forceinline__ float4 unpack4(uint2 p) {
+    const float2 f0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&p.x));
+    const float2 f1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&p.y));
+    return make_float4(f0.x, f0.y, f1.x, f1.y);
+}
+
+// part[bh][j] for j < parts: max of L3 over slice j of the tokens; part[bh][kRangeParts] and
+// [kRangeParts + 1]: min and max of L2 (from slice 0's block). One block per (bh, j), block `id`.
+__device__ __forceinline__ void merge_range(const float* __restrict__ L2,
+                                            const float* __restrict__ L3, int64_t M, int64_t N,
+                                            int parts, int64_t id, float* __restrict__ part) {
     __shared__ float red[3][8];
-    const int64_t bh = blockIdx.x / kRangeParts;
-    const int j = (int)(blockIdx.x % kRangeParts);
-    const int64_t per = (N + kRangeParts - 1) / kRangeParts;
+    const int64_t bh = id / parts;
+    const int j = (int)(id % parts);
+    const int64_t per = (N + parts - 1) / parts;
     const int64_t n0 = j * per, n1 = min(N, n0 + per);
     float mx3 = -INFINITY, mn2 = INFINITY, mx2 = -INFINITY;
+#pragma unroll 8
     for (int64_t n = n0 + threadIdx.x; n < n1; n += blockDim.x) mx3 = fmaxf(mx3, L3[bh * N + n]);
     if (j == 0)
         for (int64_t m = threadIdx.x; m < M; m += blockDim.x) {
@@ -486,38 +488,71 @@ __global__ void __launch_bounds__(256) merge_range_kernel(const float* __restric
         }
     }
 }
+// slices of the tokens: 4096 each (16 loads per thread), at most kRangeParts
+inline int range_parts(int64_t N) {
+    const int64_t n = (N + 4095) / 4096;
+    return (int)(n < kRangeParts ? n : kRangeParts);
+}
 
-// R[bh] = min_m L2 and flags[bh] = 1 when the (b, h) runs the unmerged pass.
-__global__ void merge_flags_kernel(const float* __restrict__ part, int64_t BH,
-                                   float* __restrict__ Rb, int* __restrict__ flags) {
-    const int64_t bh = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (bh >= BH) return;
+// Everything that the tensor-core backward needs ahead of its passes, none of it depending on the
+// rest: the slices' ranges for the merged pass (blocks [0, BH * parts); none when parts is 0), the
+// bf16 operands of Q (with its lo part when lo is given, as the training forward took it) and Z (the
+// next `cvt` blocks), and c3 (the rest, bound by the reads of dY and Y). Block 0 also clears the word
+// behind the flags. One launch: as four they took 25 us at 32 (b, h) of 16,384 tokens, D = 32, this
+// 13.
+template <int D>
+__global__ void __launch_bounds__(256) bwd_prologue_kernel(
+    const __nv_bfloat16* __restrict__ dY, const __nv_bfloat16* __restrict__ Y, int64_t rows,
+    float* __restrict__ c3, const float* __restrict__ Q, const float* __restrict__ Z, int64_t lat,
+    __nv_bfloat16* __restrict__ qb, __nv_bfloat16* __restrict__ qlo, __nv_bfloat16* __restrict__ zb,
+    unsigned cvt, const float* __restrict__ L2, const float* __restrict__ L3, int64_t BH, int64_t M,
+    int64_t N, int parts, float* __restrict__ rpart, int* __restrict__ any) {
+    tc::pdl_trigger();
+    int64_t id = blockIdx.x;
+    if (any != nullptr && id == 0 && threadIdx.x == 0) *any = 0;
+    if (id < BH * parts) {
+        merge_range(L2, L3, M, N, parts, id, rpart);
+        return;
+    }
+    id -= BH * parts;
+    if (id < cvt) {
+        for (int64_t i = id * 256 + threadIdx.x; i < lat / 4; i += (int64_t)cvt * 256) {
+            const float4 q = reinterpret_cast<const float4*>(Q)[i];
+            const uint2 hi = pack4(q);
+            reinterpret_cast<uint2*>(qb)[i] = hi;
+            if (qlo != nullptr) {
+                const float4 h = unpack4(hi);
+                reinterpret_cast<uint2*>(qlo)[i] =
+                    pack4(make_float4(q.x - h.x, q.y - h.y, q.z - h.z, q.w - h.w));
+            }
+            reinterpret_cast<uint2*>(zb)[i] = pack4(reinterpret_cast<const float4*>(Z)[i]);
+        }
+        return;
+    }
+    id -= cvt;
+    delta_token<D>(dY, Y, rows, c3, id * 256 + threadIdx.x);
+}
+
+// R[bh] = min_m L2; flags[bh] = 1 when the (b, h) runs the unmerged pass, and then flags[BH] = 1.
+__device__ __forceinline__ void merge_flag(const float* __restrict__ part, int parts, int64_t bh,
+                                           int64_t BH, float* __restrict__ Rb,
+                                           int* __restrict__ flags) {
     const float* o = part + bh * (kRangeParts + 2);
     float mx3 = -INFINITY;
-    for (int j = 0; j < kRangeParts; ++j) mx3 = fmaxf(mx3, o[j]);
+#pragma unroll 8
+    for (int j = 0; j < parts; ++j) mx3 = fmaxf(mx3, o[j]);
     const float R = o[kRangeParts], mx2 = o[kRangeParts + 1];
     Rb[bh] = R;
-    flags[bh] = (mx3 - R <= kMergeRange && mx2 - R <= kMergeRange) ? 0 : 1;
+    const bool fits = mx3 - R <= kMergeRange && mx2 - R <= kMergeRange;
+    flags[bh] = fits ? 0 : 1;
+    if (!fits) atomicOr(flags + BH, 1);
+}
+__global__ void merge_flags_kernel(const float* __restrict__ part, int parts, int64_t BH,
+                                   float* __restrict__ Rb, int* __restrict__ flags) {
+    const int64_t bh = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (bh < BH) merge_flag(part, parts, bh, BH, Rb, flags);
 }
 
-// The merged pass's route operand w dZ: W[bh][m][:] = bf16(2^(R[bh] - L2[bh][m]) dZ[bh][m][:]), and
-// c2 taken from it: c2w = <W, Z> / w. The pass forms w dP2 = W V^T, and dS2 = P2 (dP2 - c2)
-// cancels for a nearly one-hot P2 only when c2 sees the same rounded dZ. v, z: this thread's four
-// channels (group g of D / 4) of the row of dZ and Z.
-__device__ __forceinline__ uint2 pack4(float4 v) {
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y);
-    const __nv_bfloat162 hi = __floats2bfloat162_rn(v.z, v.w);
-    return make_uint2(*reinterpret_cast<const uint32_t*>(&lo),
-                      *reinterpret_cast<const uint32_t*>(&hi));
-}
-__device__ __forceinline__ float dot4(float4 a, float4 b) {
-    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, a.x * b.x)));
-}
-__device__ __forceinline__ float4 unpack4(uint2 p) {
-    const float2 f0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&p.x));
-    const float2 f1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&p.y));
-    return make_float4(f0.x, f0.y, f1.x, f1.y);
-}
 // the sum of x over a row's T threads (adjacent lanes)
 template <int T>
 __device__ __forceinline__ float row_sum(float x) {
@@ -527,6 +562,10 @@ __device__ __forceinline__ float row_sum(float x) {
     for (int off = T / 2; off > 0; off >>= 1) x += __shfl_xor_sync(mask, x, off);
     return x;
 }
+// The merged pass's route operand w dZ: W[bh][m][:] = bf16(2^(R[bh] - L2[bh][m]) dZ[bh][m][:]), and
+// c2 taken from it: c2w = <W, Z> / w. The pass forms w dP2 = W V^T, and dS2 = P2 (dP2 - c2)
+// cancels for a nearly one-hot P2 only when c2 sees the same rounded dZ. v, z: this thread's four
+// channels (group g of D / 4) of the row of dZ and Z.
 template <int D>
 __device__ __forceinline__ void merge_operand(float4 v, float4 z, float e, int64_t row, int g,
                                               __nv_bfloat16* W, float* c2w) {
@@ -553,20 +592,25 @@ __global__ void __launch_bounds__(256)
 
 // dZ from the partial sums of tc_dz_pass, slot by slot in order (a chunk's token-parity parts as
 // the encode's plan cuts them: 4, 2 or 1 by the route tiles of the row's group of 512): its bf16
-// copy, c2 = <dZ, Z>, and the merged pass's operand. D / 4 threads per row, four loads in flight.
+// copy, c2 = <dZ, Z>, and the merged pass's operand; and the (b, h)'s shift and flag. D / 4
+// threads per row, four loads in flight.
 template <int D>
 __global__ void __launch_bounds__(256)
     dz_reduce_kernel(const float* __restrict__ part, int M, int nchunk, int64_t rows,
                      const float* __restrict__ Z, const float* __restrict__ L2,
-                     const float* __restrict__ Rb, __nv_bfloat16* __restrict__ dzb,
+                     const float* __restrict__ rpart, int parts, float* __restrict__ Rb,
+                     int* __restrict__ flags, __nv_bfloat16* __restrict__ dzb,
                      float* __restrict__ c2, __nv_bfloat16* __restrict__ W,
                      float* __restrict__ c2w) {
     constexpr int T = D / 4;
+    tc::pdl_trigger();
+    tc::pdl_wait();
     const int64_t row = ((int64_t)blockIdx.x * 256 + threadIdx.x) / T;  // bh * M + m
     const int g = threadIdx.x % T;
     if (row >= rows) return;  // (rows in whole groups of T threads)
     const int64_t bh = row / M;
     const int m = (int)(row - bh * M);
+    if (m == 0 && g == 0) merge_flag(rpart, parts, bh, rows / M, Rb, flags);
     const int left = M - (m & ~511);
     const int ul = left > 256 ? 0 : (left > 128 ? 1 : 2);  // log2 of the parts per chunk
     const int n = nchunk << ul, mask = (1 << ul) - 1;
@@ -593,7 +637,7 @@ __global__ void __launch_bounds__(256)
     reinterpret_cast<uint2*>(dzb + row * D)[g] = pack4(a);
     const float dot = row_sum<T>(dot4(a, z));
     if (g == 0) c2[row] = dot;
-    merge_operand<D>(a, z, Rb[bh] - L2[row], row, g, W, c2w);
+    merge_operand<D>(a, z, rpart[bh * (kRangeParts + 2) + kRangeParts] - L2[row], row, g, W, c2w);
 }
 
 // Reduce of the partials dS^T K that the token passes of tc_tok.cu leave, a CTA's slot each:
@@ -611,6 +655,8 @@ __global__ void __launch_bounds__(256)
                       const float* __restrict__ pa, int64_t nchunk, const float* __restrict__ Q,
                       float* __restrict__ c1, __nv_bfloat16* __restrict__ op) {
     constexpr int T = D / 4;
+    tc::pdl_trigger();
+    tc::pdl_wait();
     const int64_t row = ((int64_t)blockIdx.x * 256 + threadIdx.x) / T;
     const int g = threadIdx.x % T;
     if (row >= rows) return;  // (rows in whole groups of T threads)
@@ -695,24 +741,20 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
     const int64_t lat_rows = p.BH * p.M;
     const int64_t lat = lat_rows * p.D;
     const unsigned red_blocks = (unsigned)((lat_rows + 7) / 8);
-    const unsigned cvt_blocks = (unsigned)min((int64_t)1024, (lat + 255) / 256);
     cudaError_t e;
 
     constexpr bool kMerged = D <= 32;
-    launch_delta_tokens<D, T>((const T*)dY, (const T*)Y, tok_rows, c3, st);
     // Q as the training forward gave it to calls 2 and 3: a hi/lo pair for D <= 32
     T* qlo = kMerged ? (T*)(ws + bp.off_qlo) : nullptr;
-    if (qlo)
-        to_bf16_hilo_kernel<<<cvt_blocks, 256, 0, st>>>(Q32, qb, qlo, lat);
-    else
-        to_bf16_kernel<<<cvt_blocks, 256, 0, st>>>(Q32, qb, lat);
-    to_bf16_kernel<<<cvt_blocks, 256, 0, st>>>(Z32, zb, lat);
-    if (kMerged) {
-        merge_range_kernel<<<(unsigned)(p.BH * kRangeParts), 256, 0, st>>>(L2, L3, p.M, p.N,
-                                                                           rpart);
-        merge_flags_kernel<<<(unsigned)((p.BH + 127) / 128), 128, 0, st>>>(rpart, p.BH, Rb,
+    const int parts = kMerged ? range_parts(p.N) : 0;
+    const unsigned cvt = (unsigned)min((int64_t)kNumSMs, (lat / 4 + 255) / 256);
+    const int64_t delta = (tok_rows * (D / 8) + 255) / 256;
+    bwd_prologue_kernel<D><<<(unsigned)(p.BH * parts + cvt + delta), 256, 0, st>>>(
+        (const T*)dY, (const T*)Y, tok_rows, c3, Q32, Z32, lat, qb, qlo, zb, cvt, L2, L3, p.BH, p.M,
+        p.N, parts, rpart, kMerged ? flags + p.BH : nullptr);
+    if (kMerged && bp.tok_slots == 0)
+        merge_flags_kernel<<<(unsigned)((p.BH + 127) / 128), 128, 0, st>>>(rpart, parts, p.BH, Rb,
                                                                             flags);
-    }
     // R3: route rows; S = Q K^T, dP = Z dY^T; column statistics L3, c3 -> dQ3, dZ partials
     TcBwdOperands r3{{qb, zb, zb}, {K, dY, dY}, nullptr, nullptr, L3, c3, pa, pb, nullptr, nullptr};
     r3.lo = qlo;
@@ -726,6 +768,7 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
     if constexpr (kMerged) {
         t23.flags = flags;  // the flagged (b, h) run the unmerged T23
         t23.want = 1;
+        t23.any = flags + p.BH;
         if (bp.tok_slots > 0) {
             // dZ as an encode of K and dY, then the token passes that also form dQ and dseeds;
             // the flagged (b, h) take R3 (for its dQ3), T23 and R2 (its dQ2 partials go to pa,
@@ -736,26 +779,34 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
             const auto blocks = [](int64_t rows) { return (unsigned)((rows * (D / 4) + 255) / 256); };
             r3.flags = r2.flags = flags;
             r3.want = r2.want = 1;
+            r3.any = r2.any = flags + p.BH;
             r2.pb = pa;
             if ((e = tc_dz_pass(p, qb, qlo, K, dY, L3, scale, pz, status, st)) != cudaSuccess)
                 return e;
-            dz_reduce_kernel<D><<<blocks(lat_rows), 256, 0, st>>>(
-                pz, (int)p.M, (int)p.nchunk, lat_rows, Z32, L2, Rb, dzb, c2, wop, c2w);
+            if ((e = launch_pdl(dz_reduce_kernel<D>, dim3(blocks(lat_rows)), dim3(256), 0, st,
+                                (const float*)pz, (int)p.M, (int)p.nchunk, lat_rows, Z32, L2,
+                                (const float*)rpart, parts, Rb, flags, dzb, c2, wop, c2w)) !=
+                cudaSuccess)
+                return e;
             TokOperands t{{K, V, dY}, {qb, wop, zb}, qlo, L3, c3, L2, c2w, Rb, flags, pt, dK, dV};
             if ((e = tc_tok_pass(p, bp, false, t, scale, status, st)) != cudaSuccess) return e;
             if ((e = tc_bwd_pass(p, bp, 0, r3, scale, status, st)) != cudaSuccess) return e;
             if ((e = tc_bwd_pass(p, bp, 3, t23, scale, status, st)) != cudaSuccess) return e;
             if ((e = tc_bwd_pass(p, bp, 1, r2, scale, status, st)) != cudaSuccess) return e;
-            tok_reduce_kernel<D, false><<<blocks(lat_rows), 256, 0, st>>>(
-                pt, lat_rows, p.B, p.H, p.M, bp.tok_nt, tiles, bp.tok_ctas, bp.tok_slots, scale,
-                flags, pb, pa, bp.nchunk, Q32, c1, dqb);
+            if ((e = launch_pdl(tok_reduce_kernel<D, false>, dim3(blocks(lat_rows)), dim3(256), 0, st,
+                                (const float*)pt, lat_rows, p.B, p.H, p.M, bp.tok_nt, tiles,
+                                bp.tok_ctas, bp.tok_slots, scale, (const int*)flags,
+                                (const float*)pb, (const float*)pa, bp.nchunk, Q32, c1, dqb)) !=
+                cudaSuccess)
+                return e;
             t = TokOperands{{Kt, Vt, Vt}, {seeds, dqb, dqb}, nullptr, nullptr, nullptr, L1, c1,
                             nullptr, nullptr, pt, dKt, dVt};
             if ((e = tc_tok_pass(p, bp, true, t, scale, status, st)) != cudaSuccess) return e;
-            tok_reduce_kernel<D, true><<<blocks(p.H * p.M), 256, 0, st>>>(
-                pt, p.H * p.M, p.B, p.H, p.M, bp.tok_nt, tiles, bp.tok_ctas, bp.tok_slots, scale,
-                nullptr, nullptr, nullptr, 0, nullptr, nullptr, (T*)dseeds);
-            return cudaGetLastError();
+            return launch_pdl(tok_reduce_kernel<D, true>, dim3(blocks(p.H * p.M)), dim3(256), 0, st,
+                              (const float*)pt, p.H * p.M, p.B, p.H, p.M, bp.tok_nt, tiles,
+                              bp.tok_ctas, bp.tok_slots, scale, (const int*)nullptr,
+                              (const float*)nullptr, (const float*)nullptr, (int64_t)0,
+                              (const float*)nullptr, (float*)nullptr, (T*)dseeds);
         }
     }
     TcBwdOperands o{};

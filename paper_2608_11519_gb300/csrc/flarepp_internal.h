@@ -95,7 +95,7 @@ struct BwdPlan {
     size_t off_qlo;             // ... and Q's lo part, Q - bf16(Q) (D <= 32)
     size_t off_w;               // ... and the merged T23 pass's w dZ [BH][M][D] bf16
     size_t off_c2w;             // ... and its c2, taken from that operand [BH][M] f32
-    size_t off_rb, off_flags;   // its shift R [BH] f32 and fallback flags [BH] int32
+    size_t off_rb, off_flags;   // its shift R [BH] f32 and fallback flags [BH] int32, then their OR
     size_t off_rpart;           // range partials [BH][kRangeParts + 2] f32
     // the token passes that also form dQ (tc_tok.cu): token tiles per (b, h), CTAs, partial slots
     // per (b, h) (0: the shape runs the separate passes), and the partials [BH][slots][M][D] f32
@@ -158,6 +158,7 @@ struct TcBwdOperands {
     const float* Rb = nullptr;  // T23C: the shift R of each (b, h)
     const int* flags = nullptr;  // when set, only the (b, h) with flags[bh] == want run
     int want = 0;
+    const int* any = nullptr;    // when set, nothing runs unless *any is set
     // Q's bf16 lo operand (Q - bf16(Q)) for the hi/lo score products of R3, R2, T23 and T23C
     // at D <= 32, or null (plain bf16 Q)
     const void* lo = nullptr;

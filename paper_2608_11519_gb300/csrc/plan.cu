@@ -218,7 +218,7 @@ BwdPlan make_bwd_plan(const Plan& p) {
         b.off_rb = off;
         off = align_up(off + (size_t)p.BH * 4, kWsAlign);
         b.off_flags = off;
-        off = align_up(off + (size_t)p.BH * 4, kWsAlign);
+        off = align_up(off + ((size_t)p.BH + 1) * 4, kWsAlign);
         b.off_rpart = off;
         off = align_up(off + (size_t)p.BH * (kRangeParts + 2) * 4, kWsAlign);
         if (p.M <= tok_max_routes(p.D) && cdiv(p.N, 128) * p.BH < INT32_MAX) {

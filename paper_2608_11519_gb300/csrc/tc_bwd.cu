@@ -149,6 +149,7 @@ struct BwdParams {
     const float* Rb;    // T23C: the shift R of each (b, h) [BH]
     const int* flags;   // when not null: only the units of (b, h) with flags[bh] == want run
     int want;
+    const int* any;     // when not null: nothing runs unless *any is set
     int* status;
     uint64_t wait_ns;     // bound of every wait (2 s unless the test hook is set)
     int64_t withhold_it;  // test hook: ring item of CTA 0 the producer never loads (-1: none)
@@ -372,6 +373,9 @@ __global__ void __launch_bounds__(BCfg<D, PASS>::kThreads, 1)
                   const __grid_constant__ CUtensorMap tmLo, const BwdParams prm) {
     using C = BCfg<D, PASS, LO>;
     constexpr int NS = C::NS;
+    pdl_trigger();
+    pdl_wait();
+    if (prm.any != nullptr && *reinterpret_cast<const volatile int*>(prm.any) == 0) return;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align_shared<1024>(smem_raw);
     uint8_t* abuf = smem;                          // kABuf x [NS][kNTA] A tiles
@@ -990,9 +994,8 @@ cudaError_t launch_pass(const void* const* srcs, const Plan& p, BwdParams prm, c
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t grid = prm.n_units < sms ? prm.n_units : sms;
-    tc_bwd_kernel<D, PASS, LO><<<(unsigned)grid, Cf::kThreads, Cf::kSmem, st>>>(
-        maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], mlo, prm);
-    return cudaGetLastError();
+    return launch_pdl(tc_bwd_kernel<D, PASS, LO>, dim3((unsigned)grid), dim3(Cf::kThreads), Cf::kSmem,
+                      st, maps[0], maps[1], maps[2], maps[3], maps[4], maps[5], mlo, prm);
 }
 
 // `lo` (srcs[6] holds Q's lo operand): the hi/lo score products, for the passes whose scores
@@ -1054,6 +1057,7 @@ cudaError_t tc_bwd_pass(const Plan& p, const BwdPlan& bp, int pass, const TcBwdO
     prm.Rb = o.Rb;
     prm.flags = o.flags;
     prm.want = o.want;
+    prm.any = o.any;
     prm.status = status;
     test_fault_for(4 + pass, &prm.wait_ns, &prm.withhold_it);
     switch (pass) {

@@ -276,6 +276,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                   const __grid_constant__ CUtensorMap tmLo, const TokParams prm) {
     using C = TokCfg<D, CALL1, LO>;
     constexpr int kS = C::kStages;
+    pdl_trigger();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align_shared<1024>(smem_raw);
     uint8_t* ds_buf = smem;
@@ -341,6 +342,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = warp_uniform(*tmem_slot);
+    // every global access below may depend on the kernel before this one
+    pdl_wait();
     auto wait = [&](uint32_t bar, uint32_t parity) {
         return warp_wait(bar, parity & 1u, abort_flag, prm.status, prm.wait_ns);
     };
@@ -890,9 +893,8 @@ cudaError_t launch(const Plan& p, const TokOperands& o, const TokParams& prm, in
     }
     lo = it[0];
     if (LO && !make_map(&lo, o.lo, D, p.M, p.BH, kItem)) return cudaErrorInvalidValue;
-    tc_tok_kernel<D, CALL1, LO><<<(unsigned)ctas, kThreads, Cf::kSmem, st>>>(
-        a[0], a[1], a[2], it[0], it[1], it[2], lo, prm);
-    return cudaGetLastError();
+    return launch_pdl(tc_tok_kernel<D, CALL1, LO>, dim3((unsigned)ctas), dim3(kThreads), Cf::kSmem,
+                      st, a[0], a[1], a[2], it[0], it[1], it[2], lo, prm);
 }
 
 }  // namespace

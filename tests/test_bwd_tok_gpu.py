@@ -50,3 +50,33 @@ def test_token_passes_match_oracle(shape):
         err = float(np.abs(g.double().cpu().numpy() - r).max())
         bound = 2e-2 * max(1.0, float(np.abs(r).max()))
         assert err <= bound, f"{name}: {err} > {bound}"
+
+
+@pytest.mark.parametrize("N,M,D", [(4097, 130, 32)])
+def test_flagged_heads_over_several_slices(N, M, D):
+    """The ranges of the log-normalisers are taken over slices of 4,096 tokens; one token more makes
+    two. Keys x 16 on head 1 take it out of the merged pass's range while head 0 stays; both match
+    the oracle at the bf16 tolerance."""
+    from test_bwd_gpu import _stat_spread
+    scale = 1.0 / math.sqrt(D)
+    w = inputs.Workload("case", 1, 2, N, M, D, "bf16")
+    x = inputs.make_inputs(w, 5)
+    x["seeds"] = (x["seeds"].float() * 10).to(torch.bfloat16)
+    K = x["K"].float()
+    K[:, 1] *= 16
+    x["K"] = K.to(torch.bfloat16)
+    dY = inputs.make_output_grad(w, 5)
+    f = inputs.to_f64_numpy(x)
+    spread = _stat_spread(f, scale)
+    assert spread[0] < 60.0 < spread[1], spread
+    xd = {k: v.cuda() for k, v in x.items()}
+    args = (xd["seeds"], xd["Kt"], xd["Vt"], xd["K"], xd["V"])
+    Y, saved = flarepp.route_fwd_train(*args, scale)
+    grads = flarepp.route_bwd(*args, Y, dY.cuda(), saved, scale)
+    torch.cuda.synchronize()
+    want = oracle.route_bwd(f["seeds"], f["Kt"], f["Vt"], f["K"], f["V"], scale,
+                            dY.double().numpy())
+    for name, g, r in zip(("dseeds", "dKt", "dVt", "dK", "dV"), grads, want):
+        err = float(np.abs(g.double().cpu().numpy() - r).max())
+        bound = 2e-2 * max(1.0, float(np.abs(r).max()))
+        assert err <= bound, f"{name}: {err} > {bound}"
