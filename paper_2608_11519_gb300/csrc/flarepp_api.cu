@@ -54,6 +54,15 @@ bool spans_overlap(const void* const* ptrs, const size_t* bytes, int n, const vo
     return false;
 }
 
+// Clear the status word (when asked to) and the tensor-core kernels' overflow words, which lie in one
+// block of the workspace: one operation on the stream.
+bool clear_words(const Plan& p, char* ws, bool tc, bool status, cudaStream_t st) {
+    const size_t first = status ? p.off_status : p.off_overflow;
+    const size_t last = tc ? p.off_overflow + 3 * sizeof(int32_t)
+                           : (status ? p.off_status + sizeof(int32_t) : first);
+    return last == first || cudaMemsetAsync(ws + first, 0, last - first, st) == cudaSuccess;
+}
+
 flarepp_status route_impl(const flarepp_shape* shape, const void* seeds, const void* Kt,
                           const void* Vt, const void* K, const void* V, float scale, void* Y,
                           void* workspace, size_t workspace_bytes, void* stream, float* Q_out,
@@ -132,10 +141,7 @@ flarepp_status route_impl(const flarepp_shape* shape, const void* seeds, const v
         return tc ? tc_encode(p, call, k, v, seeds, scale, ws, st, lo)
                   : simt_encode_f32(p, call, k, v, seeds, scale, ws, st);
     };
-    if (reset_status && cudaMemsetAsync(ws + p.off_status, 0, sizeof(int32_t), st) != cudaSuccess)
-        return FLAREPP_ERR_CUDA;
-    if (tc && cudaMemsetAsync(ws + p.off_overflow, 0, 3 * sizeof(int32_t), st) != cudaSuccess)
-        return FLAREPP_ERR_CUDA;
+    if (!clear_words(p, ws, tc, reset_status, st)) return FLAREPP_ERR_CUDA;
     if (tc && neg &&
         negate_bf16(seeds, ws + p.off_seedneg, p.H * p.M * p.D, st) != cudaSuccess)
         return FLAREPP_ERR_CUDA;
@@ -218,10 +224,7 @@ flarepp_status flare_impl(const flarepp_shape* shape, const void* Qh, const void
     char* ws = (char*)workspace;
     const bool tc = p.path == kPathTc;
     const bool neg = scale < 0.f;
-    if (reset_status && cudaMemsetAsync(ws + p.off_status, 0, sizeof(int32_t), st) != cudaSuccess)
-        return FLAREPP_ERR_CUDA;
-    if (tc && cudaMemsetAsync(ws + p.off_overflow, 0, 3 * sizeof(int32_t), st) != cudaSuccess)
-        return FLAREPP_ERR_CUDA;
+    if (!clear_words(p, ws, tc, reset_status, st)) return FLAREPP_ERR_CUDA;
     // the encode of call 1 with the learned queries, merged into Z
     if (tc && neg && negate_bf16(Qh, ws + p.off_seedneg, p.H * p.M * p.D, st) != cudaSuccess)
         return FLAREPP_ERR_CUDA;
