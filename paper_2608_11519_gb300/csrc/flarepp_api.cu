@@ -54,12 +54,15 @@ bool spans_overlap(const void* const* ptrs, const size_t* bytes, int n, const vo
     return false;
 }
 
-// Clear the status word (when asked to) and the tensor-core kernels' overflow words, which lie in one
-// block of the workspace: one operation on the stream.
-bool clear_words(const Plan& p, char* ws, bool tc, bool status, cudaStream_t st) {
-    const size_t first = status ? p.off_status : p.off_overflow;
-    const size_t last = tc ? p.off_overflow + 3 * sizeof(int32_t)
-                           : (status ? p.off_status + sizeof(int32_t) : first);
+// The words a call clears before its kernels run: the tensor-core kernels' overflow words, alone (a
+// group of a host call) or with the status word, or none (a mixer has cleared them ahead of its
+// projection). They lie in one block of the workspace: one operation on the stream.
+enum class Clear { kNone, kOverflow, kAll };
+bool clear_words(const Plan& p, char* ws, bool tc, Clear what, cudaStream_t st) {
+    const size_t first = what == Clear::kAll ? p.off_status : p.off_overflow;
+    size_t last = first;
+    if (what == Clear::kAll) last = p.off_status + sizeof(int32_t);
+    if (what != Clear::kNone && tc) last = p.off_overflow + 3 * sizeof(int32_t);
     return last == first || cudaMemsetAsync(ws + first, 0, last - first, st) == cudaSuccess;
 }
 
@@ -67,7 +70,7 @@ flarepp_status route_impl(const flarepp_shape* shape, const void* seeds, const v
                           const void* Vt, const void* K, const void* V, float scale, void* Y,
                           void* workspace, size_t workspace_bytes, void* stream, float* Q_out,
                           float* Z_out, void* const* events, int n_events,
-                          bool reset_status = true, char* saved = nullptr) {
+                          Clear clear = Clear::kAll, char* saved = nullptr) {
     Plan p;
     flarepp_status stt = make_plan(shape, &p);
     if (stt != FLAREPP_OK) return stt;
@@ -141,7 +144,7 @@ flarepp_status route_impl(const flarepp_shape* shape, const void* seeds, const v
         return tc ? tc_encode(p, call, k, v, seeds, scale, ws, st, lo)
                   : simt_encode_f32(p, call, k, v, seeds, scale, ws, st);
     };
-    if (!clear_words(p, ws, tc, reset_status, st)) return FLAREPP_ERR_CUDA;
+    if (!clear_words(p, ws, tc, clear, st)) return FLAREPP_ERR_CUDA;
     if (tc && neg &&
         negate_bf16(seeds, ws + p.off_seedneg, p.H * p.M * p.D, st) != cudaSuccess)
         return FLAREPP_ERR_CUDA;
@@ -181,7 +184,7 @@ flarepp_status route_impl(const flarepp_shape* shape, const void* seeds, const v
 // B = 32, as long as the encode: 276 us a call at the longseq shape, now 140).
 flarepp_status flare_impl(const flarepp_shape* shape, const void* Qh, const void* K, const void* V,
                           float scale, void* Y, void* workspace, size_t workspace_bytes,
-                          void* stream, float* Z_out, bool reset_status = true) {
+                          void* stream, float* Z_out, Clear clear = Clear::kAll) {
     Plan p;
     flarepp_status stt = make_plan(shape, &p);
     if (stt != FLAREPP_OK) return stt;
@@ -224,7 +227,7 @@ flarepp_status flare_impl(const flarepp_shape* shape, const void* Qh, const void
     char* ws = (char*)workspace;
     const bool tc = p.path == kPathTc;
     const bool neg = scale < 0.f;
-    if (!clear_words(p, ws, tc, reset_status, st)) return FLAREPP_ERR_CUDA;
+    if (!clear_words(p, ws, tc, clear, st)) return FLAREPP_ERR_CUDA;
     // the encode of call 1 with the learned queries, merged into Z
     if (tc && neg && negate_bf16(Qh, ws + p.off_seedneg, p.H * p.M * p.D, st) != cudaSuccess)
         return FLAREPP_ERR_CUDA;
@@ -413,11 +416,12 @@ flarepp_status route_host_impl(const flarepp_shape* shape, const void* seeds_h, 
         const size_t so = (size_t)(bh0 % p.H) * (size_t)p.M * (size_t)p.D * elt;
         ok = cudaStreamWaitEvent(st, e_in[k], 0) == cudaSuccess;
         if (!ok) break;
+        const Clear clear = k == 0 ? Clear::kAll : Clear::kOverflow;
         rc = flare ? flare_impl(&gs, db + L.off_seeds + so, db + L.off_k + o, db + L.off_v + o,
-                                scale, db + L.off_y + o, db, L.ws_bytes, st, nullptr, k == 0)
+                                scale, db + L.off_y + o, db, L.ws_bytes, st, nullptr, clear)
                    : route_impl(&gs, db + L.off_seeds + so, db + off_kt + o, db + off_vt + o,
                                 db + L.off_k + o, db + L.off_v + o, scale, db + L.off_y + o, db,
-                                L.ws_bytes, st, nullptr, nullptr, nullptr, 0, k == 0);
+                                L.ws_bytes, st, nullptr, nullptr, nullptr, 0, clear);
         if (rc != FLAREPP_OK) break;
         ok = cudaEventRecord(e_done[k], st) == cudaSuccess &&
              cudaStreamWaitEvent(cout, e_done[k], 0) == cudaSuccess &&
@@ -453,7 +457,7 @@ flarepp_status route_fwd_train_impl(const flarepp_shape* shape, const void* seed
         if (spans_overlap(ins, nb, 6, saved, sv.total)) return FLAREPP_ERR_INVALID_ARGUMENT;
     }
     return route_impl(shape, seeds, Kt, Vt, K, V, scale, Y, workspace, workspace_bytes, stream,
-                      nullptr, nullptr, nullptr, 0, true, (char*)saved);
+                      nullptr, nullptr, nullptr, 0, Clear::kAll, (char*)saved);
 }
 
 flarepp_status route_bwd_impl(const flarepp_shape* shape, const void* seeds, const void* Kt,
@@ -591,7 +595,7 @@ flarepp_status mixer_impl(const flarepp_shape* shape, int n_proj, const void* X,
         return cudaMemsetAsync(O, 0, x_bytes, st) == cudaSuccess ? FLAREPP_OK : FLAREPP_ERR_CUDA;
     char* ws = (char*)workspace;
     int* status = (int*)(ws + p.off_status);
-    if (cudaMemsetAsync(status, 0, sizeof(int32_t), st) != cudaSuccess) return FLAREPP_ERR_CUDA;
+    if (!clear_words(p, ws, true, Clear::kAll, st)) return FLAREPP_ERR_CUDA;
     auto mark = [&](int i) {
         return !events || cudaEventRecord((cudaEvent_t)events[i], st) == cudaSuccess;
     };
@@ -611,7 +615,7 @@ flarepp_status mixer_impl(const flarepp_shape* shape, int n_proj, const void* X,
     // forward keeps Y and the chain's state in `saved`.
     void* Y = saved ? saved + ms.off_y : ws + L.off_y;
     stt = route_impl(shape, seeds, proj[2], proj[3], proj[0], proj[1], scale, Y, workspace,
-                     p.total, stream, nullptr, nullptr, nullptr, 0, false, saved);
+                     p.total, stream, nullptr, nullptr, nullptr, 0, Clear::kNone, saved);
     if (stt != FLAREPP_OK) return stt;
     // O = merge(Y) Wo^T
     if (!mark(2) ||

@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                    const GemmParams prm) {
     using C = GCfg<D, MODE>;
     constexpr int kS = C::kStages;
+    pdl_trigger();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align_shared<1024>(smem_raw);
     uint8_t* staging = smem + kS * C::kStage;  // [kEpiGroups][kStaging]
@@ -185,6 +186,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = warp_uniform(*tmem_slot);
+    // every global access below may depend on the kernel before this one
+    pdl_wait();
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
@@ -405,9 +408,8 @@ cudaError_t launch(const CUtensorMap* a, const CUtensorMap& b, const CUtensorMap
     const cudaError_t attr = ensure_smem_limit((const void*)tc_gemm_kernel<D, MODE>, Cf::kSmem);
     if (attr != cudaSuccess) return attr;
     const int64_t grid = prm.n_tiles < sms ? prm.n_tiles : sms;
-    tc_gemm_kernel<D, MODE><<<(unsigned)grid, kThreads, Cf::kSmem, st>>>(
-        a[0], a[1], a[2], a[3], b, o[0], o[1], o[2], o[3], prm);
-    return cudaGetLastError();
+    return launch_pdl(tc_gemm_kernel<D, MODE>, dim3((unsigned)grid), dim3(kThreads), Cf::kSmem, st,
+                      a[0], a[1], a[2], a[3], b, o[0], o[1], o[2], o[3], prm);
 }
 
 template <int MODE>

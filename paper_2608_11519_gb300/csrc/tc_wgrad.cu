@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const WgParams prm) {
     using W = WCfg<D>;
     constexpr int kS = W::kStages;
+    pdl_trigger();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align_shared<1024>(smem_raw);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kS * W::kStage);
@@ -180,6 +181,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = warp_uniform(*tmem_slot);
+    // every global access below may depend on the kernel before this one
+    pdl_wait();
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
@@ -323,6 +326,8 @@ __global__ void __launch_bounds__(32 * kReduceWarps)
     wgrad_reduce_kernel(const float* __restrict__ part, int64_t n_chunks, int64_t R, int64_t Cc,
                         int64_t R_out, int fold, __nv_bfloat16* __restrict__ out) {
     __shared__ float4 sums[kReduceWarps][32];
+    pdl_trigger();
+    pdl_wait();
     const int w = threadIdx.x / 32, lane = threadIdx.x & 31;
     const int64_t i = ((int64_t)blockIdx.x * 32 + lane) * 4;  // Cc is a multiple of 16
     const bool in = i < R_out * Cc;
@@ -441,9 +446,8 @@ cudaError_t launch(const CUtensorMap* ma, const CUtensorMap* mb, const WgParams&
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t grid = prm.n_items < sms ? prm.n_items : sms;
-    tc_wgrad_kernel<D><<<(unsigned)grid, kThreads, Wc::kSmem, st>>>(
-        ma[0], ma[1], ma[2], ma[3], mb[0], mb[1], mb[2], mb[3], prm);
-    return cudaGetLastError();
+    return launch_pdl(tc_wgrad_kernel<D>, dim3((unsigned)grid), dim3(kThreads), Wc::kSmem, st, ma[0],
+                      ma[1], ma[2], ma[3], mb[0], mb[1], mb[2], mb[3], prm);
 }
 
 }  // namespace
@@ -524,9 +528,8 @@ cudaError_t tc_wgrad(int64_t B, int64_t N, int64_t H, int64_t D, const WgradSour
     }
     if (e != cudaSuccess) return e;
     const int64_t n = R_out * Cc;
-    wgrad_reduce_kernel<<<(unsigned)((n + 127) / 128), 32 * kReduceWarps, 0, st>>>(
-        part, w.n_chunks, R, Cc, R_out, fold, (__nv_bfloat16*)dW);
-    return cudaGetLastError();
+    return launch_pdl(wgrad_reduce_kernel, dim3((unsigned)((n + 127) / 128)), dim3(32 * kReduceWarps),
+                      0, st, (const float*)part, w.n_chunks, R, Cc, R_out, fold, (__nv_bfloat16*)dW);
 }
 
 }  // namespace flarepp
