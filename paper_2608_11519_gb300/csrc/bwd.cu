@@ -704,10 +704,11 @@ __global__ void __launch_bounds__(256)
     }
 }
 
-// The tensor-core path (bf16 inputs): c3, the bf16 operand copies of Q and Z, then
-// R3 -> reduce (dZ, the decoder's dQ, c2) -> T23 (dK, dV) and R2 -> reduce (dQ, c1) ->
-// T1 (dKt, dVt) and R1 -> reduce (dseeds). For D <= 32, T23 runs merged (T23C) for every
-// (b, h) whose statistics allow it and unmerged for the rest.
+// The tensor-core path (bf16 inputs): the prologue, then R3 -> reduce (dZ, the decoder's dQ, c2) ->
+// T23 (dK, dV) and R2 -> reduce (dQ, c1) -> T1 (dKt, dVt) and R1 -> reduce (dseeds). For D <= 32,
+// T23 runs merged (T23C) for every (b, h) whose statistics allow it and unmerged for the rest; and
+// where the routes fit (tok_max_routes), dZ comes from an encode and the token passes of tc_tok.cu
+// form dQ and dseeds as well: R3, T23 and R2 then run for the flagged (b, h) alone.
 template <int D>
 cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, const void* Kt,
                            const void* Vt, const void* K, const void* V, float scale,

@@ -73,7 +73,7 @@ struct GemmParams {
     int64_t B, N, H, C;
     int n_a;            // MODE 1: A tensors side by side (the contraction runs over n_a * C)
     int64_t n_out;      // output channels (P * C, or C)
-    int NT;             // output channels per tile (whole heads, <= 256, divides C)
+    int NT;             // output channels per tile (whole heads, <= 256, divides n_out)
     uint32_t idesc;     // MMA instruction descriptor for M = 128, N = NT
     int64_t row_tiles;  // 128-token tiles per batch element
     int64_t pair;       // row tiles per work tile (1 or 2)
