@@ -14,8 +14,8 @@
 // The contraction over C runs in slices of D channels (one head), the unit that both A
 // layouts share; each slice is one TMA box of 128 tokens x D for A and NT channels x D for B,
 // swizzled to the D-wide row. A work tile is 128 tokens (of one batch element), or 256 as two row
-// tiles that share B's slices (MODE 1), x NT output channels; persistent CTAs walk the tiles with the channel tile varying fastest, so the CTAs
-// that share a token tile run together and read it from L2.
+// tiles that share B's slices (MODE 1), x NT output channels; persistent CTAs walk the tiles with the
+// channel tile varying fastest, so the CTAs that share a token tile run together and read it from L2.
 //
 // Roles (12 warps): warp 0 the TMA producer, warp 1 the MMA issuer (one elected lane; one
 // commit per slice frees its ring stage, one per tile hands the accumulator over), warps 4..11
