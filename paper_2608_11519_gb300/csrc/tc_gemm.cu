@@ -475,7 +475,8 @@ cudaError_t tc_projection(int64_t B, int64_t N, int64_t H, int64_t D, int P, con
     prm.n_out = P * C;
     prm.NT = tile_channels(P * H, D);  // a tile may span projections
     prm.idesc = idesc_bf16_f32(kRows, prm.NT, false, false);
-    for (int p = 0; p < 4; ++p) prm.out[p] = (__nv_bfloat16*)outs[p < P ? p : p - 2];
+    // the kernel takes four store maps whatever P is: those beyond P repeat the first ones, unused
+    for (int p = 0; p < 4; ++p) prm.out[p] = (__nv_bfloat16*)outs[p % P];
     prm.status = status;
     CUtensorMap ma[4], mb, mo[4];
     if (!make_map(&ma[0], X, D, C, N, B, kRows) ||
