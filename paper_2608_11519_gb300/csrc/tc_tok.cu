@@ -545,10 +545,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                    (s == 1 || !o.first || o.tc < 2 ||
                     wait(accfree0 + 8u * (o.tc & 1u), (o.tc >> 1) - 1));
         };
-        // the segment before has given dQ back
+        // the segment before has given dQ back (the fence orders its TMEM reads before the product
+        // that starts dQ afresh in the same columns)
         auto wait_dq = [&]() {
-            return !(o.fresh && o.first) || n_fresh++ == 0 ||
-                   wait(segfree0 + 8u * ((n_fresh - 2) & 1u), (n_fresh - 2) >> 1);
+            if (!(o.fresh && o.first) || n_fresh++ == 0) return true;
+            if (!wait(segfree0 + 8u * ((n_fresh - 2) & 1u), (n_fresh - 2) >> 1)) return false;
+            tc_fence_after();
+            return true;
         };
         bool ok = true, fresh = true;
         uint32_t tc = 0;
