@@ -6,6 +6,8 @@
 //   calls 3 and 2 (CALL1 false), with u = 2^(L3 - R), w = 2^(R - L2) for the shift R of the
 //     (b, h) (the two calls' probabilities differ by the rank-one factor P2 / P3 = u w):
 //       S = K Q^T,  T = [dY | u V] [Z | w dZ]^T,  P3 = 2^(c S - L3),
+//     (u V as a bf16 pair hi + lo: V is exact in bf16, and with u V rounded once more dQ, and with it
+//     dseeds, dKt and dVt, would be further off than with V itself: dVt's error by 17 to 40 %)
 //       dS = P3 (T - c3 - u (w c2)),  E2 = P3 u
 //       dK += dS Q,   dV += E2 (w dZ),   dQ += dS^T K (calls 3 and 2 together)
 //   call 1:
@@ -22,8 +24,8 @@
 //
 // Two streams share a token tile: stream s takes the route items s, s + 2, ..., so that the dS
 // tiles of items 2b and 2b + 1 (block b) lie next to each other and one product of 128 routes
-// serves both. Each stream has its own score tiles, item ring and two warpgroups of 32 columns
-// each; dK and dV are shared, with two accumulators by the parity of the tile.
+// serves both. Each stream has its own score tiles and two warpgroups of 32 columns each; the item ring
+// and dK and dV are shared, the latter with two accumulators by the parity of the tile.
 // Roles (20 warps): warp 0 issues every product, warp 3 loads (TMA) the token tiles, the items and
 // the per-route statistics; warps 4..19 are the softmax warpgroups (stream w / 2, columns
 // 32 (w % 2) ..). One issuer serves the streams in turn: for a stream's item it issues S, the dV
@@ -67,10 +69,14 @@ struct TokCfg {
     static constexpr int kNT = CALL1 ? 2 : 3;        // token tiles: K, V (, dY) / Kt, Vt
     static constexpr int kNI = kNT + (LO ? 1 : 0);   // item tiles: Q, w dZ, Z (, lo) / Qs, dQ
     static constexpr int kATile = kRows * D * 2;
-    static constexpr int kABytes = kNT * kATile;
+    // (calls 3 and 2: u V leaves its tile as a bf16 pair, the lo part in a tile behind the loaded ones)
+    static constexpr int kABytes = (kNT + (CALL1 ? 0 : 1)) * kATile;
     static constexpr int kItemTile = kItem * D * 2;
     static constexpr int kStage = kNI * kItemTile;
-    static constexpr int kStages = 3;                // ring stages per stream
+    // ring stages, taken by the items of both streams in turn: at D = 32 the pair of u V leaves room
+    // for five in calls 3 and 2 (two a stream: the training step of 262,144 tokens, M = 512, 2165 us
+    // instead of 2104; u V rounded once, with three a stream, 2055)
+    static constexpr int kStages = D == 32 && !CALL1 ? 5 : 6;
     static constexpr int kDsTile = kRows * kItem * 2;
     static constexpr int kMaxM = (int)tok_max_routes(D);
     static constexpr uint32_t kSwz = D == 16 ? kSw32 : kSw64;
@@ -80,15 +86,15 @@ struct TokCfg {
     static constexpr uint32_t kColAcc = 4 * kItem;
     static constexpr uint32_t kColQ = kColAcc + 4 * D;
     static_assert(kColQ + (kMaxM / 128) * D <= kTmemCols, "TMEM budget");
-    // shared memory: dS [buffer][stream], token tiles [2], rings [stream][stage], statistics
+    // shared memory: dS [buffer][stream], token tiles [2], the ring, statistics
     // [segment parity][2][kMaxM], barriers
     static constexpr int kOffA = 4 * kDsTile;
     static constexpr int kOffRing = kOffA + 2 * kABytes;
-    static constexpr int kOffStat = kOffRing + 2 * kStages * kStage;
+    static constexpr int kOffStat = kOffRing + kStages * kStage;
     static constexpr int kOffBars = kOffStat + 4 * kMaxM * 4;
-    // full[2][stages], empty[2][stages], afull[2], aready[2], afree[2], sready[2], pready[2],
+    // full[stages], empty[stages], afull[2], aready[2], afree[2], sready[2], pready[2],
     // accdone[2], accfree[2], statfull[2], segfree[2], dqdone, fin
-    static constexpr int kNumBars = 4 * kStages + 18 + 2;
+    static constexpr int kNumBars = 2 * kStages + 18 + 2;
     static constexpr int kNeed = 1024 + kOffBars + kNumBars * 8 + 16;
     static constexpr int kSmem = kNeed > 122880 ? kNeed : 122880;  // one CTA per SM
     static_assert(kSmem <= 232448, "shared memory budget");
@@ -287,9 +293,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::kNumBars);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const uint32_t full0 = smem_u32(bars);          // [stream][stage]
-    const uint32_t empty0 = full0 + 16u * kS;       // [stream][stage]
-    const uint32_t afull0 = empty0 + 16u * kS;
+    const uint32_t full0 = smem_u32(bars);  // [stage]
+    const uint32_t empty0 = full0 + 8u * kS;  // [stage]
+    const uint32_t afull0 = empty0 + 8u * kS;
     const uint32_t aready0 = afull0 + 16u;
     const uint32_t afree0 = aready0 + 16u;
     const uint32_t sready0 = afree0 + 16u;
@@ -305,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
-        for (int k = 0; k < 2 * kS; ++k) {
+        for (int k = 0; k < kS; ++k) {
             mbar_init(full0 + 8u * k, 1);
             mbar_init(empty0 + 8u * k, 1);
         }
@@ -350,11 +356,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 
     if (warp == 3) {
         // ------------------------------------------------------------ TMA producer
-        uint32_t tc = 0, seg = 0, is0 = 0, is1 = 0;  // tiles, segments, items per stream
-        int64_t loaded = 0;
+        uint32_t tc = 0, seg = 0, it = 0;  // tiles, segments, items
         int prev_bh = -1;
-        int withheld_s = -1;
-        uint32_t withheld_i = 0;
+        int64_t withheld = -1;
         bool ok = true;
         for (TileIt T(prm); T.valid() && ok; T.next(), ++tc) {
             if (T.bh != prev_bh) {
@@ -391,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const uint32_t bar = afull0 + 8u * ab;
                 const uint32_t dst = smem_u32(abuf + ab * C::kABytes);
                 const int row = T.tile * kRows;
-                mbar_expect_tx(bar, C::kABytes);
+                mbar_expect_tx(bar, C::kNT * C::kATile);
                 tma_load_3d(dst, &tmA0, 0, row, T.bh, bar);
                 tma_load_3d(dst + C::kATile, &tmA1, 0, row, T.bh, bar);
                 if (!CALL1) tma_load_3d(dst + 2 * C::kATile, &tmA2, 0, row, T.bh, bar);
@@ -399,25 +403,19 @@ __global__ void __launch_bounds__(kThreads, 1)
             __syncwarp();
             const int z0 = (int)(prm.i0_per_head ? T.bh % prm.H : T.bh);
             for (int i = 0; i < prm.n_items; ++i) {
-                const int s = i & 1;
-                const uint32_t n = s == 0 ? is0 : is1;
-                const uint32_t st = n % kS;
-                if (n >= (uint32_t)kS && !wait(empty0 + 8u * (s * kS + st), n / kS - 1)) {
+                const uint32_t st = it % kS;
+                if (it >= (uint32_t)kS && !wait(empty0 + 8u * st, it / kS - 1)) {
                     ok = false;
                     break;
                 }
-                if (s == 0)
-                    ++is0;
-                else
-                    ++is1;
-                if (blockIdx.x == 0 && loaded++ == prm.withhold_it) {
-                    withheld_s = s;  // never loaded: the waits of its consumers run out
-                    withheld_i = n;
+                if (blockIdx.x == 0 && it == prm.withhold_it) {
+                    withheld = it++;  // never loaded: the waits of its consumers run out
                     continue;
                 }
+                ++it;
                 if (elect_one()) {
-                    const uint32_t bar = full0 + 8u * (s * kS + st);
-                    const uint32_t dst = smem_u32(ring + (s * kS + st) * C::kStage);
+                    const uint32_t bar = full0 + 8u * st;
+                    const uint32_t dst = smem_u32(ring + st * C::kStage);
                     const int row = i * kItem;
                     mbar_expect_tx(bar, C::kStage);
                     tma_load_3d(dst, &tmI0, 0, row, z0, bar);
@@ -433,15 +431,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!ok) {
             // after an abort: wait (bounded) until the newest copy of every buffer has landed
             const uint64_t w0 = globaltimer_ns();
-            for (int s = 0; s < 2; ++s)
-                for (uint32_t st = 0; st < (uint32_t)kS && st < (s == 0 ? is0 : is1); ++st) {
-                    const uint32_t n = s == 0 ? is0 : is1;
-                    const uint32_t x = n - 1 - ((n - 1 - st) % kS);
-                    while (!(s == withheld_s && x == withheld_i) &&
-                           !mbar_try_wait(full0 + 8u * (s * kS + st), (x / kS) & 1) &&
-                           globaltimer_ns() - w0 < prm.wait_ns) {
-                    }
+            for (uint32_t st = 0; st < (uint32_t)kS && st < it; ++st) {
+                const uint32_t x = it - 1 - ((it - 1 - st) % kS);  // the newest item in this stage
+                while (x != withheld && !mbar_try_wait(full0 + 8u * st, (x / kS) & 1) &&
+                       globaltimer_ns() - w0 < prm.wait_ns) {
                 }
+            }
             // (the token tiles issued are those of the tiles before tc, and perhaps tc itself)
             for (uint32_t b = 0; b < 2 && b < tc; ++b) {
                 const uint32_t x = tc - 1 - ((tc - 1 - b) & 1u);
@@ -462,19 +457,19 @@ __global__ void __launch_bounds__(kThreads, 1)
             bool fresh;                 // the first tile of its segment: dQ starts afresh
             uint32_t tc, st0, st1;      // its tile; ring stages of its items
         } o{};
-        uint32_t is0 = 0, is1 = 0;  // items per stream
+        uint32_t it = 0;            // items
+        uint32_t is0 = 0, is1 = 0;  // and per stream
         uint32_t bg = 0;            // blocks
         uint32_t n_fresh = 0;       // segments whose dQ products have begun
         // Stream s's turn: S and T of its item in stage st of token buffer ab (if `has`), and the
         // dV and dK products of its item of the block before (if `owed`).
         auto turn = [&](int s, bool has, uint32_t st, uint32_t ab, bool owed) {
             const uint32_t t0 = tmem + s * 2 * kItem;
-            const uint32_t ring_s = ring_u + s * kS * C::kStage;
             const uint32_t a = smem_desc_lo(a_u + ab * C::kABytes, 16);
-            const uint32_t i = smem_desc_lo(ring_s + st * C::kStage, 16);
+            const uint32_t i = smem_desc_lo(ring_u + st * C::kStage, 16);
             const uint32_t o_st = s == 0 ? o.st0 : o.st1;
             const uint32_t acc = tmem + C::kColAcc + (o.tc & 1u) * 2 * D;
-            const uint32_t im = smem_desc_lo(ring_s + o_st * C::kStage, C::kItemTile);
+            const uint32_t im = smem_desc_lo(ring_u + o_st * C::kStage, C::kItemTile);
             const bool start = o.first && s == 0;  // the products that start dK and dV
             if (has) {
 #pragma unroll
@@ -504,8 +499,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                     mma_ss(t0 + kItem, desc_of(a1 + 2 * k, kHi), desc_of(i1 + 2 * k, kHi),
                            C::kIdescS, k > 0 ? 1u : 0u);
                 if (!CALL1) {
-                    const uint32_t a2 = a + ((2 * C::kATile) >> 4);
+                    const uint32_t a2 = a + ((2 * C::kATile) >> 4), al = a + ((3 * C::kATile) >> 4);
                     const uint32_t i2 = i + ((2 * C::kItemTile) >> 4);
+#pragma unroll
+                    for (int k = 0; k < D / 16; ++k)
+                        mma_ss(t0 + kItem, desc_of(al + 2 * k, kHi), desc_of(i1 + 2 * k, kHi),
+                               C::kIdescS, 1u);
 #pragma unroll
                     for (int k = 0; k < D / 16; ++k)
                         mma_ss(t0 + kItem, desc_of(a2 + 2 * k, kHi), desc_of(i2 + 2 * k, kHi),
@@ -520,7 +519,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int k = 0; k < kItem / 16; ++k)  // dK += dS Q
                     mma_ss(acc, desc_of(ds + 2 * k, kHiDs), desc_of(im + 2 * D * k, kHi),
                            C::kIdescAcc, (!start || k > 0) ? 1u : 0u);
-                mma_commit(empty0 + 8u * (s * kS + o_st));
+                mma_commit(empty0 + 8u * o_st);
             }
         };
         // dQ += dS^T K of the block before, and what it frees.
@@ -562,20 +561,21 @@ __global__ void __launch_bounds__(kThreads, 1)
             const bool seg_end = T.last_of_segment();
             for (uint32_t b = 0; b < nb; ++b) {
                 const bool has1 = 2 * (int)b + 1 < prm.n_items;
-                const uint32_t st0 = is0 % kS, st1 = is1 % kS;
-                ok = wait(full0 + 8u * st0, is0 / kS) && (!o.any || wait_owed(0));
+                const uint32_t st0 = it % kS, st1 = (it + 1) % kS;
+                ok = wait(full0 + 8u * st0, it / kS) && (!o.any || wait_owed(0));
                 if (!ok) break;
                 tc_fence_after();
                 if (elect_one()) turn(0, true, st0, ab, o.any);
                 __syncwarp();
                 ++is0;
-                ok = (!has1 || wait(full0 + 8u * (kS + st1), is1 / kS)) &&
+                ok = (!has1 || wait(full0 + 8u * st1, (it + 1) / kS)) &&
                      (!(o.any && o.two) || wait_owed(1));
                 if (!ok) break;
                 tc_fence_after();
                 if (elect_one()) turn(1, has1, st1, ab, o.any && o.two);
                 __syncwarp();
                 if (has1) ++is1;
+                it += has1 ? 2 : 1;
                 if (o.any) {
                     ok = wait_dq();
                     if (!ok) break;
@@ -619,8 +619,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint8_t* ds_row = ds_buf + s * C::kDsTile + r * (kItem * 2);
         uint32_t seg = 0, is = 0, bg = 0, nprep = 0;
         bool ok = true;
-        // Calls 3 and 2: this row's statistics of a tile, and (all 512 threads) u V over V in its
-        // shared-memory tile: thread (w, r) takes 16-byte chunk w of row r.
+        // Calls 3 and 2: this row's statistics of a tile, and (all 512 threads) the pair u V over V
+        // in its shared-memory tile and in the one behind dY's: thread (w, r) takes 16-byte chunk w
+        // of row r.
         // load_row fetches the row's statistics (L3, c3, R) ahead.
         auto load_row = [&](const TileIt& T) -> RowStats {
             RowStats rs{0.f, 0.f, INFINITY};
@@ -645,15 +646,21 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int sw = ((r * D * 2) >> 7) & (D / 8 - 1);
                     uint4* p = reinterpret_cast<uint4*>(abuf + ab * C::kABytes + C::kATile +
                                                         r * D * 2) + (w ^ sw);
-                    uint4 v = *p;
+                    uint4 v = *p, lo;
                     uint32_t* x = reinterpret_cast<uint32_t*>(&v);
+                    uint32_t* y = reinterpret_cast<uint32_t*>(&lo);
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const float2 f =
                             __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&x[e]));
-                        x[e] = pack_bf16(f.x * rs.u, f.y * rs.u);
+                        const float a = f.x * rs.u, b = f.y * rs.u;
+                        x[e] = pack_bf16(a, b);
+                        const float2 g =
+                            __bfloat1622float2(*reinterpret_cast<__nv_bfloat162*>(&x[e]));
+                        y[e] = pack_bf16(a - g.x, b - g.y);
                     }
                     *p = v;
+                    p[2 * C::kATile / 16] = lo;
                     fence_proxy_async();
                 }
                 if (ok) mbar_arrive(aready0 + 8u * ab);
