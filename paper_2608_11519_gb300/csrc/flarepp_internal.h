@@ -248,6 +248,7 @@ void test_fault_for(int kernel, uint64_t* wait_ns, int64_t* ring_item);
 // Rows per tensor-core work unit (route group of the encode, token group of the decode).
 int64_t tc_group_rows(int64_t D);
 int64_t tc_encode_item_rows(int64_t D);  // tokens per item of the tensor-core encode
+int64_t tc_decode_item_rows(int64_t D, int64_t M, bool lo);  // routes per item of the decode
 // dZ = P3^T dY of the backward (D = 16 and 32), P3 = 2^(scale log2(e) <q, k> - L3) with Q as its hi
 // and lo operands: an encode whose partials [BH][nchunk * sub_per_chunk][M][D] are plain sums.
 cudaError_t tc_dz_pass(const Plan& p, const void* Qhi, const void* Qlo, const void* K,

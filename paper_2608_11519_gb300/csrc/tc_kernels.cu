@@ -79,8 +79,8 @@ constexpr float kFastLimit = 281474976710656.0f;  // 2^48
 // shared-memory A buffer (the lo tile after the hi tile); the decode's items carry Q's lo tile
 // as a third tile.
 // COL (the backward's dZ, an encode): every item also carries its tokens' L3.
-// DEC: 0 the encode, else a form of the decode: kNarrow with 64-route items and, at D <= 32, two O
-// accumulators per stream, kWide with items as wide as 512 TMEM columns allow beside one O.
+// DEC: 0 the encode, else a form of the decode: kNarrow with 64-route items and two O accumulators per
+// stream (48 and one at D = 64), kWide with items as wide as 512 TMEM columns allow beside one O.
 constexpr int kNarrow = 1, kWide = 2;
 template <int D, int DEC, bool LO = false, bool COL = false>
 struct Cfg {
@@ -99,12 +99,14 @@ struct Cfg {
     // A tiles are double-buffered so the next unit's land during this one. Its narrow form keeps
     // two O accumulators per stream, one per unit parity, so that a unit's epilogue can wait until
     // the next unit's first item is under way.
-    // Which decode: the wide one when it takes fewer items per unit (launch_d). Decode of
+    // Which decode: the wide one when it takes fewer items per unit (tc_decode_item_rows). Decode of
     // 8 x 262,144 tokens, narrow / wide: D = 32, M = 128 74 / 76 us, M = 512 209 / 199, M = 2048
-    // 734 / 678; D = 16, M = 64 47 / 49, M = 512 201 / 184. At D = 64 (narrow: one O either way)
-    // 48 -> 64 routes an item: M = 512 276 -> 254, M = 128 139 -> 127. With Q's lo tiles (the
-    // training forward) the narrow one is faster at every M: D = 32, M = 512 218 / 233.
-    static constexpr int kItem = D == 64 || DEC == kNarrow ? 64 : (D == 16 ? 112 : 96);
+    // 734 / 678; D = 16, M = 64 47 / 49, M = 512 201 / 184; D = 64, M = 512 276 / 254, M = 128
+    // 139 / 127. With as many items either way the wide one only adds columns: 8 x 65,536 tokens,
+    // D = 64, M = 144 38 / 45 us. With Q's lo tiles (the training forward) the narrow one is faster at
+    // every M: D = 32, M = 512 218 / 233.
+    static constexpr int kItem = D == 64 ? (DEC == kNarrow ? 48 : 64)
+                                         : (DEC == kNarrow ? 64 : (D == 16 ? 112 : 96));
     static constexpr int B = 1;                         // score buffers per stream
     // shared-memory A buffers (four for the decode at small M measured no faster than two)
     static constexpr int kABufS = DEC ? 2 : 1;
@@ -121,11 +123,11 @@ struct Cfg {
     // route tiles gives each stream one token parity) looks ahead only kStages / n_par of its
     // own items, and the copy of its next item cannot start before the stream frees the stage
     // kStages items back; so the encode takes as many stages as shared memory holds, up to 16.
-    // The decode's streams take every item, and 8 stages cover the copy latency (6 at D = 64, what
-    // shared memory leaves beside the A buffers).
+    // The decode's streams take every item, and 8 stages cover the copy latency (6 in the wide form at
+    // D = 64, what shared memory leaves beside the A buffers).
     static constexpr int kStat = COL ? kItem * 4 : 0;  // bytes of an item's column statistics
     static constexpr int kStagesFit = (232448 - 2048 - kABufS * kABytes) / (kStage + kStat);
-    static constexpr int kStages = DEC ? (D == 64 ? 6 : 8) : (kStagesFit < 16 ? kStagesFit : 16);
+    static constexpr int kStages = DEC ? (D == 64 && DEC == kWide ? 6 : 8) : (kStagesFit < 16 ? kStagesFit : 16);
     // barriers: full[S], empty[S], a_full[kABufS] (a unit's A tiles landed), a_free[kABufS]
     //           (one arrive per softmax warpgroup once it has seen the unit's last S: the
     //           buffer may be refilled), sync[NS][2] = {s_ready, o_done} per stream (S of an
@@ -1132,8 +1134,7 @@ cudaError_t launch_d(int64_t D, bool lo, const CUtensorMap& a, const CUtensorMap
     switch (D) {
         case 16: return launch<16, DEC, false>(a, b, c, l, prm, st);
         case 32: return launch<32, DEC, false>(a, b, c, l, prm, st);
-        case 64:  // (the wide decode is the narrow one there)
-            return launch<64, DEC != 0 ? kNarrow : 0, false>(a, b, c, l, prm, st);
+        case 64: return launch<64, DEC, false>(a, b, c, l, prm, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -1148,6 +1149,14 @@ uint32_t item_rows(int64_t D, bool lo = false) {
 }
 
 int64_t tc_encode_item_rows(int64_t D) { return item_rows<0>(D); }
+
+// The wide form when its units have fewer items, but not with Q's lo tiles.
+int64_t tc_decode_item_rows(int64_t D, int64_t M, bool lo) {
+    const int64_t narrow = item_rows<kNarrow>(D, lo);
+    if (lo) return narrow;
+    const int64_t wide = item_rows<kWide>(D);
+    return cdiv(M, wide) < cdiv(M, narrow) ? wide : narrow;
+}
 
 void test_fault_for(int kernel, uint64_t* wait_ns, int64_t* ring_item) {
     std::lock_guard<std::mutex> lock(g_fault_mu);
@@ -1216,10 +1225,8 @@ cudaError_t tc_decode(const Plan& p, const void* K, float scale, void* Y, char* 
                       cudaStream_t st, float* lse, bool lo, const void* Qh) {
     CUtensorMap ma, mb, mc, ml;
     lo = lo && p.D <= 32;
-    // the wide form when its units have fewer items, but not with Q's lo tiles
-    const int64_t narrow = item_rows<kNarrow>(p.D, lo), wide = item_rows<kWide>(p.D, lo);
-    const bool use_wide = !lo && cdiv(p.M, wide) < cdiv(p.M, narrow);
-    const uint32_t item = (uint32_t)(use_wide ? wide : narrow);
+    const uint32_t item = (uint32_t)tc_decode_item_rows(p.D, p.M, lo);
+    const bool use_wide = !lo && item == item_rows<kWide>(p.D);
     if (!make_map(&ma, K, p.D, p.N, p.BH, kTileRows) ||
         !make_map(&mb, Qh ? Qh : ws + p.off_qop, p.D, p.M, Qh ? p.H : p.BH,
                   item) ||
