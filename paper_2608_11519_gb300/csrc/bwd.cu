@@ -34,8 +34,6 @@ constexpr int kRoute = 16;  // routes staged per step of a token pass
 
 __device__ __forceinline__ float ld_f32(const float* p) { return *p; }
 __device__ __forceinline__ float ld_f32(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-__device__ __forceinline__ void st_out(float* p, float x) { *p = x; }
-__device__ __forceinline__ void st_out(__nv_bfloat16* p, float x) { *p = __float2bfloat16_rn(x); }
 
 __device__ __forceinline__ float ex2(float x) {
     float y;
@@ -161,7 +159,92 @@ __global__ void __launch_bounds__(128, D == 16 ? 4 : 2) route_pass_kernel(
     }
 }
 
-// Reduce of the route passes' partials, one warp per latent row, chunks in ascending order.
+// ---- reduces of partial sums. A row's slots are shared out to `ways` groups of D / 4 threads (four
+// channels a thread; reduce_ways), way w adding the slots w, w + ways, ... in ascending order; the ways'
+// sums are then added in way order.
+template <int D>
+unsigned reduce_blocks(int64_t rows, int ways) {
+    const int64_t per_block = kRedThreads / ways / (D / 4);
+    return (unsigned)((rows + per_block - 1) / per_block);
+}
+// This thread's row, channel group and way.
+template <int D>
+struct RedThread {
+    int64_t row;
+    int g, way;
+    __device__ __forceinline__ explicit RedThread(int ways) {
+        const int per = kRedThreads / ways, i = (int)threadIdx.x % per;
+        way = (int)threadIdx.x / per;
+        row = (int64_t)blockIdx.x * (per / (D / 4)) + i / (D / 4);
+        g = i % (D / 4);
+    }
+};
+__device__ __forceinline__ void add4(float4& a, float4 v) {
+    a.x += v.x;
+    a.y += v.y;
+    a.z += v.z;
+    a.w += v.w;
+}
+// The sum over the slots that next() gives, one after the other (null: no more); four loads in flight.
+template <typename Next>
+__device__ __forceinline__ float4 sum_slots(Next next) {
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (;;) {
+        const float4* p[4];
+        float4 v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) p[e] = next();
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = p[e] ? *p[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) add4(a, v[e]);
+        if (!p[3]) return a;
+    }
+}
+// The ways' sums added in way order: valid in the threads of way 0. Every thread of the block calls it.
+__device__ __forceinline__ float4 add_ways(float4 a, int ways, float4* sums) {
+    if (ways == 1) return a;
+    const int per = kRedThreads / ways;
+    sums[threadIdx.x] = a;
+    __syncthreads();
+    if ((int)threadIdx.x < per)
+        for (int k = 1; k < ways; ++k) add4(a, sums[threadIdx.x + k * per]);
+    __syncthreads();
+    return a;
+}
+__device__ __forceinline__ float4 scaled(float s, float4 a) {
+    return make_float4(s * a.x, s * a.y, s * a.z, s * a.w);
+}
+// four floats as four bf16 and back
+__device__ __forceinline__ uint2 pack4(float4 v) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y);
+    const __nv_bfloat162 hi = __floats2bfloat162_rn(v.z, v.w);
+    return make_uint2(*reinterpret_cast<const uint32_t*>(&lo),
+                      *reinterpret_cast<const uint32_t*>(&hi));
+}
+__device__ __forceinline__ float4 unpack4(uint2 p) {
+    const float2 f0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&p.x));
+    const float2 f1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&p.y));
+    return make_float4(f0.x, f0.y, f1.x, f1.y);
+}
+__device__ __forceinline__ void st_out4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void st_out4(__nv_bfloat16* p, float4 v) {
+    *reinterpret_cast<uint2*>(p) = pack4(v);
+}
+__device__ __forceinline__ float dot4(float4 a, float4 b) {
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, a.x * b.x)));
+}
+// the sum of x over a row's T threads (adjacent lanes)
+template <int T>
+__device__ __forceinline__ float row_sum(float x) {
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned mask = ((1u << T) - 1u) << (lane & ~(unsigned)(T - 1));
+#pragma unroll
+    for (int off = T / 2; off > 0; off >>= 1) x += __shfl_xor_sync(mask, x, off);
+    return x;
+}
+
+// Reduce of the route passes' partials.
 //   MODE 3: dZ = sum pa, dQ = s sum pb, c2 = <dZ, Z>
 //   MODE 2: dQ += s sum pb, c1 = <dQ, Q>
 //   MODE 1: dseeds[h, m] = s sum_b sum_chunks pb (rows = H * M)
@@ -169,77 +252,59 @@ __global__ void __launch_bounds__(128, D == 16 ? 4 : 2) route_pass_kernel(
 // then taken from that copy: the passes of call 1 form dP = dQ K~^T from the bf16 dQ, and
 // dS = P (dP - c1) cancels for a nearly one-hot P only when c1 = <dQ, Q> uses the same dQ.
 template <int D, typename T, int MODE>
-__global__ void bwd_reduce_kernel(const float* __restrict__ pa, const float* __restrict__ pb,
-                                  int64_t rows, int64_t B, int64_t H, int64_t M, int64_t nchunk,
-                                  float scale, const float* __restrict__ O,
-                                  float* __restrict__ dz, float* __restrict__ dq,
-                                  float* __restrict__ cout, T* __restrict__ dseeds,
-                                  __nv_bfloat16* __restrict__ op) {
-    constexpr int PER = (D + 31) / 32;
-    const int lane = threadIdx.x & 31;
-    const int64_t row = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    if (row >= rows) return;
-    float sa[PER], sb[PER];
-#pragma unroll
-    for (int i = 0; i < PER; ++i) sa[i] = sb[i] = 0.f;
-    if (MODE == 1) {
-        const int64_t h = row / M, m = row % M;
-        for (int64_t b = 0; b < B; ++b)
-#pragma unroll 8
-            for (int64_t c = 0; c < nchunk; ++c) {
-                const int64_t r = ((b * H + h) * nchunk + c) * M + m;
-#pragma unroll
-                for (int i = 0; i < PER; ++i) {
-                    const int d = lane + 32 * i;
-                    if (d < D) sb[i] += pb[r * D + d];
-                }
+__global__ void __launch_bounds__(kRedThreads)
+    bwd_reduce_kernel(const float* __restrict__ pa, const float* __restrict__ pb, int64_t rows,
+                      int64_t B, int64_t H, int64_t M, int64_t nchunk, int ways, float scale,
+                      const float* __restrict__ O, float* __restrict__ dz, float* __restrict__ dq,
+                      float* __restrict__ cout, T* __restrict__ dseeds,
+                      __nv_bfloat16* __restrict__ op) {
+    __shared__ float4 sums[kRedThreads];
+    const RedThread<D> t(ways);
+    const bool in = t.row < rows;
+    const int64_t bh = in ? t.row / M : 0, m = in ? t.row % M : 0;  // MODE 1: the head
+    const int64_t st = M * (D / 4);
+    const auto slots = [&](const float* part) {
+        int64_t b = in ? 0 : B, c = t.way;
+        return sum_slots([=]() mutable -> const float4* {
+            if (MODE != 1) {
+                if (!in || c >= nchunk) return nullptr;
+            } else {
+                for (; b < B && c >= nchunk; ++b) c -= nchunk;
+                if (b >= B) return nullptr;
             }
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int d = lane + 32 * i;
-            if (d < D) st_out(dseeds + row * D + d, scale * sb[i]);
-        }
+            const int64_t slot = (MODE == 1 ? b * H + bh : bh) * nchunk + c;
+            c += ways;
+            return reinterpret_cast<const float4*>(part) + slot * st + m * (D / 4) + t.g;
+        });
+    };
+    const float4 sb = add_ways(slots(pb), ways, sums);
+    float4 sa = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (MODE == 3) sa = add_ways(slots(pa), ways, sums);
+    if (!in || t.way != 0) return;
+    const int64_t at = t.row * D + 4 * t.g;
+    if (MODE == 1) {
+        st_out4(dseeds + at, scaled(scale, sb));
         return;
     }
-    const int64_t bh = row / M, m = row % M;
-#pragma unroll 8
-    for (int64_t c = 0; c < nchunk; ++c) {
-        const int64_t r = (bh * nchunk + c) * M + m;
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int d = lane + 32 * i;
-            if (d < D) {
-                sb[i] += pb[r * D + d];
-                if (MODE == 3) sa[i] += pa[r * D + d];
-            }
+    const float4 o = *reinterpret_cast<const float4*>(O + at);
+    float4 v = scaled(scale, sb);
+    float dot;
+    if (MODE == 3) {
+        st_out4(dz + at, sa);
+        st_out4(dq + at, v);
+        if (op) st_out4(op + at, sa);
+        dot = dot4(sa, o);
+    } else {
+        add4(v, *reinterpret_cast<const float4*>(dq + at));
+        st_out4(dq + at, v);
+        if (op) {
+            st_out4(op + at, v);
+            v = unpack4(pack4(v));
         }
+        dot = dot4(v, o);
     }
-    float dot = 0.f;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const int d = lane + 32 * i;
-        if (d < D) {
-            if (MODE == 3) {
-                dz[row * D + d] = sa[i];
-                dq[row * D + d] = scale * sb[i];
-                dot = fmaf(sa[i], O[row * D + d], dot);
-                if (op) op[row * D + d] = __float2bfloat16_rn(sa[i]);
-            } else {
-                const float v = dq[row * D + d] + scale * sb[i];
-                dq[row * D + d] = v;
-                float vc = v;
-                if (op) {
-                    const __nv_bfloat16 vb = __float2bfloat16_rn(v);
-                    op[row * D + d] = vb;
-                    vc = __bfloat162float(vb);
-                }
-                dot = fmaf(vc, O[row * D + d], dot);
-            }
-        }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-    if (lane == 0) cout[row] = dot;
+    dot = row_sum<D / 4>(dot);
+    if (t.g == 0) cout[t.row] = dot;
 }
 
 // Token pass, float32; two threads per R tokens n, every route streamed.
@@ -374,7 +439,10 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, co
     const int route_threads = (int)bp.m_tile;
     const unsigned token_blocks =
         (unsigned)((two_tokens ? (p.N + 127) / 128 : (p.N + 63) / 64) * p.BH);
-    const unsigned red_blocks = (unsigned)((lat_rows + 7) / 8);
+    const int64_t seed_rows = p.H * p.M;
+    const int ways = reduce_ways(lat_rows, D, bp.nchunk);
+    const int seed_ways = reduce_ways(seed_rows, D, p.B * bp.nchunk);
+    const unsigned red_blocks = reduce_blocks<D>(lat_rows, ways);
 
     launch_delta_tokens<D, float>(dY, Y, tok_rows, c3, st);
     const auto route = [&](auto kernel, const float* a, int per_head, const float* k,
@@ -395,27 +463,26 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, co
     // call 3: dZ and the decoder's dQ
     if ((e = route(route_pass_kernel<D, 3>, Q32, 0, K, dY, Z32, none, none)) != cudaSuccess)
         return e;
-    bwd_reduce_kernel<D, float, 3><<<red_blocks, 256, 0, st>>>(pa, pb, lat_rows, p.B, p.H, p.M,
-                                                               bp.nchunk, scale, Z32, dz, dq, c2,
-                                                               nullptr, nullptr);
+    bwd_reduce_kernel<D, float, 3><<<red_blocks, kRedThreads, 0, st>>>(
+        pa, pb, lat_rows, p.B, p.H, p.M, bp.nchunk, ways, scale, Z32, dz, dq, c2, nullptr, nullptr);
     // calls 3 and 2: dK and dV per token
     if ((e = token(two_tokens ? token_pass_kernel<D, 23, kTwo> : token_pass_kernel<D, 23, 1>, K, V,
                    dY, Q32, 0, dz, Z32, L2, c2, dK, dV)) != cudaSuccess)
         return e;
     // call 2: the encoder's dQ, added to the decoder's
     if ((e = route(route_pass_kernel<D, 2>, Q32, 0, K, V, dz, L2, c2)) != cudaSuccess) return e;
-    bwd_reduce_kernel<D, float, 2><<<red_blocks, 256, 0, st>>>(nullptr, pb, lat_rows, p.B, p.H, p.M,
-                                                               bp.nchunk, scale, Q32, nullptr, dq,
-                                                               c1, nullptr, nullptr);
+    bwd_reduce_kernel<D, float, 2><<<red_blocks, kRedThreads, 0, st>>>(
+        nullptr, pb, lat_rows, p.B, p.H, p.M, bp.nchunk, ways, scale, Q32, nullptr, dq, c1, nullptr,
+        nullptr);
     // call 1: dKt, dVt per token, then the seeds' gradient
     if ((e = token(two_tokens ? token_pass_kernel<D, 1, kTwo> : token_pass_kernel<D, 1, 1>, Kt, Vt,
                    none, seeds, 1, dq, none, L1, c1, dKt, dVt)) != cudaSuccess)
         return e;
     if ((e = route(route_pass_kernel<D, 1>, seeds, 1, Kt, Vt, dq, L1, c1)) != cudaSuccess) return e;
-    const int64_t seed_rows = p.H * p.M;
-    bwd_reduce_kernel<D, float, 1><<<(unsigned)((seed_rows + 7) / 8), 256, 0, st>>>(
-        nullptr, pb, seed_rows, p.B, p.H, p.M, bp.nchunk, scale, nullptr, nullptr, nullptr,
-        nullptr, dseeds, nullptr);
+    bwd_reduce_kernel<D, float, 1>
+        <<<reduce_blocks<D>(seed_rows, seed_ways), kRedThreads, 0, st>>>(
+            nullptr, pb, seed_rows, p.B, p.H, p.M, bp.nchunk, seed_ways, scale, nullptr, nullptr,
+            nullptr, nullptr, dseeds, nullptr);
     return cudaGetLastError();
 }
 
@@ -425,22 +492,6 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, co
 // whenever max_n L3 - R and max_m L2 - R do; a (b, h) outside that range (scores spread
 // over more than ~60 binary orders) is flagged and runs the unmerged T23 pass instead.
 constexpr float kMergeRange = 60.f;
-
-// four floats as four bf16 and back
-__device__ __forceinline__ uint2 pack4(float4 v) {
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y);
-    const __nv_bfloat162 hi = __floats2bfloat162_rn(v.z, v.w);
-    return make_uint2(*reinterpret_cast<const uint32_t*>(&lo),
-                      *reinterpret_cast<const uint32_t*>(&hi));
-}
-__device__ __forceinline__ float dot4(float4 a, float4 b) {
-    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, a.x * b.x)));
-}
-__device__ __forceinline__ float4 unpack4(uint2 p) {
-    const float2 f0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&p.x));
-    const float2 f1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&p.y));
-    return make_float4(f0.x, f0.y, f1.x, f1.y);
-}
 
 // part[bh][j] for j < parts: max of L3 over slice j of the tokens; part[bh][kRangeParts] and
 // [kRangeParts + 1]: min and max of L2 (from slice 0's block). One block per (bh, j), block `id`.
@@ -553,15 +604,6 @@ __global__ void merge_flags_kernel(const float* __restrict__ part, int parts, in
     if (bh < BH) merge_flag(part, parts, bh, BH, Rb, flags);
 }
 
-// the sum of x over a row's T threads (adjacent lanes)
-template <int T>
-__device__ __forceinline__ float row_sum(float x) {
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned mask = ((1u << T) - 1u) << (lane & ~(unsigned)(T - 1));
-#pragma unroll
-    for (int off = T / 2; off > 0; off >>= 1) x += __shfl_xor_sync(mask, x, off);
-    return x;
-}
 // The merged pass's route operand w dZ: W[bh][m][:] = bf16(2^(R[bh] - L2[bh][m]) dZ[bh][m][:]), and
 // c2 taken from it: c2w = <W, Z> / w. The pass forms w dP2 = W V^T, and dS2 = P2 (dP2 - c2)
 // cancels for a nearly one-hot P2 only when c2 sees the same rounded dZ. v, z: this thread's four
@@ -590,117 +632,114 @@ __global__ void __launch_bounds__(256)
                      W, c2w);
 }
 
-// dZ from the partial sums of tc_dz_pass, slot by slot in order (a chunk's token-parity parts as
-// the encode's plan cuts them: 4, 2 or 1 by the route tiles of the row's group of 512): its bf16
-// copy, c2 = <dZ, Z>, and the merged pass's operand; and the (b, h)'s shift and flag. D / 4
-// threads per row, four loads in flight.
+// dZ from the partial sums of tc_dz_pass (a chunk's token-parity parts as the encode's plan cuts them: 4,
+// 2 or 1 by the route tiles of the row's group of 512): its bf16 copy, c2 = <dZ, Z>, and the merged
+// pass's operand; and the (b, h)'s shift and flag.
 template <int D>
-__global__ void __launch_bounds__(256)
-    dz_reduce_kernel(const float* __restrict__ part, int M, int nchunk, int64_t rows,
+__global__ void __launch_bounds__(kRedThreads)
+    dz_reduce_kernel(const float* __restrict__ part, int M, int nchunk, int64_t rows, int ways,
                      const float* __restrict__ Z, const float* __restrict__ L2,
                      const float* __restrict__ rpart, int parts, float* __restrict__ Rb,
                      int* __restrict__ flags, __nv_bfloat16* __restrict__ dzb,
                      float* __restrict__ c2, __nv_bfloat16* __restrict__ W,
                      float* __restrict__ c2w) {
-    constexpr int T = D / 4;
+    __shared__ float4 sums[kRedThreads];
     tc::pdl_trigger();
     tc::pdl_wait();
-    const int64_t row = ((int64_t)blockIdx.x * 256 + threadIdx.x) / T;  // bh * M + m
-    const int g = threadIdx.x % T;
-    if (row >= rows) return;  // (rows in whole groups of T threads)
-    const int64_t bh = row / M;
-    const int m = (int)(row - bh * M);
-    if (m == 0 && g == 0) merge_flag(rpart, parts, bh, rows / M, Rb, flags);
+    const RedThread<D> t(ways);
+    const bool in = t.row < rows;
+    const int64_t bh = in ? t.row / M : 0;  // row = bh * M + m
+    const int m = in ? (int)(t.row - bh * M) : 0;
+    if (in && m == 0 && t.g == 0 && t.way == 0) merge_flag(rpart, parts, bh, rows / M, Rb, flags);
     const int left = M - (m & ~511);
     const int ul = left > 256 ? 0 : (left > 128 ? 1 : 2);  // log2 of the parts per chunk
-    const int n = nchunk << ul, mask = (1 << ul) - 1;
-    const float4* p = reinterpret_cast<const float4*>(part + (bh * nchunk * 4 * M + m) * D) + g;
-    const int64_t st = (int64_t)M * T;
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = 0; s0 < n; s0 += 4) {
-        float4 v[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int s = s0 + e;
-            v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (s < n) v[e] = p[((int64_t)(s >> ul) * 4 + (s & mask)) * st];
-        }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            a.x += v[e].x;
-            a.y += v[e].y;
-            a.z += v[e].z;
-            a.w += v[e].w;
-        }
-    }
-    const float4 z = reinterpret_cast<const float4*>(Z + row * D)[g];
-    reinterpret_cast<uint2*>(dzb + row * D)[g] = pack4(a);
-    const float dot = row_sum<T>(dot4(a, z));
-    if (g == 0) c2[row] = dot;
-    merge_operand<D>(a, z, rpart[bh * (kRangeParts + 2) + kRangeParts] - L2[row], row, g, W, c2w);
+    const int n = in ? nchunk << ul : 0, mask = (1 << ul) - 1;
+    const float4* p = reinterpret_cast<const float4*>(part + (bh * nchunk * 4 * M + m) * D) + t.g;
+    const int64_t st = (int64_t)M * (D / 4);
+    int s = t.way;
+    float4 a = sum_slots([=]() mutable -> const float4* {
+        if (s >= n) return nullptr;
+        const float4* q = p + ((int64_t)(s >> ul) * 4 + (s & mask)) * st;
+        s += ways;
+        return q;
+    });
+    a = add_ways(a, ways, sums);
+    if (!in || t.way != 0) return;
+    const int64_t at = t.row * D + 4 * t.g;
+    const float4 z = *reinterpret_cast<const float4*>(Z + at);
+    st_out4(dzb + at, a);
+    const float dot = row_sum<D / 4>(dot4(a, z));
+    if (t.g == 0) c2[t.row] = dot;
+    merge_operand<D>(a, z, rpart[bh * (kRangeParts + 2) + kRangeParts] - L2[t.row], t.row, t.g, W,
+                     c2w);
 }
 
-// Reduce of the partials dS^T K that the token passes of tc_tok.cu leave, a CTA's slot each:
-// T = D / 4 threads per route row (four channels each), slots in CTA order.
+// Reduce of the partials dS^T K that the token passes of tc_tok.cu leave, a CTA's slot each, in CTA
+// order.
 //   DSEEDS false: dQ = s sum (of the flagged (b, h) s times the sum of the route passes' partials,
 //     pb of R3 and pa of R2, nchunk each), as bf16, and c1 = <dQ, Q> from that copy (as
 //     bwd_reduce_kernel's MODE 2)
 //   DSEEDS true: dseeds[h, m] = s sum over the batch and the slots (rows = H * M)
-// Four loads are in flight per thread.
 template <int D, bool DSEEDS>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kRedThreads)
     tok_reduce_kernel(const float* __restrict__ part, int64_t rows, int64_t B, int64_t H, int64_t M,
-                      int64_t nt, int64_t tiles, int64_t ctas, int64_t slots, float scale,
+                      int64_t nt, int64_t tiles, int64_t ctas, int64_t slots, int ways, float scale,
                       const int* __restrict__ flags, const float* __restrict__ pb,
                       const float* __restrict__ pa, int64_t nchunk, const float* __restrict__ Q,
                       float* __restrict__ c1, __nv_bfloat16* __restrict__ op) {
-    constexpr int T = D / 4;
+    __shared__ float4 sums[kRedThreads];
     tc::pdl_trigger();
     tc::pdl_wait();
-    const int64_t row = ((int64_t)blockIdx.x * 256 + threadIdx.x) / T;
-    const int g = threadIdx.x % T;
-    if (row >= rows) return;  // (rows in whole groups of T threads)
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto add = [&](const float* base, int64_t n, int64_t stride) {
-        const float4* p = reinterpret_cast<const float4*>(base) + g;
-        const int64_t st = stride / 4;
-        int64_t k = 0;
-        for (; k + 4 <= n; k += 4) {
-            const float4 v0 = p[k * st], v1 = p[(k + 1) * st], v2 = p[(k + 2) * st],
-                         v3 = p[(k + 3) * st];
-            a.x += v0.x; a.y += v0.y; a.z += v0.z; a.w += v0.w;
-            a.x += v1.x; a.y += v1.y; a.z += v1.z; a.w += v1.w;
-            a.x += v2.x; a.y += v2.y; a.z += v2.z; a.w += v2.w;
-            a.x += v3.x; a.y += v3.y; a.z += v3.z; a.w += v3.w;
-        }
-        for (; k < n; ++k) {
-            const float4 v = p[k * st];
-            a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
-        }
+    const RedThread<D> t(ways);
+    const bool in = t.row < rows;
+    const int64_t hb = in ? t.row / M : 0, m = in ? t.row % M : 0;  // DSEEDS: the head, else bh
+    const int64_t st = M * (D / 4);
+    // the slots of (b, h): one per CTA whose run of tiles reaches it
+    const auto count = [=](int64_t bh) {
+        return ((bh + 1) * nt * ctas - 1) / tiles - ((bh * nt + 1) * ctas - 1) / tiles + 1;
     };
-    auto add_slots = [&](int64_t bh, int64_t m) {
-        const int64_t c0 = ((bh * nt + 1) * ctas - 1) / tiles;
-        const int64_t c1_ = (((bh + 1) * nt) * ctas - 1) / tiles;
-        add(part + (bh * slots * M + m) * D, c1_ - c0 + 1, M * D);
+    const auto at_slot = [=](const float* base, int64_t slot) {
+        return reinterpret_cast<const float4*>(base) + slot * st + m * (D / 4) + t.g;
     };
-    if constexpr (DSEEDS) {
-        const int64_t h = row / M, m = row % M;
-        for (int64_t b = 0; b < B; ++b) add_slots(b * H + h, m);
-        reinterpret_cast<uint2*>(op + row * D)[g] =
-            pack4(make_float4(scale * a.x, scale * a.y, scale * a.z, scale * a.w));
+    float4 a;
+    if (DSEEDS) {
+        int64_t b = 0, s = t.way, n = in ? count(hb) : 0;
+        a = sum_slots([=]() mutable -> const float4* {
+            while (s >= n) {  // on to the next batch element
+                s -= n;
+                if (!in || ++b >= B) {
+                    n = 0;
+                    s = 0;
+                    return nullptr;
+                }
+                n = count(b * H + hb);
+            }
+            const float4* q = at_slot(part, (b * H + hb) * slots + s);
+            s += ways;
+            return q;
+        });
     } else {
-        const int64_t bh = row / M, m = row % M;
-        if (flags == nullptr || flags[bh] == 0) {
-            add_slots(bh, m);
-        } else {
-            add(pb + (bh * nchunk * M + m) * D, nchunk, M * D);
-            add(pa + (bh * nchunk * M + m) * D, nchunk, M * D);
-        }
-        const uint2 pk = pack4(make_float4(scale * a.x, scale * a.y, scale * a.z, scale * a.w));
-        reinterpret_cast<uint2*>(op + row * D)[g] = pk;
+        const bool flagged = flags != nullptr && in && flags[hb] != 0;
+        const int64_t n = !in ? 0 : (flagged ? 2 * nchunk : count(hb));
+        int64_t s = t.way;
+        a = sum_slots([=]() mutable -> const float4* {
+            if (s >= n) return nullptr;
+            const float4* q = !flagged ? at_slot(part, hb * slots + s)
+                              : s < nchunk ? at_slot(pb, hb * nchunk + s)
+                                           : at_slot(pa, hb * nchunk + s - nchunk);
+            s += ways;
+            return q;
+        });
+    }
+    a = add_ways(a, ways, sums);
+    if (!in || t.way != 0) return;
+    const int64_t at = t.row * D + 4 * t.g;
+    const uint2 pk = pack4(scaled(scale, a));
+    *reinterpret_cast<uint2*>(op + at) = pk;
+    if (!DSEEDS) {
         const float dot =
-            row_sum<T>(dot4(unpack4(pk), reinterpret_cast<const float4*>(Q + row * D)[g]));
-        if (g == 0) c1[row] = dot;
+            row_sum<D / 4>(dot4(unpack4(pk), *reinterpret_cast<const float4*>(Q + at)));
+        if (t.g == 0) c1[t.row] = dot;
     }
 }
 
@@ -741,7 +780,7 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
     const int64_t tok_rows = p.BH * p.N;
     const int64_t lat_rows = p.BH * p.M;
     const int64_t lat = lat_rows * p.D;
-    const unsigned red_blocks = (unsigned)((lat_rows + 7) / 8);
+    const int64_t seed_rows = p.H * p.M;
     cudaError_t e;
 
     constexpr bool kMerged = D <= 32;
@@ -777,15 +816,20 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
             float* pz = (float*)(ws + bp.off_pz);
             float* pt = (float*)(ws + bp.off_pt);
             const int64_t tiles = bp.tok_nt * p.BH;
-            const auto blocks = [](int64_t rows) { return (unsigned)((rows * (D / 4) + 255) / 256); };
+            // (the slots that rows have at most: four token parities a chunk; the CTAs' in all)
+            const int ways_z = reduce_ways(lat_rows, D, p.nchunk * 4);
+            const int ways_q = reduce_ways(lat_rows, D, bp.tok_slots);
+            const int ways_s = reduce_ways(seed_rows, D, bp.tok_slots * p.B);
+            const dim3 threads(kRedThreads);
             r3.flags = r2.flags = flags;
             r3.want = r2.want = 1;
             r3.any = r2.any = flags + p.BH;
             r2.pb = pa;
             if ((e = tc_dz_pass(p, qb, qlo, K, dY, L3, scale, pz, status, st)) != cudaSuccess)
                 return e;
-            if ((e = launch_pdl(dz_reduce_kernel<D>, dim3(blocks(lat_rows)), dim3(256), 0, st,
-                                (const float*)pz, (int)p.M, (int)p.nchunk, lat_rows, Z32, L2,
+            if ((e = launch_pdl(dz_reduce_kernel<D>, dim3(reduce_blocks<D>(lat_rows, ways_z)), threads,
+                                0, st, (const float*)pz, (int)p.M, (int)p.nchunk, lat_rows, ways_z,
+                                Z32, L2,
                                 (const float*)rpart, parts, Rb, flags, dzb, c2, wop, c2w)) !=
                 cudaSuccess)
                 return e;
@@ -794,27 +838,31 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
             if ((e = tc_bwd_pass(p, bp, 0, r3, scale, status, st)) != cudaSuccess) return e;
             if ((e = tc_bwd_pass(p, bp, 3, t23, scale, status, st)) != cudaSuccess) return e;
             if ((e = tc_bwd_pass(p, bp, 1, r2, scale, status, st)) != cudaSuccess) return e;
-            if ((e = launch_pdl(tok_reduce_kernel<D, false>, dim3(blocks(lat_rows)), dim3(256), 0, st,
+            if ((e = launch_pdl(tok_reduce_kernel<D, false>,
+                                dim3(reduce_blocks<D>(lat_rows, ways_q)), threads, 0, st,
                                 (const float*)pt, lat_rows, p.B, p.H, p.M, bp.tok_nt, tiles,
-                                bp.tok_ctas, bp.tok_slots, scale, (const int*)flags,
+                                bp.tok_ctas, bp.tok_slots, ways_q, scale, (const int*)flags,
                                 (const float*)pb, (const float*)pa, bp.nchunk, Q32, c1, dqb)) !=
                 cudaSuccess)
                 return e;
             t = TokOperands{{Kt, Vt, Vt}, {seeds, dqb, dqb}, nullptr, nullptr, nullptr, L1, c1,
                             nullptr, nullptr, pt, dKt, dVt};
             if ((e = tc_tok_pass(p, bp, true, t, scale, status, st)) != cudaSuccess) return e;
-            return launch_pdl(tok_reduce_kernel<D, true>, dim3(blocks(p.H * p.M)), dim3(256), 0, st,
-                              (const float*)pt, p.H * p.M, p.B, p.H, p.M, bp.tok_nt, tiles,
-                              bp.tok_ctas, bp.tok_slots, scale, (const int*)nullptr,
+            return launch_pdl(tok_reduce_kernel<D, true>,
+                              dim3(reduce_blocks<D>(seed_rows, ways_s)), threads, 0, st,
+                              (const float*)pt, seed_rows, p.B, p.H, p.M, bp.tok_nt, tiles,
+                              bp.tok_ctas, bp.tok_slots, ways_s, scale, (const int*)nullptr,
                               (const float*)nullptr, (const float*)nullptr, (int64_t)0,
                               (const float*)nullptr, (float*)nullptr, (T*)dseeds);
         }
     }
     TcBwdOperands o{};
     if ((e = tc_bwd_pass(p, bp, 0, r3, scale, status, st)) != cudaSuccess) return e;
-    bwd_reduce_kernel<D, T, 3><<<red_blocks, 256, 0, st>>>(pa, pb, lat_rows, p.B, p.H, p.M,
-                                                           bp.nchunk, scale, Z32, dz, dq, c2,
-                                                           nullptr, dzb);
+    const int ways = reduce_ways(lat_rows, D, bp.nchunk);
+    const int seed_ways = reduce_ways(seed_rows, D, p.B * bp.nchunk);
+    const unsigned red_blocks = reduce_blocks<D>(lat_rows, ways);
+    bwd_reduce_kernel<D, T, 3><<<red_blocks, kRedThreads, 0, st>>>(
+        pa, pb, lat_rows, p.B, p.H, p.M, bp.nchunk, ways, scale, Z32, dz, dq, c2, nullptr, dzb);
     if constexpr (kMerged) {
         merge_operand_kernel<D><<<(unsigned)((lat / 4 + 255) / 256), 256, 0, st>>>(
             dz, Z32, L2, Rb, p.M, lat_rows, wop, c2w);
@@ -828,9 +876,9 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
     }
     if ((e = tc_bwd_pass(p, bp, 3, t23, scale, status, st)) != cudaSuccess) return e;
     if ((e = tc_bwd_pass(p, bp, 1, r2, scale, status, st)) != cudaSuccess) return e;
-    bwd_reduce_kernel<D, T, 2><<<red_blocks, 256, 0, st>>>(nullptr, pb, lat_rows, p.B, p.H, p.M,
-                                                           bp.nchunk, scale, Q32, nullptr, dq, c1,
-                                                           nullptr, dqb);
+    bwd_reduce_kernel<D, T, 2><<<red_blocks, kRedThreads, 0, st>>>(
+        nullptr, pb, lat_rows, p.B, p.H, p.M, bp.nchunk, ways, scale, Q32, nullptr, dq, c1, nullptr,
+        dqb);
     // T1: token rows; S = Kt Qs^T, dP = Vt dQ^T; column statistics L1, c1 -> dKt, dVt
     o = TcBwdOperands{{Kt, Vt, Vt}, {seeds, dqb, dqb}, nullptr, nullptr, L1, c1, nullptr,
                       nullptr, dKt, dVt};
@@ -839,9 +887,8 @@ cudaError_t route_bwd_tc_d(const Plan& p, const BwdPlan& bp, const void* seeds, 
     o = TcBwdOperands{{seeds, dqb, dqb}, {Kt, Vt, Vt}, L1, c1, nullptr, nullptr, nullptr, pb,
                       nullptr, nullptr};
     if ((e = tc_bwd_pass(p, bp, 2, o, scale, status, st)) != cudaSuccess) return e;
-    const int64_t seed_rows = p.H * p.M;
-    bwd_reduce_kernel<D, T, 1><<<(unsigned)((seed_rows + 7) / 8), 256, 0, st>>>(
-        nullptr, pb, seed_rows, p.B, p.H, p.M, bp.nchunk, scale, nullptr, nullptr, nullptr,
+    bwd_reduce_kernel<D, T, 1><<<reduce_blocks<D>(seed_rows, seed_ways), kRedThreads, 0, st>>>(
+        nullptr, pb, seed_rows, p.B, p.H, p.M, bp.nchunk, seed_ways, scale, nullptr, nullptr, nullptr,
         nullptr, (T*)dseeds, nullptr);
     return cudaGetLastError();
 }

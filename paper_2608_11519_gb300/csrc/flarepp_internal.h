@@ -120,6 +120,19 @@ cudaError_t simt_encode_f32(const Plan& p, int call, const void* k, const void* 
 cudaError_t simt_decode_f32(const Plan& p, const void* K, float scale, void* Y, char* ws,
                             cudaStream_t st, float* lse = nullptr, const float* Qh = nullptr);
 
+// Ways that share a row's slots in the reduces of the backward's partial sums (blocks of kRedThreads, D / 4
+// threads to a row and way). One way going through every slot is a chain of loads, and where a shape has
+// few rows and many slots that chain is the whole time (16 routes of one (b, h), 420 slots of dZ: 117 us,
+// with 32 ways 10); so the ways grow until they fill the machine or leave eight slots to a way.
+constexpr int kRedThreads = 256;
+inline int reduce_ways(int64_t rows, int64_t D, int64_t slots) {
+    const int64_t threads = rows * (D / 4);
+    const int most = D == 64 ? 16 : 32;  // a block holds whole rows
+    int ways = 1;
+    while (ways < most && slots > 8 * ways && threads * ways < 2 * kRedThreads * kNumSMs) ways *= 2;
+    return ways;
+}
+
 // ---- backward (bwd.cu): the passes of App. A.5. f32 inputs run on CUDA cores, bf16 inputs
 // on the tensor-core passes of tc_bwd.cu. `saved` is the training forward's state, `ws`
 // the backward workspace; outputs in the input dtype.
