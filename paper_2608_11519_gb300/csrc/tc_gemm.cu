@@ -12,8 +12,8 @@
 //     mixer's backward with B = W_in^T.
 //
 // The contraction over C runs in slices of D channels (one head), the unit that both A
-// layouts share; each slice is one TMA box of 128 tokens x D for A and NT channels x D for B,
-// swizzled to the D-wide row. A work tile is 128 tokens (of one batch element), or 256 as two row
+// layouts share, or of half a head (slice_channels); each slice is one TMA box of 128 tokens x D for A
+// and NT channels x D for B, swizzled to the D-wide row. A work tile is 128 tokens (of one batch element), or 256 as two row
 // tiles that share B's slices (MODE 1), x NT output channels; persistent CTAs walk the tiles with the
 // channel tile varying fastest, so the CTAs that share a token tile run together and read it from L2.
 //
@@ -48,15 +48,22 @@ constexpr int kMaxNT = 256;   // output channels per tile, at most
 constexpr uint64_t kWaitLimitNs = 2000000000ull;
 constexpr uint32_t kTmemCols = 512;
 
+// Channels per slice of the contraction: a head, or half of one where two row tiles beside a head of 64
+// would leave room for two stages only. dX at C = 512, four projections, 65,536 tokens: 128.6 us with
+// whole heads and two stages, 97.3 with halves and five (one row tile and three stages: 115); 10 x 2,000
+// tokens 64.0, 50.1 and 50.5.
+constexpr int slice_channels(int64_t D, int mode) { return mode == 1 && D == 64 ? 32 : (int)D; }
+
 template <int D, int MODE>
 struct GCfg {
-    static constexpr int kASlice = kRows * D * 2;
-    static constexpr int kBSlice = kMaxNT * D * 2;
+    static constexpr int kKD = slice_channels(D, MODE);
+    static constexpr int kASlice = kRows * kKD * 2;
+    static constexpr int kBSlice = kMaxNT * kKD * 2;
     static constexpr int kHalves = MODE == 1 ? 2 : 1;  // row tiles per work tile, at most
     static constexpr int kStage = kHalves * kASlice + kBSlice;
     static constexpr int kStages = (160 * 1024) / kStage > 8 ? 8 : (160 * 1024) / kStage;
-    static constexpr uint32_t kSwz = D == 16 ? kSw32 : (D == 32 ? kSw64 : kSw128);
-    static constexpr uint32_t kSBO = 8 * D * 2;
+    static constexpr uint32_t kSwz = kKD == 16 ? kSw32 : (kKD == 32 ? kSw64 : kSw128);
+    static constexpr uint32_t kSBO = 8 * kKD * 2;
     // per epilogue warpgroup: [128 rows][D] bf16 blocks for TMA stores, as many as its heads of a tile
     static constexpr int kSlots = kMaxNT / 2 / D;
     static constexpr int kStaging = kSlots * kRows * D * 2;
@@ -67,6 +74,7 @@ struct GCfg {
         1024 + kStages * kStage + kEpiGroups * kStaging + kNumBars * 8 + 16;
     static constexpr int kSmem = kNeed > 122880 ? kNeed : 122880;  // one CTA per SM
     static_assert(kSmem <= 232448, "shared memory budget");
+    static_assert(kStages >= 3, "with two stages the loads of a slice wait for the products before it");
 };
 
 struct GemmParams {
@@ -152,7 +160,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t swritten0 = sfree0 + 8u * kEpiGroups;   // [kEpiGroups], count 128
     const int warp = warp_index();
     const int lane = threadIdx.x & 31;
-    const int slices = (int)(prm.C / D) * (MODE == 1 ? prm.n_a : 1);
+    const int slices = (int)(prm.C / C::kKD) * (MODE == 1 ? prm.n_a : 1);
 
     if (threadIdx.x == 0) {
         for (int st = 0; st < kS; ++st) {
@@ -193,7 +201,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // ------------------------------------------------------------ TMA producer
         uint32_t it = 0;
         bool ok = true;
-        const uint32_t b_bytes = (uint32_t)(prm.NT * D * 2);
+        const uint32_t b_bytes = (uint32_t)(prm.NT * C::kKD * 2);
         for (int64_t t = blockIdx.x; t < prm.n_tiles && ok; t += gridDim.x) {
             const GTile T = gtile(prm, t);
             for (int h = 0; h < slices; ++h, ++it) {
@@ -206,14 +214,16 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (elect_one()) {
                     const uint32_t dst = smem_u32(smem + st * C::kStage);
                     mbar_expect_tx(full0 + 8u * st, (uint32_t)(T.halves * C::kASlice) + b_bytes);
-                    // MODE 1: slice h is head h % H of A tensor h / H
-                    const int p = MODE == 0 ? 0 : h / (int)prm.H;
-                    const int z = MODE == 0 ? (int)T.b : (int)(T.b * prm.H + h % (int)prm.H);
+                    // MODE 1: head hd % H of A tensor hd / H, from its channel `part` on
+                    constexpr int kParts = D / C::kKD;
+                    const int hd = h / kParts, part = h % kParts * C::kKD;
+                    const int p = MODE == 0 ? 0 : hd / (int)prm.H;
+                    const int z = MODE == 0 ? (int)T.b : (int)(T.b * prm.H + hd % (int)prm.H);
                     const CUtensorMap* ma = p == 0 ? &tmA : p == 1 ? &tmA1 : p == 2 ? &tmA2 : &tmA3;
                     for (int x = 0; x < (MODE == 0 ? 1 : T.halves); ++x)
-                        tma_load_3d(dst + x * C::kASlice, ma, MODE == 0 ? h * D : 0,
+                        tma_load_3d(dst + x * C::kASlice, ma, MODE == 0 ? h * D : part,
                                     (int)((T.rt + x) * kRows), z, full0 + 8u * st);
-                    tma_load_3d(dst + C::kHalves * C::kASlice, &tmB, h * D, (int)(T.ct * prm.NT), 0,
+                    tma_load_3d(dst + C::kHalves * C::kASlice, &tmB, h * C::kKD, (int)(T.ct * prm.NT), 0,
                                 full0 + 8u * st);
                 }
                 __syncwarp();
@@ -257,7 +267,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const uint32_t acc = tmem + ((seq + x) & 1) * kMaxNT;
                         const uint64_t ad = smem_desc(a0 + x * C::kASlice, 16, C::kSBO, C::kSwz);
 #pragma unroll
-                        for (int k = 0; k < D / 16; ++k)  // 32 bytes on: 2 in the descriptors' units
+                        for (int k = 0; k < C::kKD / 16; ++k)  // 32 bytes on: 2 in the descriptors' units
                             mma_ss(acc, ad + 2 * k, bd + 2 * k, prm.idesc, (h > 0 || k > 0) ? 1u : 0u);
                         if (h == slices - 1) mma_commit(accfull0 + 8u * ((seq + x) & 1));
                     }
@@ -383,18 +393,18 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
-// A bf16 tensor of dims {inner, rows, z} (inner contiguous), boxes of D x box_rows x 1,
-// swizzled to the D-wide row.
-bool make_map(CUtensorMap* m, const void* base, int64_t D, int64_t inner, int64_t rows,
+// A bf16 tensor of dims {inner, rows, z} (inner contiguous), boxes of KD x box_rows x 1,
+// swizzled to the KD-wide row.
+bool make_map(CUtensorMap* m, const void* base, int64_t KD, int64_t inner, int64_t rows,
               int64_t z, uint32_t box_rows) {
     auto fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)rows, (cuuint64_t)z};
     cuuint64_t strides[2] = {(cuuint64_t)(inner * 2), (cuuint64_t)(rows * inner * 2)};
-    cuuint32_t box[3] = {(cuuint32_t)D, box_rows, 1};
+    cuuint32_t box[3] = {(cuuint32_t)KD, box_rows, 1};
     cuuint32_t estr[3] = {1, 1, 1};
-    const CUtensorMapSwizzle sw = D == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
-                                          : (D == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+    const CUtensorMapSwizzle sw = KD == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
+                                          : (KD == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
                                                      : CU_TENSOR_MAP_SWIZZLE_128B);
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
               estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -513,10 +523,11 @@ cudaError_t tc_heads_projection(int64_t B, int64_t N, int64_t H, int64_t D, int 
     prm.out[0] = prm.out[1] = prm.out[2] = prm.out[3] = (__nv_bfloat16*)O;
     prm.status = status;
     CUtensorMap ma[4], mb, mo[4];
+    const int KD = slice_channels(D, 1);
     for (int p = 0; p < 4; ++p)
-        if (!make_map(&ma[p], As[p < n_a ? p : 0], D, D, N, B * H, kRows))
+        if (!make_map(&ma[p], As[p < n_a ? p : 0], KD, D, N, B * H, kRows))
             return cudaErrorInvalidValue;
-    if (!make_map(&mb, W, D, n_a * C, C, 1, (uint32_t)prm.NT) ||
+    if (!make_map(&mb, W, KD, n_a * C, C, 1, (uint32_t)prm.NT) ||
         !make_store_map(&mo[0], O, C, N, B, (uint32_t)D))
         return cudaErrorInvalidValue;
     mo[1] = mo[2] = mo[3] = mo[0];
