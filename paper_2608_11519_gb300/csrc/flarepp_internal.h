@@ -230,7 +230,9 @@ struct WgradSource {
 };
 struct WgradPlan {
     int NT;
-    int64_t row_tiles, row_groups, col_tiles, chunk_len, chunks_per_b, n_chunks;
+    int64_t row_tiles, row_groups, col_tiles;
+    int64_t stages_per_b;         // 64-token stages of a batch element
+    int64_t chunk_len, n_chunks;  // stages per chunk; chunks over the whole batch
     size_t part_bytes;  // float32 partials [n_chunks][R][Cc]
 };
 WgradPlan wgrad_plan(int64_t B, int64_t N, int64_t R, int64_t Cc);

@@ -12,16 +12,16 @@
 //   HEADS: up to four tensors [B*H][N][D] side by side (channel r: tensor r / C, head
 //          (r % C) / D, column r % D), or
 //   PLAIN: one matrix [B][N][C] (channel r: column r).
-// A work item is (256 rows of dW, NT columns of dW, a chunk of one batch element's tokens), the
-// rows as two halves of 128 that share B's tile, each with an accumulator of its own: the reads
+// A work item is (256 rows of dW, NT columns of dW, a chunk of the tokens: a run of 64-token stages that
+// may reach over several batch elements), the rows as two halves of 128 that share B's tile, each with an accumulator of its own: the reads
 // bound the kernel, and with 128 rows every tile of B is fetched twice as often (dW_in of 262,144
 // tokens, C = 256, four projections: 164 -> 128 us; HBM's bytes alone 99). The item writes its
 // float32 partial sum to part[chunk][R][Cc], and a reduce kernel adds the chunks (in a fixed order:
 // deterministic).
 //
 // Roles (8 warps): warp 0 the TMA producer, warp 1 the MMA issuer, warps 4..7 the epilogue
-// (TMEM lane = row of dW). There is about one item per SM, so that nothing is left to overlap an
-// item's epilogue with and the partial sums are few. Every wait is bounded (2 s of %globaltimer), as
+// (TMEM lane = row of dW). There is about one item per SM where the tiles allow (wgrad_plan), so that
+// nothing is left to overlap an item's epilogue with and the partial sums are few. Every wait is bounded (2 s of %globaltimer), as
 // in the other kernels.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -68,14 +68,15 @@ struct WgParams {
     int a_apb, b_apb;      // atoms per TMA box of each operand
     int NT;
     uint32_t idesc;
-    int64_t chunk_len, chunks_per_b, n_chunks;
+    int64_t stages_per_b, stages;  // 64-token stages of a batch element, and of all
+    int64_t chunk_len, n_chunks;   // stages per chunk
     int64_t row_tiles, row_groups, col_tiles, n_items;
     float* part;  // [n_chunks][R][Cc]
     int* status;
 };
 
 struct WItem {
-    int64_t rt, ct, b, n0, n1, chunk;
+    int64_t rt, ct, g0, g1, chunk;  // stages [g0, g1)
     int halves;  // row tiles rt, rt + 1, ... of this item
 };
 
@@ -87,9 +88,8 @@ __device__ __forceinline__ WItem witem(const WgParams& p, int64_t v) {
     w.rt = t / p.col_tiles * kHalves;
     w.halves = (int)min((int64_t)kHalves, p.row_tiles - w.rt);
     w.ct = t % p.col_tiles;
-    w.b = w.chunk / p.chunks_per_b;
-    w.n0 = (w.chunk % p.chunks_per_b) * p.chunk_len;
-    w.n1 = min(p.N, w.n0 + p.chunk_len);
+    w.g0 = w.chunk * p.chunk_len;
+    w.g1 = min(p.stages, w.g0 + p.chunk_len);
     return w;
 }
 
@@ -191,7 +191,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int64_t v = blockIdx.x; v < prm.n_items && ok; v += gridDim.x) {
             const WItem I = witem(prm, v);
             const uint32_t bytes = (uint32_t)(I.halves * W::kAStage + (prm.NT / D) * W::kAtom);
-            for (int64_t n = I.n0; n < I.n1; n += kTok, ++it) {
+            int64_t b = I.g0 / prm.stages_per_b, in_b = I.g0 % prm.stages_per_b;
+            for (int64_t g = I.g0; g < I.g1; ++g, ++it) {
                 const int st = it % kS;
                 if (it >= (uint32_t)kS &&
                     !warp_wait(empty0 + 8u * st, ((it / kS) - 1) & 1, abort_flag, prm.status)) {
@@ -201,15 +202,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (elect_one()) {
                     const uint32_t dst = smem_u32(smem + st * W::kStage);
                     mbar_expect_tx(full0 + 8u * st, bytes);
+                    const int n = (int)(in_b * kTok);
                     for (int x = 0; x < I.halves; ++x)
                         load_atoms<D>(dst + x * W::kAStage, prm.a_heads, &tA0, &tA1, &tA2, &tA3,
-                                      (I.rt + x) * kRowsW, kRowsW, prm.a_apb, prm.C, I.b, (int)n,
+                                      (I.rt + x) * kRowsW, kRowsW, prm.a_apb, prm.C, b, n,
                                       full0 + 8u * st);
                     load_atoms<D>(dst + kHalves * W::kAStage, prm.b_heads, &tB0, &tB1, &tB2, &tB3,
-                                  I.ct * prm.NT, prm.NT, prm.b_apb, prm.C, I.b, (int)n,
-                                  full0 + 8u * st);
+                                  I.ct * prm.NT, prm.NT, prm.b_apb, prm.C, b, n, full0 + 8u * st);
                 }
                 __syncwarp();
+                if (++in_b == prm.stages_per_b) {
+                    in_b = 0;
+                    ++b;
+                }
             }
         }
         if (!ok) {
@@ -233,7 +238,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                      warp_wait(accempty0 + 8u * ((seq + x) & 1), (((seq + x) >> 1) - 1) & 1,
                                abort_flag, prm.status);
             if (!ok) break;
-            for (int64_t n = I.n0; n < I.n1; n += kTok, ++it) {
+            for (int64_t g = I.g0; g < I.g1; ++g, ++it) {
                 const int st = it % kS;
                 if (!warp_wait(full0 + 8u * st, (it / kS) & 1, abort_flag, prm.status)) {
                     ok = false;
@@ -255,7 +260,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                         for (int k = 0; k < kTok / 16; ++k)
                             mma_ss(acc, ad + 2 * D * k, bd + 2 * D * k, prm.idesc,
-                                   (n == I.n0 && k == 0) ? 0u : 1u);
+                                   (g == I.g0 && k == 0) ? 0u : 1u);
                     }
                     mma_commit(empty0 + 8u * st);
                 }
@@ -476,15 +481,28 @@ WgradPlan wgrad_plan(int64_t B, int64_t N, int64_t R, int64_t Cc) {
     w.NT = nt;
     w.row_tiles = (R + kRowsW - 1) / kRowsW;
     w.col_tiles = Cc / nt;
-    // one item per SM (chunks of whole 64-token stages inside one batch element)
+    // The chunk count of least time, in units of a stage (about 1.2 us with every SM at it): waves of
+    // items, each its stages and an epilogue (256 KB of partial sums an item: about 8), and the reduce's
+    // reads of the partial sums (5 for a full wave's). Chunks run over the batch: cut inside a batch
+    // element, 10 of them at C = 512 are 160 items for the four projections on 152 SMs, two waves
+    // (dW_in of 10 x 2,000 tokens 86 us, with chunks over the batch 52).
     w.row_groups = (w.row_tiles + kHalves - 1) / kHalves;
-    const int64_t tiles = w.row_groups * w.col_tiles;
-    int64_t per_b = kNumSMs / (tiles * B);
-    if (per_b < 1) per_b = 1;
-    w.chunk_len = ((N + per_b - 1) / per_b + kTok - 1) / kTok * kTok;
-    if (w.chunk_len < kTok) w.chunk_len = kTok;
-    w.chunks_per_b = (N + w.chunk_len - 1) / w.chunk_len;
-    w.n_chunks = B * w.chunks_per_b;
+    w.stages_per_b = (N + kTok - 1) / kTok;
+    const int64_t tiles = w.row_groups * w.col_tiles, stages = B * w.stages_per_b;
+    double best = 1e300;
+    int64_t n = 0, waves = cdiv(tiles, kNumSMs) - 1;
+    for (int k = 0; k < 6 && n < stages; ++k) {
+        n = ++waves * kNumSMs / tiles;  // the most chunks with these waves
+        if (n > stages) n = stages;
+        const int64_t len = cdiv(stages, n), chunks = cdiv(stages, len);
+        const double cost = (double)cdiv(tiles * chunks, kNumSMs) * ((double)len + 8.0) +
+                            5.0 * (double)(tiles * chunks) / kNumSMs;
+        if (cost < best) {
+            best = cost;
+            w.chunk_len = len;
+            w.n_chunks = chunks;
+        }
+    }
     w.part_bytes = (size_t)w.n_chunks * (size_t)R * (size_t)Cc * sizeof(float);
     return w;
 }
@@ -505,8 +523,9 @@ cudaError_t tc_wgrad(int64_t B, int64_t N, int64_t H, int64_t D, const WgradSour
     prm.b_heads = b.heads;
     prm.NT = w.NT;
     prm.idesc = idesc_bf16_f32(kRowsW, w.NT, true, true);
+    prm.stages_per_b = w.stages_per_b;
+    prm.stages = B * w.stages_per_b;
     prm.chunk_len = w.chunk_len;
-    prm.chunks_per_b = w.chunks_per_b;
     prm.n_chunks = w.n_chunks;
     prm.row_tiles = w.row_tiles;
     prm.col_tiles = w.col_tiles;
