@@ -86,7 +86,7 @@ void launch_delta_tokens(const T* dY, const T* Y, int64_t rows, float* c3, cudaS
 // dS here is P o (dP - c); the factor s is applied by the reduce.
 // grid.x = nchunk * n_mtiles * BH; block = m_tile threads.
 template <int D, int MODE>
-__global__ void __launch_bounds__(128, D == 16 ? 4 : 2) route_pass_kernel(
+__global__ void __launch_bounds__(128, simt_route_warps(D) / 4) route_pass_kernel(
     const float* __restrict__ a, int a_per_head, const float* __restrict__ kb,
     const float* __restrict__ wb, const float* __restrict__ g, const float* __restrict__ Lrow,
     const float* __restrict__ crow, const float* __restrict__ Lcol,

@@ -109,6 +109,14 @@ BwdPlan make_bwd_plan(const Plan& p);
 
 // Routes per thread of the CUDA-core encode: two when a full tile of 128 routes leaves two warps.
 constexpr int simt_encode_rows(int64_t M, int64_t D) { return M >= 128 && D <= 32 ? 2 : 1; }
+// Warps per SM that the registers of the CUDA-core encode (by rows per thread) and of the backward's route
+// passes allow; the kernels' launch bounds hold them to it. A quarter of an SM's registers serves a
+// quarter of its warps: two of 200 registers or more, three of up to 168, four of up to 128.
+constexpr int simt_encode_warps(int rows, int64_t D) { return rows == 2 || D == 16 ? 12 : 8; }
+constexpr int simt_route_warps(int64_t D) { return D == 16 ? 16 : 8; }
+// Fixed scratch of flarepp_route_fwd_noalloc (noalloc.cu).
+constexpr size_t kNoAllocScratchBytes = size_t(64) << 20;
+
 // ---- CUDA-core kernels (simt_kernels.cuh, instantiated in simt_f32.cu), float32 inputs
 // Encode one call over all chunks: call 1 takes the seeds ([H][M][D]), call 2 takes Q32
 // from the workspace. Writes the chunk partials.

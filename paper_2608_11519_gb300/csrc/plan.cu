@@ -17,6 +17,32 @@ constexpr int64_t kMaxTmaCoord = 2147483647 - 4096;  // TMA coordinates are sign
 
 bool mul_ok(int64_t a, int64_t b, int64_t* out) { return !__builtin_mul_overflow(a, b, out); }
 
+// Tokens per chunk of a CUDA-core pass over `tiles` ((b, h), route tile) pairs: the count of least time,
+// in units of a token (about 0.2 us: a CTA's tokens are a chain, as fast alone on an SM as among the
+// `places` CTAs that registers allow there). A wave of CTAs takes its chunk's tokens and about 16 more
+// for rows and partials; the partials' bytes are written and read again (0.56 MB a token); and the
+// merge's chain grows with the chunks. Tried are the largest counts of eight numbers of waves.
+int64_t simt_chunk_len(int64_t N, int64_t tiles, int64_t places, double bytes, double most_bytes,
+                       double per_chunk) {
+    const int64_t full = places * kNumSMs, most = cdiv(N, 16);
+    double best = 1e300;
+    int64_t best_len = most * 16, n = 0, waves = cdiv(tiles, full) - 1;
+    for (int k = 0; k < 8 && n < most; ++k) {
+        n = ++waves * full / tiles;
+        if ((double)n * bytes > most_bytes) n = (int64_t)(most_bytes / bytes);
+        if (n > most) n = most;
+        if (n < 1) n = 1;
+        const int64_t len = cdiv(cdiv(N, n), 16) * 16, chunks = cdiv(N, len);
+        const double cost = (double)cdiv(tiles * chunks, full) * ((double)len + 16.0) +
+                            (double)chunks * (bytes / 0.56e6 + per_chunk);
+        if (cost < best) {
+            best = cost;
+            best_len = len;
+        }
+    }
+    return best_len;
+}
+
 }  // namespace
 
 flarepp_status make_plan(const flarepp_shape* s, Plan* p) {
@@ -44,17 +70,21 @@ flarepp_status make_plan(const flarepp_shape* s, Plan* p) {
     if (bh == 0 || s->N == 0 || s->M == 0) return FLAREPP_OK;  // nothing to plan
 
     if (p->path == kPathSimt) {
-        // CUDA-core encode: up to 128 routes per CTA, one or two per thread; chunks sized so that
-        // the grid is one wave of the CTAs that registers allow per SM (four of 128 threads, six
-        // of 64 with two routes each; two at D = 64).
+        // CUDA-core encode: up to 128 routes per CTA, one or two per thread. The partials stay within
+        // 32 MB, and the whole workspace within the fixed scratch of the call that does not allocate
+        // where one chunk does, so that more chunks never take a shape from that call.
         p->m_tile = s->M >= 128 ? 128 : cdiv(s->M, 32) * 32;
         p->n_mtiles = cdiv(s->M, p->m_tile);
         p->sub_per_chunk = 1;
-        const int64_t target =
-            (simt_encode_rows(s->M, s->D) == 2 ? 6 : (s->D <= 32 ? 4 : 2)) * kNumSMs;
-        int64_t want = target / (bh * p->n_mtiles);
-        if (want < 1) want = 1;
-        p->chunk_len = cdiv(cdiv(s->N, want), 16) * 16;
+        const int rows = simt_encode_rows(s->M, s->D);
+        const double bytes = (double)bh * (double)s->M * (double)(s->D + 2) * 4.0;
+        const double rest = 2.0 * (double)bh * (double)s->M * (double)s->D * 4.0 + 2048.0;
+        const double scratch = (double)kNoAllocScratchBytes;
+        double most = 32.0 * 1048576.0;
+        if (rest - 2048.0 + bytes <= scratch && scratch - rest < most) most = scratch - rest;
+        p->chunk_len = simt_chunk_len(s->N, bh * p->n_mtiles,
+                                      simt_encode_warps(rows, s->D) / (p->m_tile / rows / 32), bytes,
+                                      most, 0.1);
         p->nchunk = cdiv(s->N, p->chunk_len);
     } else {
         // Tensor-core encode: a work unit is (bh, group of <= 512 routes, chunk of tokens) and
@@ -171,11 +201,11 @@ BwdPlan make_bwd_plan(const Plan& p) {
         if (want < 1) want = 1;
         b.chunk_len = cdiv(cdiv(p.N, want), item) * item;
     } else {
-        // one thread per route, up to 128 routes per CTA; chunks for one wave of the CTAs that
-        // registers allow per SM (four, two at D >= 32)
-        int64_t want = (p.D == 16 ? 4 : 2) * kNumSMs / (p.BH * b.n_mtiles);
-        if (want < 1) want = 1;
-        b.chunk_len = cdiv(cdiv(p.N, want), 16) * 16;
+        // one thread per route, up to 128 routes per CTA
+        b.chunk_len = simt_chunk_len(p.N, p.BH * b.n_mtiles,
+                                     simt_route_warps(p.D) / (b.m_tile / 32),
+                                     (double)p.BH * (double)p.M * (double)p.D * 4.0,
+                                     32.0 * 1048576.0, 0.03);
     }
     b.nchunk = cdiv(p.N, b.chunk_len);
     const size_t part = (size_t)p.BH * (size_t)b.nchunk * (size_t)p.M * (size_t)p.D * 4;

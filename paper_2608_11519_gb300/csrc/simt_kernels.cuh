@@ -97,7 +97,7 @@ __device__ __forceinline__ void softmax_tile(const f2 (*q)[D / 2], f2 (*o)[D / 2
 // grid.x = nchunk * n_mtiles * BH; block = m_tile / R threads, thread t with the routes t, t + block,
 // ... of the tile.
 template <int D, int R>
-__global__ void __launch_bounds__(128 / R, R == 2 ? 6 : 1) simt_encode_kernel(
+__global__ void __launch_bounds__(128 / R, simt_encode_warps(R, D) * R / 4) simt_encode_kernel(
     const float* __restrict__ k, const float* __restrict__ v, const float* __restrict__ q,
     int q_per_head, int64_t H, int64_t N, int64_t M, int64_t chunk_len, int64_t nchunk,
     int64_t n_mtiles, float sl2, float* __restrict__ pmax, float* __restrict__ psum,
