@@ -429,16 +429,11 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, co
     const int64_t tok_rows = p.BH * p.N;
     const int64_t lat_rows = p.BH * p.M;
     const unsigned route_blocks = (unsigned)(bp.nchunk * bp.n_mtiles * p.BH);
-    // two tokens per pair of threads where registers allow (8 x 16,384 tokens, M = 128, D = 32: 153 and
-    // 120 us; one token per pair 199 and 128, one per thread 210 and 130), once 128 tokens per block
-    // take both places that registers leave on every SM. One route per thread in the route passes: pairs
-    // with one or two routes are slower (132 or 140 us for call 3, 98 or 93 for calls 2 and 1; this
-    // 108 and 84).
+    // One route per thread in the route passes: pairs of threads with one or two routes are slower (8 x
+    // 16,384 tokens, M = 128, D = 32: 132 or 140 us for call 3, 98 or 93 for calls 2 and 1; this 108 and 84).
     constexpr int kTwo = D <= 32 ? 2 : 1;
-    const bool two_tokens = D <= 32 && ((p.N + 127) / 128) * p.BH >= 2 * kNumSMs;
+    const bool two23 = simt_two_tokens(D, false, p.N, p.BH), two1 = simt_two_tokens(D, true, p.N, p.BH);
     const int route_threads = (int)bp.m_tile;
-    const unsigned token_blocks =
-        (unsigned)((two_tokens ? (p.N + 127) / 128 : (p.N + 63) / 64) * p.BH);
     const int64_t seed_rows = p.H * p.M;
     const int ways = reduce_ways(lat_rows, D, bp.nchunk);
     const int seed_ways = reduce_ways(seed_rows, D, p.B * bp.nchunk);
@@ -451,10 +446,11 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, co
                           per_head, k, w, g, Lr, cr, (const float*)L3, (const float*)c3, p.H, p.N,
                           p.M, bp.chunk_len, bp.nchunk, bp.n_mtiles, sl2, pa, pb);
     };
-    const auto token = [&](auto kernel, const float* k, const float* w, const float* y,
+    const auto token = [&](auto kernel, bool two, const float* k, const float* w, const float* y,
                            const float* a, int per_head, const float* g, const float* z,
                            const float* Lr, const float* cr, float* o0, float* o1) {
-        return launch_pdl(kernel, dim3(token_blocks), dim3(128), 0, st, k, w, y, a, per_head, g, z,
+        const unsigned blocks = (unsigned)((two ? (p.N + 127) / 128 : (p.N + 63) / 64) * p.BH);
+        return launch_pdl(kernel, dim3(blocks), dim3(128), 0, st, k, w, y, a, per_head, g, z,
                           Lr, cr, (const float*)L3, (const float*)c3, p.H, p.N, p.M, sl2, scale, o0,
                           o1);
     };
@@ -466,7 +462,7 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, co
     bwd_reduce_kernel<D, float, 3><<<red_blocks, kRedThreads, 0, st>>>(
         pa, pb, lat_rows, p.B, p.H, p.M, bp.nchunk, ways, scale, Z32, dz, dq, c2, nullptr, nullptr);
     // calls 3 and 2: dK and dV per token
-    if ((e = token(two_tokens ? token_pass_kernel<D, 23, kTwo> : token_pass_kernel<D, 23, 1>, K, V,
+    if ((e = token(two23 ? token_pass_kernel<D, 23, kTwo> : token_pass_kernel<D, 23, 1>, two23, K, V,
                    dY, Q32, 0, dz, Z32, L2, c2, dK, dV)) != cudaSuccess)
         return e;
     // call 2: the encoder's dQ, added to the decoder's
@@ -475,7 +471,7 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, co
         nullptr, pb, lat_rows, p.B, p.H, p.M, bp.nchunk, ways, scale, Q32, nullptr, dq, c1, nullptr,
         nullptr);
     // call 1: dKt, dVt per token, then the seeds' gradient
-    if ((e = token(two_tokens ? token_pass_kernel<D, 1, kTwo> : token_pass_kernel<D, 1, 1>, Kt, Vt,
+    if ((e = token(two1 ? token_pass_kernel<D, 1, kTwo> : token_pass_kernel<D, 1, 1>, two1, Kt, Vt,
                    none, seeds, 1, dq, none, L1, c1, dKt, dVt)) != cudaSuccess)
         return e;
     if ((e = route(route_pass_kernel<D, 1>, seeds, 1, Kt, Vt, dq, L1, c1)) != cudaSuccess) return e;

@@ -114,6 +114,29 @@ constexpr int simt_encode_rows(int64_t M, int64_t D) { return M >= 128 && D <= 3
 // quarter of its warps: two of 200 registers or more, three of up to 168, four of up to 128.
 constexpr int simt_encode_warps(int rows, int64_t D) { return rows == 2 || D == 16 ? 12 : 8; }
 constexpr int simt_route_warps(int64_t D) { return D == 16 ? 16 : 8; }
+
+// The backward's token passes (128 threads; `rows` tokens per pair of threads, one or two): blocks per SM
+// that registers allow (two tokens 130 to 255 registers, one 96 to 168), and whether two are taken.
+constexpr int simt_token_places(int64_t D, int rows, bool call1) {
+    return D == 64 ? 2 : rows == 2 ? (D == 16 ? 3 : 2) : (D == 32 ? 3 : (call1 ? 5 : 4));
+}
+// Two tokens read the staged rows half as often but leave fewer, longer blocks, so a last wave with few
+// of them costs more. A wave's time with two tokens over that with one, measured: D = 16 1.3 (calls 3
+// and 2) and 1.08 (call 1), D = 32 1.0 and 1.19; a last wave takes half that time and the rest by how full
+// it is; and where one token a pair takes one wave, two only make it longer. 8 x 16,384 tokens, M = 128, D = 32: 153 and 119 us with two, 199 and 128 with one (one token per
+// thread 210 and 130); D = 16 89 and 71 against 96 and 73. 60,000 tokens, M = 256, D = 16, 13 blocks beyond
+// a full wave of two: 104 and 84 against 97 and 74. At D = 64 two would spill.
+inline bool simt_two_tokens(int64_t D, bool call1, int64_t N, int64_t BH) {
+    if (D == 64 || cdiv(N, 64) * BH <= simt_token_places(D, 1, call1) * kNumSMs) return false;
+    const auto waves = [&](int64_t tokens, int rows) {
+        const int64_t blocks = cdiv(N, tokens) * BH;
+        const int64_t full = (int64_t)simt_token_places(D, rows, call1) * kNumSMs;
+        const int64_t rest = blocks % full;
+        return (double)(blocks / full) + (rest ? 0.5 + 0.5 * (double)rest / (double)full : 0.0);
+    };
+    const double ratio = D == 16 ? (call1 ? 1.08 : 1.3) : (call1 ? 1.19 : 1.0);
+    return ratio * waves(128, 2) < waves(64, 1);
+}
 // Fixed scratch of flarepp_route_fwd_noalloc (noalloc.cu).
 constexpr size_t kNoAllocScratchBytes = size_t(64) << 20;
 
