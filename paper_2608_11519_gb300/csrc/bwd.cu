@@ -77,16 +77,21 @@ void launch_delta_tokens(const T* dY, const T* Y, int64_t rows, float* c3, cudaS
     delta_tokens_kernel<D, T><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(dY, Y, rows, c3);
 }
 
-// Route pass of call MODE (3, 2 or 1) over one chunk of tokens, float32; thread = route m.
+// Threads per route of the route passes: two at D = 64 in call 3, where one thread's two rows and two sums
+// are 256 registers and spill (868 bytes; 8 x 16,384 tokens, M = 128: 789 us, with two 280).
+constexpr int route_threads(int D, int mode) { return D == 64 && mode == 3 ? 2 : 1; }
+
+// Route pass of call MODE (3, 2 or 1) over one chunk of tokens, float32; thread, or pair, = route m.
 //   MODE 3: a = Q, keys b = K, w = dY, g = Z, column statistics L3[n], c3[n];
 //           pa += P w (dZ), pb += dS k (dQ / s)
 //   MODE 2: a = Q, keys = K, w = V, g = dZ, row statistics L2[m], c2[m]; pb += dS k
 //   MODE 1: a = seeds (per head), keys = Kt, w = Vt, g = dQ, row statistics L1[m], c1[m];
 //           pb += dS kt
 // dS here is P o (dP - c); the factor s is applied by the reduce.
-// grid.x = nchunk * n_mtiles * BH; block = m_tile threads.
+// grid.x = nchunk * n_mtiles * BH; block = m_tile route_threads threads.
 template <int D, int MODE>
-__global__ void __launch_bounds__(128, simt_route_warps(D) / 4) route_pass_kernel(
+__global__ void __launch_bounds__(128 * route_threads(D, MODE),
+                                  simt_route_warps(D) / 4 / route_threads(D, MODE)) route_pass_kernel(
     const float* __restrict__ a, int a_per_head, const float* __restrict__ kb,
     const float* __restrict__ wb, const float* __restrict__ g, const float* __restrict__ Lrow,
     const float* __restrict__ crow, const float* __restrict__ Lcol,
@@ -104,7 +109,9 @@ __global__ void __launch_bounds__(128, simt_route_warps(D) / 4) route_pass_kerne
     bid /= nchunk;
     const int64_t mt = bid % n_mtiles;
     const int64_t bh = bid / n_mtiles;
-    const int64_t m = mt * blockDim.x + threadIdx.x;
+    constexpr int P = route_threads(D, MODE);
+    const int64_t m = (mt * blockDim.x + threadIdx.x) / P;
+    const int h = (int)threadIdx.x % P;
     const bool active = m < M;
     const int64_t mm = active ? m : 0;
     const int64_t n_begin = c * chunk_len;
@@ -120,11 +127,19 @@ __global__ void __launch_bounds__(128, simt_route_warps(D) / 4) route_pass_kerne
     };
     stage(0, n_begin);
 
-    f2 ar[D / 2], gr[D / 2], accA[MODE == 3 ? D / 2 : 1], accB[D / 2];
-    load_row<D>(ar, a + ((a_per_head ? bh % H : bh) * M + mm) * D, sl2, true);
-    load_row<D>(gr, g + (bh * M + mm) * D, 1.f, true);
+    constexpr int W = D / 2 / P;  // packed pairs of channels per thread
+    f2 ar[W], gr[W], accA[MODE == 3 ? W : 1], accB[W];
+    const float* ap = a + ((a_per_head ? bh % H : bh) * M + mm) * D;
+    const float* gp = g + (bh * M + mm) * D;
+    if constexpr (P == 2) {
+        load_half<D>(ar, ap, sl2, h);
+        load_half<D>(gr, gp, 1.f, h);
+    } else {
+        load_row<D>(ar, ap, sl2, true);
+        load_row<D>(gr, gp, 1.f, true);
+    }
 #pragma unroll
-    for (int d = 0; d < D / 2; ++d) {
+    for (int d = 0; d < W; ++d) {
         accB[d] = 0;
         if (MODE == 3) accA[d] = 0;
     }
@@ -143,19 +158,35 @@ __global__ void __launch_bounds__(128, simt_route_warps(D) / 4) route_pass_kerne
         __syncthreads();
 #pragma unroll(D == 64 ? 1 : (MODE == 3 ? 2 : 8))
         for (int j = 0; j < kTok; ++j) {
-            const float x = dot_row<D>(ar, ks[buf][j]);
-            const float dp = dot_row<D>(gr, ws[buf][j]);
-            const float p = j < cnt ? ex2(x - (MODE == 3 ? lc[buf][j] : Lr)) : 0.f;
-            const float ds = p * (dp - (MODE == 3 ? cc[buf][j] : cr));
-            axpy_row<D>(accB, ds, ks[buf][j]);
-            if (MODE == 3) axpy_row<D>(accA, p, ws[buf][j]);
+            const auto weights = [&](float x, float dp, float& p, float& ds) {
+                p = j < cnt ? ex2(x - (MODE == 3 ? lc[buf][j] : Lr)) : 0.f;
+                ds = p * (dp - (MODE == 3 ? cc[buf][j] : cr));
+            };
+            float p, ds;
+            if constexpr (P == 2) {
+                f2 kj[W], wj[W];
+                read_half<D>(kj, ks[buf][j], h);
+                read_half<D>(wj, ws[buf][j], h);
+                weights(dot_half<D>(ar, kj), dot_half<D>(gr, wj), p, ds);
+                axpy_half<D>(accB, ds, kj);
+                if (MODE == 3) axpy_half<D>(accA, p, wj);
+            } else {
+                weights(dot_row<D>(ar, ks[buf][j]), dot_row<D>(gr, ws[buf][j]), p, ds);
+                axpy_row<D>(accB, ds, ks[buf][j]);
+                if (MODE == 3) axpy_row<D>(accA, p, ws[buf][j]);
+            }
         }
         __syncthreads();  // this buffer is staged into again in the next step
     }
     if (active) {
         const int64_t row = (bh * nchunk + c) * M + m;
-        store_row<D>(pb + row * D, accB, 1.f);
-        if (MODE == 3) store_row<D>(pa + row * D, accA, 1.f);
+        if constexpr (P == 2) {
+            store_half<D>(pb + row * D, accB, 1.f, h);
+            if (MODE == 3) store_half<D>(pa + row * D, accA, 1.f, h);
+        } else {
+            store_row<D>(pb + row * D, accB, 1.f);
+            if (MODE == 3) store_row<D>(pa + row * D, accA, 1.f);
+        }
     }
 }
 
@@ -433,16 +464,15 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, co
     // 16,384 tokens, M = 128, D = 32: 132 or 140 us for call 3, 98 or 93 for calls 2 and 1; this 108 and 84).
     constexpr int kTwo = D <= 32 ? 2 : 1;
     const bool two23 = simt_two_tokens(D, false, p.N, p.BH), two1 = simt_two_tokens(D, true, p.N, p.BH);
-    const int route_threads = (int)bp.m_tile;
     const int64_t seed_rows = p.H * p.M;
     const int ways = reduce_ways(lat_rows, D, bp.nchunk);
     const int seed_ways = reduce_ways(seed_rows, D, p.B * bp.nchunk);
     const unsigned red_blocks = reduce_blocks<D>(lat_rows, ways);
 
     launch_delta_tokens<D, float>(dY, Y, tok_rows, c3, st);
-    const auto route = [&](auto kernel, const float* a, int per_head, const float* k,
+    const auto route = [&](auto kernel, int per_route, const float* a, int per_head, const float* k,
                            const float* w, const float* g, const float* Lr, const float* cr) {
-        return launch_pdl(kernel, dim3(route_blocks), dim3((unsigned)route_threads), 0, st, a,
+        return launch_pdl(kernel, dim3(route_blocks), dim3((unsigned)(bp.m_tile * per_route)), 0, st, a,
                           per_head, k, w, g, Lr, cr, (const float*)L3, (const float*)c3, p.H, p.N,
                           p.M, bp.chunk_len, bp.nchunk, bp.n_mtiles, sl2, pa, pb);
     };
@@ -457,7 +487,8 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, co
     const float* none = nullptr;
     cudaError_t e;
     // call 3: dZ and the decoder's dQ
-    if ((e = route(route_pass_kernel<D, 3>, Q32, 0, K, dY, Z32, none, none)) != cudaSuccess)
+    if ((e = route(route_pass_kernel<D, 3>, route_threads(D, 3), Q32, 0, K, dY, Z32, none, none)) !=
+        cudaSuccess)
         return e;
     bwd_reduce_kernel<D, float, 3><<<red_blocks, kRedThreads, 0, st>>>(
         pa, pb, lat_rows, p.B, p.H, p.M, bp.nchunk, ways, scale, Z32, dz, dq, c2, nullptr, nullptr);
@@ -466,7 +497,9 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, co
                    dY, Q32, 0, dz, Z32, L2, c2, dK, dV)) != cudaSuccess)
         return e;
     // call 2: the encoder's dQ, added to the decoder's
-    if ((e = route(route_pass_kernel<D, 2>, Q32, 0, K, V, dz, L2, c2)) != cudaSuccess) return e;
+    if ((e = route(route_pass_kernel<D, 2>, route_threads(D, 2), Q32, 0, K, V, dz, L2, c2)) !=
+        cudaSuccess)
+        return e;
     bwd_reduce_kernel<D, float, 2><<<red_blocks, kRedThreads, 0, st>>>(
         nullptr, pb, lat_rows, p.B, p.H, p.M, bp.nchunk, ways, scale, Q32, nullptr, dq, c1, nullptr,
         nullptr);
@@ -474,7 +507,9 @@ cudaError_t route_bwd_d(const Plan& p, const BwdPlan& bp, const float* seeds, co
     if ((e = token(two1 ? token_pass_kernel<D, 1, kTwo> : token_pass_kernel<D, 1, 1>, two1, Kt, Vt,
                    none, seeds, 1, dq, none, L1, c1, dKt, dVt)) != cudaSuccess)
         return e;
-    if ((e = route(route_pass_kernel<D, 1>, seeds, 1, Kt, Vt, dq, L1, c1)) != cudaSuccess) return e;
+    if ((e = route(route_pass_kernel<D, 1>, route_threads(D, 1), seeds, 1, Kt, Vt, dq, L1, c1)) !=
+        cudaSuccess)
+        return e;
     bwd_reduce_kernel<D, float, 1>
         <<<reduce_blocks<D>(seed_rows, seed_ways), kRedThreads, 0, st>>>(
             nullptr, pb, seed_rows, p.B, p.H, p.M, bp.nchunk, seed_ways, scale, nullptr, nullptr,

@@ -122,10 +122,11 @@ constexpr int simt_token_places(int64_t D, int rows, bool call1) {
 }
 // Two tokens read the staged rows half as often but leave fewer, longer blocks, so a last wave with few
 // of them costs more. A wave's time with two tokens over that with one, measured: D = 16 1.3 (calls 3
-// and 2) and 1.08 (call 1), D = 32 1.0 and 1.19; a last wave takes half that time and the rest by how full
-// it is; and where one token a pair takes one wave, two only make it longer. 8 x 16,384 tokens, M = 128, D = 32: 153 and 119 us with two, 199 and 128 with one (one token per
-// thread 210 and 130); D = 16 89 and 71 against 96 and 73. 60,000 tokens, M = 256, D = 16, 13 blocks beyond
-// a full wave of two: 104 and 84 against 97 and 74. At D = 64 two would spill.
+// and 2) and 1.08 (call 1), D = 32 1.0 and 1.19; a last wave takes half that time and the rest by how
+// full it is; and where one token a pair takes one wave, two only make it longer. 8 x 16,384 tokens,
+// M = 128, D = 32: 153 and 119 us with two, 199 and 128 with one (one token per thread 210 and 130);
+// D = 16 89 and 71 against 96 and 73. 60,000 tokens, M = 256, D = 16, 13 blocks beyond a full wave of
+// two: 104 and 84 against 97 and 74. At D = 64 two would spill.
 inline bool simt_two_tokens(int64_t D, bool call1, int64_t N, int64_t BH) {
     if (D == 64 || cdiv(N, 64) * BH <= simt_token_places(D, 1, call1) * kNumSMs) return false;
     const auto waves = [&](int64_t tokens, int rows) {

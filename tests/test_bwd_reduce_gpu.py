@@ -19,6 +19,7 @@ SHAPES = [  # B, H, N, M, D, dtype
     (33, 1, 150, 9, 32, "bf16"),    # the seeds' sum over the batch
     (1, 1, 30000, 7, 16, "f32"),
     (17, 1, 200, 4, 64, "f32"),
+    (2, 1, 500, 150, 64, "f32"),    # two threads per route in call 3, a ragged route tile
 ]
 
 
