@@ -20,6 +20,8 @@ SHAPES = [  # B, H, N, M, D, dtype
     (1, 1, 30000, 7, 16, "f32"),
     (17, 1, 200, 4, 64, "f32"),
     (2, 1, 500, 150, 64, "f32"),    # two threads per route in call 3, a ragged route tile
+    (38, 8, 249, 9, 32, "f32"),     # two tokens per pair of threads, 608 blocks of them
+    (57, 8, 113, 7, 16, "f32"),     # and 456
 ]
 
 

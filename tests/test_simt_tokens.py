@@ -14,6 +14,7 @@ CSRC = os.path.join(ROOT, "paper_2608_11519_gb300", "csrc")
 CASES = [
     (32, 0, 16384, 8, 1), (32, 1, 16384, 8, 1), (16, 0, 16384, 8, 1), (16, 1, 16384, 8, 1),
     (16, 1, 60000, 8, 1),
+    (32, 0, 249, 304, 1), (32, 1, 249, 304, 1), (16, 0, 113, 456, 1), (16, 1, 113, 456, 1),
     (16, 0, 60000, 1, 0), (16, 1, 60000, 1, 0),  # 469 blocks of 128 tokens, 456 places
     (16, 1, 781, 160, 0),
     (32, 0, 1024, 4, 0), (32, 1, 1024, 4, 0), (16, 0, 500, 1, 0),
