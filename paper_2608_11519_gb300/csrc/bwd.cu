@@ -1,6 +1,8 @@
-// Backward of the routing chain (App. A.5): the CUDA-core passes (float32 inputs), the
-// kernels both paths share (c of call 3, the reduces of the route passes' partials) and
-// the launch sequence of both paths; the tensor-core passes are in tc_bwd.cu.
+// Backward of the routing chain (App. A.5): the CUDA-core passes (float32 inputs), the small
+// kernels of both paths (c of call 3, the tensor-core path's prologue, the reduces of partial
+// sums) and the launch sequence of both paths. The tensor-core passes are in tc_tok.cu (the token
+// passes that also form dQ and dseeds), tc_kernels.cu (dZ, an encode with column statistics) and
+// tc_bwd.cu (the separate passes).
 //
 // Every SDPA of the chain is differentiated from its saved output O and log-normaliser L:
 //   P = 2^(x - L) with x = scale * log2(e) <a, b> (L kept in base 2 by the forward),
@@ -16,8 +18,10 @@
 // streams a chunk of tokens, accumulating the latent-side sums (dZ, dQ, dQs) into per-chunk
 // partials that a reduce kernel adds in chunk order. A token pass gives two threads to one or two
 // tokens and streams every route, producing that token's dK, dV (calls 2 and 3 together) or
-// dKt, dVt (call 1). The tensor-core path has the same structure (passes R3, T23, R2, T1,
-// R1) with bf16 copies of Q, Z, dZ and dQ as MMA operands.
+// dKt, dVt (call 1). The tensor-core path works with bf16 copies of Q, Z, dZ and dQ as MMA operands:
+// up to tok_max_routes(D) routes as dZ, the token pass of calls 3 and 2 with dQ, and the token pass of
+// call 1 with dseeds; otherwise (D = 64, more routes, and heads whose log-normalisers spread too far)
+// in the structure above, passes R3, T23, R2, T1, R1.
 #include <cuda_bf16.h>
 #include <math.h>
 

@@ -14,9 +14,9 @@
 //
 // Work is cut into four TMEM "streams". Stream s owns one score buffer of 128 x kItem fp32
 // (S is rewritten in place as bf16 P, the A operand of the PV product) and a 128 x D fp32
-// accumulator O (two in the decode at D <= 32, one per unit parity), and reads one resident A
-// tile in shared memory, so that S = A * B^T is a SMEM x SMEM product and all TMEM columns go
-// to S and O. The decode double-buffers its A tiles, so the next unit's tiles land while the
+// accumulator O (two in the decode's narrow form at D <= 32, one per unit parity), and reads one
+// resident A tile in shared memory, so that S = A * B^T is a SMEM x SMEM product and all TMEM
+// columns go to S and O. The decode double-buffers its A tiles, so the next unit's tiles land while the
 // current unit runs. Roles (24 warps, a register split gives warpgroups 0 and 1 40 registers
 // per thread and the four softmax warpgroups 96):
 //   warps 0..3    one MMA warp per stream: for item j, the PV of item j-1 and the S of
@@ -150,7 +150,7 @@ struct Cfg {
     static constexpr uint32_t kColO = NS * B * kItem;  // kOBuf x NS x D
     static_assert(kColO + kOBuf * NS * D <= kTmemCols, "TMEM budget");
     static_assert(kSmem <= 232448, "shared memory budget");
-    static_assert(kStages >= (DEC ? 4 : 2 * B * NS), "ring depth: the full wait precedes the PV");
+    static_assert(kStages >= (DEC ? 2 : 2 * NS), "ring depth: no release may wait for the full wait");
     static_assert(B == 1, "the s_ready / o_done protocol has one score buffer per stream");
 };
 
@@ -351,7 +351,7 @@ __device__ __forceinline__ float exp_chunk(const uint32_t* sr, uint32_t* pr, int
 // nc2: (-c, -c). No sum is kept.
 template <int W>
 __device__ __forceinline__ void exp_chunk_col(const uint32_t* sr, uint32_t* pr, int base, int nv,
-                                              float c, uint64_t nc2, const float* L) {
+                                              uint64_t nc2, const float* L) {
     const bool full = base + W <= nv;
 #pragma unroll
     for (int k = 0; k < W / 2; k += 2) {
@@ -486,7 +486,7 @@ __device__ __forceinline__ bool softmax_step(SoftmaxStream& S, const Unit& U, ui
             uint32_t sr[32];
             tmem_ld32(scol + 32 * h, sr);
             tmem_wait_ld32(sr);
-            exp_chunk_col<32>(sr, pr + 16 * h, 32 * h, nv, c, nc2, L + 32 * h);
+            exp_chunk_col<32>(sr, pr + 16 * h, 32 * h, nv, nc2, L + 32 * h);
             tmem_st16(scol + 16 * h, pr + 16 * h);
         }
         if constexpr (C::kItem % 32 == 16) {
@@ -494,7 +494,7 @@ __device__ __forceinline__ bool softmax_step(SoftmaxStream& S, const Unit& U, ui
             uint32_t sr[16];
             tmem_ld16(scol + base, sr);
             tmem_wait_ld16(sr);
-            exp_chunk_col<16>(sr, pr + base / 2, base, nv, c, nc2, L + base);
+            exp_chunk_col<16>(sr, pr + base / 2, base, nv, nc2, L + base);
             tmem_st8(scol + base / 2, pr + base / 2);
         }
         tmem_wait_st();
@@ -772,8 +772,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const uint32_t st = it % C::kStages;
                 // the item's full barrier first (the softmax is still busy with item j - 1, so
                 // this wait is off the P -> PV -> S round trip), then the P of item j - 1.
-                // Item i lands once item i - kStages is released; with kStages >= 2 NS that
-                // item's PV was issued in an earlier iteration, so this wait closes no cycle.
+                // Item i lands once every stream has released item i - kStages. S of the stream's
+                // item before this one is issued already, and the softmax that sees it releases the
+                // one before that: 2 items back in the decode, whose streams take every item, at most
+                // 2 NS back in the encode, whose streams may take every NS-th. With that many stages
+                // no release waits for this wait, and it closes no cycle.
                 if (!warp_wait(full0 + 8u * st, (it / C::kStages) & 1, abort_flag, prm.status, prm.wait_ns)) {
                     ok = false;
                     break;

@@ -209,8 +209,8 @@ def _on_device(arg):
         default = params[arg].default
 
         # A small call is bound by the host: without binding the whole signature, entering a device
-        # context that is current already and wrapping pointers, route_fwd on 8 x 1,000 tokens takes
-        # 42 us instead of 51 (float32, 4 x 1,024 tokens: 30 instead of 40).
+        # context that is current already and wrapping pointers, route_fwd on 8 x 1,000 bf16 tokens
+        # takes 42 us instead of 51.
         @functools.wraps(fn)
         def call(*a, **kw):
             v = a[at] if len(a) > at else kw.get(arg)
