@@ -3,6 +3,7 @@
 // configuration, so this file and the kernel sources together determine what each kernel
 // reads and writes.
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -17,28 +18,59 @@ constexpr int64_t kMaxTmaCoord = 2147483647 - 4096;  // TMA coordinates are sign
 
 bool mul_ok(int64_t a, int64_t b, int64_t* out) { return !__builtin_mul_overflow(a, b, out); }
 
-// Tokens per chunk of a CUDA-core pass over `tiles` ((b, h), route tile) pairs: the count of least time,
-// in units of a token (about 0.2 us: a CTA's tokens are a chain, as fast alone on an SM as among the
-// `places` CTAs that registers allow there). A wave of CTAs takes its chunk's tokens and about 16 more
-// for rows and partials; the partials' bytes are written and read again (0.56 MB a token); and the
-// merge's chain grows with the chunks. Tried are the largest counts of eight numbers of waves.
-int64_t simt_chunk_len(int64_t N, int64_t tiles, int64_t places, double bytes, double most_bytes,
-                       double per_chunk) {
+// What a CUDA-core pass costs, in us: a token, with one warp on each of an SM's four schedulers, and more
+// for each further one; and what a chunk adds to the merge of the partials. Fitted to the passes at 1 to
+// 16 warps per SM (20,000 to 200,000 tokens of one (b, h), and 8 x 16,384): a warp's tokens are a chain, so
+// up to one warp per scheduler more CTAs are free, and beyond it they cost less than they bring.
+struct SimtCost {
+    double token, more, chunk;
+};
+SimtCost encode_cost(int rows, int64_t D) {
+    if (rows == 2) return D == 16 ? SimtCost{0.09, 0.05, 0.034} : SimtCost{0.21, 0.10, 0.034};
+    if (D == 16) return {0.047, 0.01, 0.034};
+    return D == 32 ? SimtCost{0.085, 0.03, 0.034} : SimtCost{0.16, 0.10, 0.034};
+}
+SimtCost route_cost(int64_t D) {
+    if (D == 16) return {0.085, 0.02, 0.006};
+    return D == 32 ? SimtCost{0.118, 0.06, 0.006} : SimtCost{0.3, 0.2, 0.006};
+}
+
+// Tokens per chunk of a CUDA-core pass over `tiles` ((b, h), route tile) pairs, one CTA of `warps` warps per
+// tile and chunk, up to `places` of them on an SM: the count of least time by the costs above (with 3 us
+// and half a us for every CTA that an SM starts, and the partials' bytes written and read again in L2).
+// Tried are the counts that give every scheduler 1, 2, ... warps, whole numbers of waves, and a smaller
+// one that balances tokens against the merge: few routes of one (b, h) are one chain of loads there
+// (20,000 tokens, M = 16: 1,250 chunks fill the machine and take 55 us more a call than 417).
+int64_t simt_chunk_len(int64_t N, int64_t tiles, int64_t places, int64_t warps, SimtCost c,
+                       double bytes, double most_bytes) {
     const int64_t full = places * kNumSMs, most = cdiv(N, 16);
+    const double chunk = bytes / 5.0e6 + c.chunk;
     double best = 1e300;
-    int64_t best_len = most * 16, n = 0, waves = cdiv(tiles, full) - 1;
-    for (int k = 0; k < 8 && n < most; ++k) {
-        n = ++waves * full / tiles;
+    int64_t best_len = most * 16;
+    auto attempt = [&](int64_t n) {
         if ((double)n * bytes > most_bytes) n = (int64_t)(most_bytes / bytes);
         if (n > most) n = most;
         if (n < 1) n = 1;
-        const int64_t len = cdiv(cdiv(N, n), 16) * 16, chunks = cdiv(N, len);
-        const double cost = (double)cdiv(tiles * chunks, full) * ((double)len + 16.0) +
-                            (double)chunks * (bytes / 0.56e6 + per_chunk);
+        const int64_t len = cdiv(cdiv(N, n), 16) * 16, chunks = cdiv(N, len), ctas = tiles * chunks;
+        const auto wave = [&](int64_t per_sm) {
+            return (double)len * (c.token + c.more * (double)(cdiv(per_sm * warps, 4) - 1));
+        };
+        const int64_t rest = ctas % full;
+        const double cost = 3.0 + 0.5 * (double)ctas / kNumSMs + (double)(ctas / full) * wave(places) +
+                            (rest ? wave(cdiv(rest, kNumSMs)) : 0.0) + (double)chunks * chunk;
         if (cost < best) {
             best = cost;
             best_len = len;
         }
+    };
+    attempt((int64_t)sqrt((double)N * c.token / (chunk + 0.5 * (double)tiles / kNumSMs)));
+    for (int64_t level = 4; level / warps < places; level += 4)
+        if (level >= warps) attempt(level / warps * kNumSMs / tiles);
+    const int64_t waves = cdiv(tiles, full);
+    for (int64_t k = waves; k < waves + 7; ++k) {
+        const int64_t n = k * full / tiles;
+        attempt(n);
+        if (n >= most || (double)n * bytes >= most_bytes) break;
     }
     return best_len;
 }
@@ -82,9 +114,9 @@ flarepp_status make_plan(const flarepp_shape* s, Plan* p) {
         const double scratch = (double)kNoAllocScratchBytes;
         double most = 32.0 * 1048576.0;
         if (rest - 2048.0 + bytes <= scratch && scratch - rest < most) most = scratch - rest;
-        p->chunk_len = simt_chunk_len(s->N, bh * p->n_mtiles,
-                                      simt_encode_warps(rows, s->D) / (p->m_tile / rows / 32), bytes,
-                                      most, 0.1);
+        const int64_t warps = p->m_tile / rows / 32;
+        p->chunk_len = simt_chunk_len(s->N, bh * p->n_mtiles, simt_encode_warps(rows, s->D) / warps,
+                                      warps, encode_cost(rows, s->D), bytes, most);
         p->nchunk = cdiv(s->N, p->chunk_len);
     } else {
         // Tensor-core encode: a work unit is (bh, group of <= 512 routes, chunk of tokens) and
@@ -202,10 +234,10 @@ BwdPlan make_bwd_plan(const Plan& p) {
         b.chunk_len = cdiv(cdiv(p.N, want), item) * item;
     } else {
         // one thread per route, up to 128 routes per CTA
-        b.chunk_len = simt_chunk_len(p.N, p.BH * b.n_mtiles,
-                                     simt_route_warps(p.D) / (b.m_tile / 32),
-                                     (double)p.BH * (double)p.M * (double)p.D * 4.0,
-                                     32.0 * 1048576.0, 0.03);
+        const int64_t warps = b.m_tile / 32;
+        b.chunk_len = simt_chunk_len(p.N, p.BH * b.n_mtiles, simt_route_warps(p.D) / warps, warps,
+                                     route_cost(p.D), (double)p.BH * (double)p.M * (double)p.D * 4.0,
+                                     32.0 * 1048576.0);
     }
     b.nchunk = cdiv(p.N, b.chunk_len);
     const size_t part = (size_t)p.BH * (size_t)b.nchunk * (size_t)p.M * (size_t)p.D * 4;

@@ -1,6 +1,6 @@
 """The float32 passes' chunk plans (make_plan and make_bwd_plan, plan.cu, compiled here as host code): the
 waves of CTAs take little more than an even share of the tokens, whatever the batch and the width of the
-route tiles, and more chunks never take a shape from the call that works in a fixed scratch of 64 MiB
+route tiles, without more chunks than the merge can take, and more chunks never take a shape from the call that works in a fixed scratch of 64 MiB
 (the plan that this is held against cut the tokens for about four waves of CTAs)."""
 import os
 import shutil
@@ -12,6 +12,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_2608_11519_gb300", "csrc")
 
 HARNESS = r"""
+#include <math.h>
 #include <stdio.h>
 #include <random>
 #include "flarepp_internal.h"
@@ -37,16 +38,21 @@ int main() {
         const bool two = M >= 128 && D <= 32;
         const int64_t enc = warps(two ? 168 : (D == 16 ? 168 : 255)) / (two ? 2 : tile / 32);
         const int64_t route = warps(D == 16 ? 128 : 255) / (tile / 32);
-        auto fits = [&](int64_t len, int64_t chunks, int64_t places, double bytes, double cap) {
+        // the waves' tokens and the merge's chunks (in tokens: 0.04 us each in the encode's) beside an
+        // even share and what balancing the two has to leave
+        auto fits = [&](int64_t len, int64_t chunks, int64_t places, double bytes, double cap,
+                        double merge) {
             const double time = (double)cdiv(tiles * chunks, places * kNumSMs) * (double)len;
             const double share = (double)tiles * (double)N / (double)(places * kNumSMs);
+            const double even = sqrt((merge + bytes / 0.56e6) * (double)N);
             return len % 16 == 0 && chunks == cdiv(N, len) &&
-                   (time <= 1.35 * share + 48.0 + 16.0 * (double)cdiv(tiles, places * kNumSMs) ||
+                   (time + merge * (double)chunks <=
+                        1.6 * share + 64.0 + 2.5 * even + 16.0 * (double)cdiv(tiles, places * kNumSMs) ||
                     4.0 * (double)chunks * bytes > cap);  // (or more partials would take too much)
         };
         const double e = (double)bh * M * (D + 2) * 4.0;
-        const bool ok = fits(p.chunk_len, p.nchunk, enc, e, 32e6) &&
-                        fits(b.chunk_len, b.nchunk, route, (double)bh * M * D * 4.0, 32e6) &&
+        const bool ok = fits(p.chunk_len, p.nchunk, enc, e, 32e6, D == 16 ? 1.0 : (D == 32 ? 0.4 : 0.15)) &&
+                        fits(b.chunk_len, b.nchunk, route, (double)bh * M * D * 4.0, 32e6, 0.03) &&
                         (p.nchunk == 1 || (double)p.nchunk * e <= 32.0 * 1048576.0);
         // the workspace with chunks for four waves of 608 CTAs
         int64_t want = cdiv(608, tiles);
@@ -62,7 +68,7 @@ int main() {
     };
     for (int64_t B : {1, 2, 20, 32, 40})
         for (int64_t H : {1, 5, 8})
-            for (int64_t N : {1, 15, 781, 1024, 16384, 60000, 262144})
+            for (int64_t N : {1, 15, 781, 1024, 16384, 20000, 60000, 262144})
                 for (int64_t M : {1, 16, 32, 33, 64, 96, 100, 128, 256, 300, 2048})
                     for (int64_t D : {16, 32, 64}) check(B, H, N, M, D);
     std::mt19937_64 g(9);
