@@ -97,3 +97,27 @@ def test_gradients_of_call_1_with_offset_values(N, M, D, centres, scale, offset,
     for name, bound in BOUND.items():
         err = float((got[name].double() - want[name]).norm() / want[name].norm())
         assert err <= bound, f"{name}: {err} > {bound}"
+
+
+def test_float32_sums_over_many_tokens():
+    """The float32 route passes sum at most 256 tokens in a register before they add to the chunk's partial.
+    With one route P3 = 1, dZ is the sum of dY over the tokens and dV_n = P2_n dZ: the direction of dV_n is
+    that of dZ, whatever the error of P2. 1,216 heads leave one chunk of 1,500 tokens to each. dY = 1 + noise
+    added up in one float32 chain has an error of sqrt(1500 / 3) 2^-24 0.41 = 5.4e-7 rms (every sum so far
+    rounded once), in parts of 256 2.2e-7 and 0.9e-7 for adding the parts; the product with P2 adds 0.2e-7.
+    The bound is the geometric mean of 5.4e-7 and 2.4e-7."""
+    B, H, N, M, D = 152, 8, 1500, 1, 32
+    g = torch.Generator(device="cuda").manual_seed(3)
+
+    def normal(*shape):
+        return torch.randn(*shape, generator=g, device="cuda")
+
+    scale = D ** -0.5
+    args = (normal(H, M, D), normal(B, H, N, D), normal(B, H, N, D), normal(B, H, N, D), normal(B, H, N, D))
+    dY = 1.0 + 0.25 * normal(B, H, N, D)
+    Y, saved = flarepp.route_fwd_train(*args, scale)
+    dV = flarepp.route_bwd(*args, Y, dY, saved, scale)[4].double()
+    want = dY.double().sum(2, keepdim=True)
+    want = want / want.norm(dim=-1, keepdim=True)
+    err = float((dV / dV.norm(dim=-1, keepdim=True) - want).pow(2).sum(-1).mean().sqrt())
+    assert err <= 3.6e-7, err
