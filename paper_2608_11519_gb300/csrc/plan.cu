@@ -46,11 +46,13 @@ int64_t simt_chunk_len(int64_t N, int64_t tiles, int64_t places, int64_t warps, 
     const int64_t full = places * kNumSMs, most = cdiv(N, 16);
     const double chunk = bytes / 5.0e6 + c.chunk;
     double best = 1e300;
-    int64_t best_len = most * 16;
+    int64_t best_len = most * 16, tried = 0;
     auto attempt = [&](int64_t n) {
         if ((double)n * bytes > most_bytes) n = (int64_t)(most_bytes / bytes);
         if (n > most) n = most;
         if (n < 1) n = 1;
+        if (n == tried) return;  // (short sequences come to the same count again and again)
+        tried = n;
         const int64_t len = cdiv(cdiv(N, n), 16) * 16, chunks = cdiv(N, len), ctas = tiles * chunks;
         const auto wave = [&](int64_t per_sm) {
             return (double)len * (c.token + c.more * (double)(cdiv(per_sm * warps, 4) - 1));
