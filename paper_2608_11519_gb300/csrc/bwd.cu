@@ -154,8 +154,8 @@ __global__ void __launch_bounds__(128 * route_threads(D, MODE),
 
     // The sums go to the chunk's partials every kFlush tokens and start afresh: a float32 sum of hundreds
     // of terms after one another loses more than the sum of its parts (dseeds of 25 x 4,000 tokens,
-    // M = 150, D = 64, in chunks of 672: 17 % more error than in chunks of 320, with this 3 % less). It costs 1 % of
-    // a training step (8 x 16,384 tokens, M = 128, D = 32: 785 -> 794 us).
+    // M = 150, D = 64, in chunks of 672: 17 % more error than in chunks of 320, with this 3 % less). It
+    // costs 1 % of a training step (8 x 16,384 tokens, M = 128, D = 32: 785 -> 794 us).
     const int64_t row = (bh * nchunk + c) * M + m;
     auto put = [&](float* part, f2* acc, bool first) {
         float* dst = part + row * D;
