@@ -19,12 +19,13 @@ constexpr int64_t kMaxTmaCoord = 2147483647 - 4096;  // TMA coordinates are sign
 bool mul_ok(int64_t a, int64_t b, int64_t* out) { return !__builtin_mul_overflow(a, b, out); }
 
 // What a CUDA-core pass costs, in us: a token, with one warp on each of an SM's four schedulers, and more
-// for each further one; and what a chunk adds to the merge of the partials. Fitted to the passes at 1 to
+// for each further one; and what a chunk beyond kFreeChunks adds to the merge of the partials. Fitted to the passes at 1 to
 // 16 warps per SM (20,000 to 200,000 tokens of one (b, h), and 8 x 16,384): a warp's tokens are a chain, so
 // up to one warp per scheduler more CTAs are free, and beyond it they cost less than they bring.
 struct SimtCost {
     double token, more, chunk;
 };
+constexpr int64_t kFreeChunks = 64;  // the merge's first loads, which its launch takes anyway
 SimtCost encode_cost(int rows, int64_t D) {
     if (rows == 2) return D == 16 ? SimtCost{0.09, 0.05, 0.034} : SimtCost{0.21, 0.10, 0.034};
     if (D == 16) return {0.047, 0.01, 0.034};
@@ -44,7 +45,7 @@ SimtCost route_cost(int64_t D) {
 int64_t simt_chunk_len(int64_t N, int64_t tiles, int64_t places, int64_t warps, SimtCost c,
                        double bytes, double most_bytes) {
     const int64_t full = places * kNumSMs, most = cdiv(N, 16);
-    const double chunk = bytes / 5.0e6 + c.chunk;
+    const double traffic = bytes / 5.0e6;
     double best = 1e300;
     int64_t best_len = most * 16, tried = 0;
     auto attempt = [&](int64_t n) {
@@ -59,13 +60,15 @@ int64_t simt_chunk_len(int64_t N, int64_t tiles, int64_t places, int64_t warps, 
         };
         const int64_t rest = ctas % full;
         const double cost = 3.0 + 0.5 * (double)ctas / kNumSMs + (double)(ctas / full) * wave(places) +
-                            (rest ? wave(cdiv(rest, kNumSMs)) : 0.0) + (double)chunks * chunk;
+                            (rest ? wave(cdiv(rest, kNumSMs)) : 0.0) + (double)chunks * traffic +
+                            (chunks > kFreeChunks ? (double)(chunks - kFreeChunks) * c.chunk : 0.0);
         if (cost < best) {
             best = cost;
             best_len = len;
         }
     };
-    attempt((int64_t)sqrt((double)N * c.token / (chunk + 0.5 * (double)tiles / kNumSMs)));
+    attempt(kFreeChunks);
+    attempt((int64_t)sqrt((double)N * c.token / (traffic + c.chunk + 0.5 * (double)tiles / kNumSMs)));
     for (int64_t level = 4; level / warps < places; level += 4)
         if (level >= warps) attempt(level / warps * kNumSMs / tiles);
     const int64_t waves = cdiv(tiles, full);
